@@ -149,7 +149,7 @@ def measured_peak_hbm():
         return 6800.0, "fallback"
 
 
-KERNEL_SOURCES = ("hv_render.cu", "hv_device.cuh", "hv_learned.cuh", "hv_internal.h")
+KERNEL_SOURCES = ("hv_render.cu", "hv_sweep.cuh", "hv_device.cuh", "hv_learned.cuh", "hv_internal.h")
 PROFILES = {2: "k_render_points_gmm100M.md", 3: "k_render_lines_walk50M.md", 4: "k_render_polygons_star2M.md"}
 
 

@@ -39,13 +39,6 @@ __host__ __device__ inline int32_t mid32(int32_t a, int32_t b) {
     return (int32_t)(((int64_t)a + (int64_t)b) >> 1);
 }
 
-// |o - s|^2 <= R^2 (Algorithm 1, closed comparison).  |dx|, |dy| < 2^31.
-__device__ __forceinline__ bool point_within(int32_t ox, int32_t oy, int32_t sx, int32_t sy,
-                                             int64_t R2) {
-    int64_t dx = (int64_t)ox - sx, dy = (int64_t)oy - sy;
-    return dx * dx + dy * dy <= R2;
-}
-
 // Unsigned 64 x 64 -> 128-bit product compare: a*a <= b*c.
 __device__ __forceinline__ bool sq_le_prod(uint64_t a, uint64_t b, uint64_t c) {
     uint64_t lo1 = a * a, hi1 = __umul64hi(a, a);

@@ -12,20 +12,20 @@
 // Work decomposition.  One CTA (8 warps) renders a strip of 256 x rows pixels
 // of one tile (rows = 16 for large batches, 8 or 4 for small ones; batches
 // too small to fill the GPU even then split each 4-row strip into 2 or 4
-// column parts, one CTA each).  The CTA
-// first culls the R-tree (or, with the learned index, the subtrees of the
-// key ranges the model finds) against the strip's box expanded by R, breadth
-// first, into a frontier of at most kFCap nodes in shared memory (the deepest
-// level that fits), binned by 8-pixel block column.  Each warp then takes
-// 8 x 4 pixel blocks (one pixel per lane, up to four samples per lane): it
-// tests its column's frontier entries against its still-undecided samples,
-// descends the intersecting subtrees depth first (a ballot over the 32 child
-// boxes decides which children to visit; for points, children that certainly
-// cover samples decide them on the spot), evaluates the exact predicate on
-// the records of each visited leaf, and stops as soon as every sample of the
-// block is decided.  Results go to a per-pixel byte array in shared memory;
-// the epilogue encodes the strip (MASK bits, COVERAGE bytes or RGBA) with
-// coalesced 16-byte stores.
+// column parts, one CTA each).  The CTA first culls the R-tree (or, with the
+// learned index, the subtrees of the key ranges the model finds) against the
+// strip's box expanded by R, breadth first, into a frontier of at most kFCap
+// nodes in shared memory (the deepest level that fits).  Points are then
+// drawn object by object into a bit per sample of the strip (hv_sweep.cuh).
+// For segments and polygons the frontier is binned by 8-pixel block column,
+// and each warp takes 8 x 4 pixel blocks (one pixel per lane, up to four
+// samples per lane): it tests its column's frontier entries against its
+// still-undecided samples, descends the intersecting subtrees depth first (a
+// ballot over the 32 child boxes decides which children to visit), evaluates
+// the exact predicate on the records of each visited leaf, and stops as soon
+// as every sample of the block is decided.  Results go to a per-pixel byte
+// array in shared memory; the epilogue encodes the strip (MASK bits,
+// COVERAGE bytes or RGBA) with coalesced 16-byte stores.
 #include "hv_device.cuh"
 #include "hv_internal.h"
 #include "hv_learned.cuh"
@@ -155,12 +155,18 @@ __device__ __noinline__ void check_failed(const Params& p, uint32_t code, uint64
 // over the blocks reads only the final one (f_buf), and the other serves the
 // warps as scratch for segment leaves (Src::seg_scratch, pair_scratch) until
 // the barrier that ends the pass.
-struct Smem {
-    uint8_t res[kStripRows * kTile];
+struct Front {
     int4 fbox[2][kFCap];
     uint32_t fid[2][kFCap];
     const int32_t* lvl_base[2][kMaxLevels + 1];   // [0]: tree being traversed, [1]: its side tree
     uint32_t lvl_n[2][kMaxLevels + 1];            // nodes per level
+    int f_count, f_level, f_buf, next_count;
+    int lvl_count[kMaxLevels + 1];
+    unsigned long long prof[kPN];   // phase profile of the CTA (kProf only)
+};
+
+struct Smem : Front {
+    uint8_t res[kStripRows * kTile];
     uint32_t stk_node[kWarps][kMaxLevels + 1];
     uint32_t stk_mask[kWarps][kMaxLevels + 1];
     uint32_t lanemask[kWarps][kMaxLevels + 1][32];
@@ -170,20 +176,19 @@ struct Smem {
     int bucket_off[kBlocksX + 1];
     int bucket_cur[kBlocksX];
     int binned;
-    int f_count, f_level, f_buf, next_count, next_block;
-    unsigned long long prof[kPN];   // phase profile of the CTA (kProf only)
+    int next_block;
 };
 
 // Add the cycles since t0 (or a count) to a phase counter of the CTA (one
 // lane per warp).
 template <bool kProf>
-__device__ __forceinline__ void prof_add(Smem& sm, int k, unsigned long long v, int lane) {
+__device__ __forceinline__ void prof_add(Front& sm, int k, unsigned long long v, int lane) {
     if constexpr (kProf) {
         if (lane == 0) atomicAdd(&sm.prof[k], v);
     }
 }
 template <bool kProf>
-__device__ __forceinline__ void prof_since(Smem& sm, int k, long long t0, int lane) {
+__device__ __forceinline__ void prof_since(Front& sm, int k, long long t0, int lane) {
     if constexpr (kProf) prof_add<kProf>(sm, k, (unsigned long long)(clock64() - t0), lane);
 }
 
@@ -213,17 +218,8 @@ struct Lane {
     uint32_t U;            // warp-uniform: lanes with an undecided sample
     int nk;                // samples per lane (1 or 4)
     int32_t bx0, by0;      // warp-uniform: centre of the block's first pixel
-    int32_t q;             // certain-cover half-side floor(R / sqrt 2) (points), else -1
     int L;                 // warp-uniform: log2 of the pixel size
-    bool narrow;           // warp-uniform: R + 2 off <= kNarrow (32-bit distance tests)
 };
-
-// A sample that a box reaches in Chebyshev distance lies within ext + off =
-// R + 2 off of it along each axis; with that at most kNarrow each squared
-// gap is below 2^31 and the sum of two below 2^32, so squared distances of
-// reachable samples are exact in unsigned 32-bit arithmetic.
-constexpr int32_t kNarrow = 46340;   // floor(sqrt(2^31))
-
 
 // Fold per-sample coverage masks (bit l: lane l's sample k was covered) into
 // the warp's undecided state.
@@ -262,7 +258,6 @@ __device__ __forceinline__ uint32_t rect_lanes(const Lane& s, int32_t x0, int32_
 // Does the box [x0, x1] x [y0, y1] come within Euclidean distance R of an
 // undecided sample of one of the lanes in `cand`?  Exact for every sample;
 // stops at the first that qualifies.
-template <bool kNarrowOk>
 __device__ __forceinline__ bool round_reach(const Lane& s, int32_t x0, int32_t y0, int32_t x1,
                                             int32_t y1, uint32_t cand) {
     // box edges relative to the block's first pixel centre, clamped to
@@ -270,27 +265,6 @@ __device__ __forceinline__ bool round_reach(const Lane& s, int32_t x0, int32_t y
     // 2^30 - 2^26 > R from every sample, so it never decides a gap within R
     const int32_t ax = max(min(x0 - s.bx0, kGridHalf), -kGridHalf), bx = max(min(x1 - s.bx0, kGridHalf), -kGridHalf);
     const int32_t ay = max(min(y0 - s.by0, kGridHalf), -kGridHalf), by = max(min(y1 - s.by0, kGridHalf), -kGridHalf);
-    if (kNarrowOk && s.narrow) {
-        // lanes in cand reach the box in Chebyshev distance: every gap below
-        // is at most R + 2 off
-        const uint32_t R2 = (uint32_t)s.R2;
-        while (cand) {
-            int l = __ffs(cand) - 1;
-            cand &= cand - 1;
-            const int32_t sx = (l & 7) << s.L, sy = (l >> 3) << s.L;
-            const uint32_t gxm = (uint32_t)max(max(ax - (sx - s.off), (sx - s.off) - bx), 0);
-            const uint32_t gxp = (uint32_t)max(max(ax - (sx + s.off), (sx + s.off) - bx), 0);
-            const uint32_t gym = (uint32_t)max(max(ay - (sy - s.off), (sy - s.off) - by), 0);
-            const uint32_t gyp = (uint32_t)max(max(ay - (sy + s.off), (sy + s.off) - by), 0);
-            const uint32_t xm = gxm * gxm, xp = gxp * gxp, ym = gym * gym, yp = gyp * gyp;
-            const bool h0 = (s.Uk[0] >> l) & 1u && xm + ym <= R2;
-            const bool h1 = (s.Uk[1] >> l) & 1u && xp + ym <= R2;
-            const bool h2 = (s.Uk[2] >> l) & 1u && xm + yp <= R2;
-            const bool h3 = (s.Uk[3] >> l) & 1u && xp + yp <= R2;
-            if (h0 | h1 | h2 | h3) return true;
-        }
-        return false;
-    }
     while (cand) {
         int l = __ffs(cand) - 1;
         cand &= cand - 1;
@@ -311,58 +285,18 @@ __device__ __forceinline__ bool round_reach(const Lane& s, int32_t x0, int32_t y
     return false;
 }
 
-// Samples that a non-empty box of points certainly covers: a sample within
-// Chebyshev distance q of every point of the box, with 2 q^2 <= R^2, is
-// within Euclidean distance R of each of them, whatever the points are.  Per
-// sample k, the lanes whose sample k lies in [x1 - q, x0 + q] x [y1 - q,
-// y0 + q] (undecided ones only).  Exact: no sample is marked that the
-// predicate would not cover, so no output depends on it.
-__device__ __forceinline__ void certain_lanes(const Lane& s, int32_t x0, int32_t y0, int32_t x1, int32_t y1,
-                                              uint32_t m[4]) {
-    m[0] = m[1] = m[2] = m[3] = 0u;
-    if (x0 > x1 || y0 > y1 || x0 < -kGridHalf || y0 < -kGridHalf) return;
-    // clamping the differences only narrows the interval (conservative)
-    const int32_t lx = max(x1 - s.bx0, -kGridHalf) - s.q, hx = min(x0 - s.bx0, kGridHalf) + s.q;
-    const int32_t ly = max(y1 - s.by0, -kGridHalf) - s.q, hy = min(y0 - s.by0, kGridHalf) + s.q;
-    if (lx > hx || ly > hy) return;   // the box is wider than 2q
-    uint32_t col[2], row[2];
-#pragma unroll
-    for (int k = 0; k < 2; k++) {
-        // sample offset -off (k = 0) or +off (k = 1) from the pixel centre
-        const int32_t o = k ? -s.off : s.off;
-        const int32_t c0 = max(-((-(lx + o)) >> s.L), 0), c1 = min((hx + o) >> s.L, 7);
-        const int32_t r0 = max(-((-(ly + o)) >> s.L), 0), r1 = min((hy + o) >> s.L, 3);
-        col[k] = c0 > c1 ? 0u : (0xFFu << c0) & (0xFFu >> (7 - c1));
-        row[k] = r0 > r1 ? 0u : (0x01010101u << (8 * r0)) & (0x01010101u >> (8 * (3 - r1)));
-    }
-#pragma unroll
-    for (int k = 0; k < 4; k++) m[k] = (col[k & 1] * row[k >> 1]) & s.Uk[k];
-}
-
-// Each lane offers one box (a child of the node being visited); the samples
-// any of them certainly covers are decided for the whole warp.
-__device__ __forceinline__ void certain_cover(Lane& s, int32_t x0, int32_t y0, int32_t x1, int32_t y1, int lane) {
-    if (s.q < 0) return;
-    uint32_t m[4];
-    certain_lanes(s, x0, y0, x1, y1, m);
-    if (!__any_sync(kFull, (m[0] | m[1] | m[2] | m[3]) != 0u)) return;
-    apply_cover(s, __reduce_or_sync(kFull, m[0]), __reduce_or_sync(kFull, m[1]), __reduce_or_sync(kFull, m[2]),
-                __reduce_or_sync(kFull, m[3]), lane);
-}
-
 // Lanes `cm` can reach and one of their undecided samples really is within
 // reach.  For the fill (R = 0, centres) the Chebyshev test is already exact.
 template <class V>
 __device__ __forceinline__ bool reaches(const Lane& s, uint32_t cm, int32_t x0, int32_t y0, int32_t x1, int32_t y1) {
     uint32_t cand = cm & s.U;
     if (!cand) return false;
-    return V::kFill || round_reach<V::kNarrowReach>(s, x0, y0, x1, y1, cand);
+    return V::kFill || round_reach(s, x0, y0, x1, y1, cand);
 }
 
 // One box against the lanes' own undecided samples (lanes in `lanes` only,
 // each lane its four samples, no loop): whether the box comes within R of
 // any of them.  The same exact test as round_reach, transposed.
-template <bool kNarrowOk>
 __device__ __forceinline__ bool box_reach_lanes(const Lane& s, int32_t x0, int32_t y0, int32_t x1, int32_t y1,
                                                 uint32_t lanes, int lane) {
     bool hit = false;
@@ -374,19 +308,11 @@ __device__ __forceinline__ bool box_reach_lanes(const Lane& s, int32_t x0, int32
         const uint32_t gxp = (uint32_t)max(max(ax - (sx + s.off), (sx + s.off) - bx), 0);
         const uint32_t gym = (uint32_t)max(max(ay - (sy - s.off), (sy - s.off) - by), 0);
         const uint32_t gyp = (uint32_t)max(max(ay - (sy + s.off), (sy + s.off) - by), 0);
-        if (kNarrowOk && s.narrow) {
-            // the lane is in the box's Chebyshev reach: gaps at most R + 2 off
-            const uint32_t R2 = (uint32_t)s.R2;
-            const uint32_t xm = gxm * gxm, xp = gxp * gxp, ym = gym * gym, yp = gyp * gyp;
-            hit = ((s.und & 1u) && xm + ym <= R2) || ((s.und & 2u) && xp + ym <= R2) ||
-                  ((s.und & 4u) && xm + yp <= R2) || ((s.und & 8u) && xp + yp <= R2);
-        } else {
-            const uint64_t R2 = (uint64_t)s.R2;
-            const uint64_t xm = (uint64_t)gxm * gxm, xp = (uint64_t)gxp * gxp;
-            const uint64_t ym = (uint64_t)gym * gym, yp = (uint64_t)gyp * gyp;
-            hit = ((s.und & 1u) && xm + ym <= R2) || ((s.und & 2u) && xp + ym <= R2) ||
-                  ((s.und & 4u) && xm + yp <= R2) || ((s.und & 8u) && xp + yp <= R2);
-        }
+        const uint64_t R2 = (uint64_t)s.R2;
+        const uint64_t xm = (uint64_t)gxm * gxm, xp = (uint64_t)gxp * gxp;
+        const uint64_t ym = (uint64_t)gym * gym, yp = (uint64_t)gyp * gyp;
+        hit = ((s.und & 1u) && xm + ym <= R2) || ((s.und & 2u) && xp + ym <= R2) ||
+              ((s.und & 4u) && xm + yp <= R2) || ((s.und & 8u) && xp + yp <= R2);
     }
     return __any_sync(kFull, hit);
 }
@@ -470,93 +396,6 @@ __device__ __forceinline__ uint32_t crossing_columns(int4 e, const Lane& s, int3
 // the exact predicate on the undecided samples within its reach; the
 // per-sample hits are OR-reduced over the warp.
 
-struct PointLeaf {
-    static constexpr bool kFill = false;
-    static constexpr bool kCertain = true;   // boxes of points certainly cover nearby samples
-    static constexpr bool kOutline = false;
-    static constexpr bool kNarrowReach = true;   // 32-bit node tests when R + 2 off is small
-    // frontier entries and children filtered exactly when listed, by their
-    // Chebyshev reach when taken (see blocks_pass)
-    static constexpr bool kExactWhenTaken = false, kScanChebyshev = false, kChildChebyshev = false;
-    static constexpr bool kOneVisitSite = false;
-    __device__ static uint32_t visit(const Params& p, const Src& src, uint32_t leaf, Lane& s, int lane) {
-        if ((uint64_t)leaf * 32 >= src.n) {
-            if (lane == 0) check_failed(p, 4, leaf);
-            return kVisitEmpty;
-        }
-        uint64_t i = (uint64_t)leaf * 32 + lane;
-        log_read(p, kLogLeaf, leaf, lane);
-        int2 o = make_int2(kEmptyHi, kEmptyHi);
-        if (i < src.n) o = __ldg((const int2*)src.obj + i);
-        // the exact test on the undecided samples in each point's reach
-        uint32_t pm = rect_lanes(s, o.x, o.y, o.x, o.y) & s.U;
-        if (!__any_sync(kFull, pm != 0)) return kVisitEmpty;
-        const uint32_t U_before = s.U;
-        // the point relative to the block's first pixel centre; lanes in pm
-        // are within reach, so the 32-bit differences below are exact
-        const int32_t dxo = max(min(o.x - s.bx0, kGridHalf), -kGridHalf);
-        const int32_t dyo = max(min(o.y - s.by0, kGridHalf), -kGridHalf);
-        const uint64_t R2 = (uint64_t)s.R2;
-        uint32_t c[4] = {0u, 0u, 0u, 0u};
-        if (s.narrow) {
-            // lanes in pm lie within ext of the point along each axis, so
-            // |dx -+ off|, |dy -+ off| <= R + 2 off <= kNarrow
-            const uint32_t R2n = (uint32_t)R2;
-            if (s.nk == 1) {
-                while (pm) {
-                    int l = __ffs(pm) - 1;
-                    pm &= pm - 1;
-                    const int32_t dx = dxo - ((l & 7) << s.L), dy = dyo - ((l >> 3) << s.L);
-                    if ((uint32_t)(dx * dx) + (uint32_t)(dy * dy) <= R2n) c[0] |= 1u << l;
-                }
-            } else {
-                while (pm) {
-                    int l = __ffs(pm) - 1;
-                    pm &= pm - 1;
-                    const int32_t dx = dxo - ((l & 7) << s.L), dy = dyo - ((l >> 3) << s.L);
-                    const uint32_t xm = (uint32_t)((dx + s.off) * (dx + s.off));
-                    const uint32_t xp = (uint32_t)((dx - s.off) * (dx - s.off));
-                    const uint32_t ym = (uint32_t)((dy + s.off) * (dy + s.off));
-                    const uint32_t yp = (uint32_t)((dy - s.off) * (dy - s.off));
-                    const uint32_t bit = 1u << l;
-                    if (xm + ym <= R2n) c[0] |= bit;
-                    if (xp + ym <= R2n) c[1] |= bit;
-                    if (xm + yp <= R2n) c[2] |= bit;
-                    if (xp + yp <= R2n) c[3] |= bit;
-                }
-            }
-        } else if (s.nk == 1) {
-            while (pm) {
-                int l = __ffs(pm) - 1;
-                pm &= pm - 1;
-                const int32_t dx = dxo - ((l & 7) << s.L), dy = dyo - ((l >> 3) << s.L);
-                if ((uint64_t)((int64_t)dx * dx) + (uint64_t)((int64_t)dy * dy) <= R2) c[0] |= 1u << l;
-            }
-        } else {
-            while (pm) {
-                int l = __ffs(pm) - 1;
-                pm &= pm - 1;
-                // point minus sample: sample k sits at -+off in x (bit 0) and y (bit 1)
-                const int32_t dx = dxo - ((l & 7) << s.L), dy = dyo - ((l >> 3) << s.L);
-                const uint64_t xm = (uint64_t)((int64_t)(dx + s.off) * (dx + s.off));
-                const uint64_t xp = (uint64_t)((int64_t)(dx - s.off) * (dx - s.off));
-                const uint64_t ym = (uint64_t)((int64_t)(dy + s.off) * (dy + s.off));
-                const uint64_t yp = (uint64_t)((int64_t)(dy - s.off) * (dy - s.off));
-                const uint32_t bit = 1u << l;
-                if (xm + ym <= R2) c[0] |= bit;
-                if (xp + ym <= R2) c[1] |= bit;
-                if (xm + yp <= R2) c[2] |= bit;
-                if (xp + yp <= R2) c[3] |= bit;
-            }
-        }
-        // decided samples may be hit again: apply_cover only clears bits
-        const uint32_t c0 = __reduce_or_sync(kFull, c[0]), c1 = __reduce_or_sync(kFull, c[1]);
-        const uint32_t c2 = __reduce_or_sync(kFull, c[2]), c3 = __reduce_or_sync(kFull, c[3]);
-        apply_cover(s, c0, c1, c2, c3, lane);
-        return (c0 | c1 | c2 | c3) & U_before ? kVisitDecided : kVisitTested;
-    }
-};
-
 // Per warp, a segment leaf's pieces (their screen parameters, below) and its
 // (piece, pixel) pairs in reach are staged
 // in shared memory, and the warp's lanes take the pairs in turn: a leaf whose
@@ -570,9 +409,7 @@ static_assert(kPairCap * kWarps * 2 <= kFCap * 4, "pair scratch exceeds a fronti
 template <bool kLineLayer>
 struct SegLeaf {
     static constexpr bool kFill = false;
-    static constexpr bool kCertain = false;
     static constexpr bool kOutline = !kLineLayer;   // the outline of a polygon layer
-    static constexpr bool kNarrowReach = false;
     // frontier entries listed by their Chebyshev reach, tested exactly when
     // taken (measured faster for segments, slower for points)
     static constexpr bool kExactWhenTaken = true, kScanChebyshev = true, kChildChebyshev = false;
@@ -730,9 +567,7 @@ struct SegLeaf {
 // unfilled pixel centre, count that polygon's own edges crossing the ray.
 struct FillLeaf {
     static constexpr bool kFill = true;
-    static constexpr bool kCertain = false;
     static constexpr bool kOutline = false;
-    static constexpr bool kNarrowReach = false;
     // R = 0 at the centres: the Chebyshev test is already exact
     static constexpr bool kExactWhenTaken = false, kScanChebyshev = false, kChildChebyshev = false;
     static constexpr bool kOneVisitSite = true;
@@ -813,7 +648,6 @@ struct FillLeaf {
 
 // Child boxes of one inner node: lane c computes the lanes child c can
 // reach, keeps it in `lm`, and the ballot selects the children to visit.
-// Point trees first decide the samples the children certainly cover.
 template <class V>
 __device__ __forceinline__ uint32_t child_hits(const Params& p, const Src& src,
                                                const int32_t* base, Lane& s, int lane, uint32_t* lm) {
@@ -821,7 +655,6 @@ __device__ __forceinline__ uint32_t child_hits(const Params& p, const Src& src,
         log_read(p, V::kFill ? kLogPolyNode : kLogNode, (uint64_t)(base - src.nodes) >> 7, lane);
     int32_t x0 = __ldg(base + lane), y0 = __ldg(base + 32 + lane);
     int32_t x1 = __ldg(base + 64 + lane), y1 = __ldg(base + 96 + lane);
-    certain_cover(s, x0, y0, x1, y1, lane);
     uint32_t cm = rect_lanes(s, x0, y0, x1, y1);
     lm[lane] = cm;
     if constexpr (V::kChildChebyshev)
@@ -867,7 +700,7 @@ __device__ void descend(const Params& p, Smem& sm, const Src& src, int level, ui
         if constexpr (V::kChildChebyshev) {
             // listed by its Chebyshev reach only: the exact test now
             const int32_t* nb = src.lvl[lvl] + (uint64_t)stk_node[lvl] * 128;
-            if (!box_reach_lanes<V::kNarrowReach>(s, __ldg(nb + c), __ldg(nb + 32 + c), __ldg(nb + 64 + c),
+            if (!box_reach_lanes(s, __ldg(nb + c), __ldg(nb + 32 + c), __ldg(nb + 64 + c),
                                                   __ldg(nb + 96 + c), sm.lanemask[warp][lvl][c] & s.U, lane))
                 continue;
         }
@@ -937,7 +770,7 @@ __device__ void descend_one_site(const Params& p, Smem& sm, const Src& src, int 
             if constexpr (V::kChildChebyshev) {
                 // listed by its Chebyshev reach only: the exact test now
                 const int32_t* nb = src.lvl[lvl] + (uint64_t)stk_node[lvl] * 128;
-                if (!box_reach_lanes<V::kNarrowReach>(s, __ldg(nb + c), __ldg(nb + 32 + c), __ldg(nb + 64 + c),
+                if (!box_reach_lanes(s, __ldg(nb + c), __ldg(nb + 32 + c), __ldg(nb + 64 + c),
                                                       __ldg(nb + 96 + c), sm.lanemask[warp][lvl][c] & s.U, lane))
                     continue;
             }
@@ -969,7 +802,7 @@ __device__ void descend_one_site(const Params& p, Smem& sm, const Src& src, int 
 
 // Level bases of a tree into shared memory slot `slot` (0: the tree being
 // traversed, 1: its side tree).
-__device__ __forceinline__ void set_levels(Smem& sm, int slot, const TreeArg& t, int tid) {
+__device__ __forceinline__ void set_levels(Front& sm, int slot, const TreeArg& t, int tid) {
 #pragma unroll
     for (int l = 0; l <= kMaxLevels; l++)
         if (tid == l) {
@@ -981,67 +814,90 @@ __device__ __forceinline__ void set_levels(Smem& sm, int slot, const TreeArg& t,
 
 // Refine the shared frontier breadth first: replace every entry by its
 // children that meet the box, one level at a time, while the next level fits
-// (the deepest level that fits is kept).
-__device__ void refine(const Params& p, const TreeArg& t, bool fill, Smem& sm, int32_t x0, int32_t y0,
+// (the deepest level that fits is kept).  One barrier per level: every level
+// counts its entries in a counter of its own, and the loop's state is kept
+// by every thread alike.
+__device__ void refine(const Params& p, const TreeArg& t, bool fill, Front& sm, int32_t x0, int32_t y0,
                        int32_t x1, int32_t y1, int tid) {
-    int lane = tid & 31, warp = tid >> 5;
-    while (sm.f_level >= 1 && sm.f_count > 0) {
-        int cur = sm.f_buf, lvl = sm.f_level, cnt = sm.f_count;
-        __syncthreads();
-        if (tid == 0) sm.next_count = 0;
-        __syncthreads();
+    const int lane = tid & 31, warp = tid >> 5;
+    int cur = sm.f_buf, lvl = sm.f_level, cnt = sm.f_count;
+    if (tid <= kMaxLevels) sm.lvl_count[tid] = 0;
+    __syncthreads();
+    while (lvl >= 1 && cnt > 0) {
         const int32_t* base = sm.lvl_base[0][lvl];
-        for (int e = warp; e < cnt; e += kWarps) {
-            uint32_t node = sm.fid[cur][e];
-            if (node >= sm.lvl_n[0][lvl]) {
-                if (lane == 0) check_failed(p, 8, ((uint64_t)lvl << 40) | node);
-                continue;
+        // two entries per step: their boxes are loaded together
+        for (int e = warp; e < cnt; e += 2 * kWarps) {
+            const int32_t* nd[2];
+            uint32_t node[2];
+            int4 b[2];
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                const int ek = e + k * kWarps;
+                nd[k] = nullptr;
+                node[k] = 0;
+                if (ek < cnt) {
+                    node[k] = sm.fid[cur][ek];
+                    if (node[k] < sm.lvl_n[0][lvl])
+                        nd[k] = base + (uint64_t)node[k] * 128;
+                    else if (lane == 0)
+                        check_failed(p, 8, ((uint64_t)lvl << 40) | node[k]);
+                }
+                b[k] = make_int4(kEmptyLo, kEmptyLo, kEmptyHi, kEmptyHi);
+                if (nd[k])
+                    b[k] = make_int4(__ldg(nd[k] + lane), __ldg(nd[k] + 32 + lane), __ldg(nd[k] + 64 + lane),
+                                     __ldg(nd[k] + 96 + lane));
             }
-            const int32_t* nd = base + (uint64_t)node * 128;
-            if (p.log != nullptr)
-                log_read(p, fill ? kLogPolyNode : kLogNode, (uint64_t)(nd - t.nodes) >> 7, lane);
-            int4 b = make_int4(__ldg(nd + lane), __ldg(nd + 32 + lane), __ldg(nd + 64 + lane),
-                               __ldg(nd + 96 + lane));
-            bool hit = box_hit(b, x0, y0, x1, y1);
-            uint32_t m = __ballot_sync(kFull, hit);
-            int pos = 0;
-            if (lane == 0 && m) pos = atomicAdd(&sm.next_count, __popc(m));
-            pos = __shfl_sync(kFull, pos, 0);
-            if (hit) {
-                int slot = pos + __popc(m & ((1u << lane) - 1u));
-                if (slot < kFCap) {
-                    sm.fid[cur ^ 1][slot] = node * 32u + (uint32_t)lane;
-                    sm.fbox[cur ^ 1][slot] = b;
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                if (p.log != nullptr && nd[k])
+                    log_read(p, fill ? kLogPolyNode : kLogNode, (uint64_t)(nd[k] - t.nodes) >> 7, lane);
+                const bool hit = box_hit(b[k], x0, y0, x1, y1);
+                const uint32_t m = __ballot_sync(kFull, hit);
+                if (m == 0) continue;
+                int pos = 0;
+                if (lane == 0) pos = atomicAdd(&sm.lvl_count[lvl], __popc(m));
+                pos = __shfl_sync(kFull, pos, 0);
+                if (hit) {
+                    const int slot = pos + __popc(m & ((1u << lane) - 1u));
+                    if (slot < kFCap) {
+                        sm.fid[cur ^ 1][slot] = node[k] * 32u + (uint32_t)lane;
+                        sm.fbox[cur ^ 1][slot] = b[k];
+                    }
                 }
             }
         }
         __syncthreads();
-        int nc = sm.next_count;
-        __syncthreads();
+        const int nc = sm.lvl_count[lvl];
         if (nc > kFCap) break;  // keep the current (coarser) frontier
-        if (tid == 0) {
-            sm.f_buf = cur ^ 1;
-            sm.f_count = nc;
-            sm.f_level = lvl - 1;
-        }
-        __syncthreads();
+        cur ^= 1;
+        cnt = nc;
+        lvl--;
     }
+    if (tid == 0) {
+        sm.f_buf = cur;
+        sm.f_count = cnt;
+        sm.f_level = lvl;
+    }
+    __syncthreads();
 }
 
-// Breadth-first cull of a tree against a box into the shared frontier,
-// starting from the root.
-__device__ void cull(const Params& p, const TreeArg& t, bool fill, Smem& sm, int32_t x0, int32_t y0,
+// Breadth-first cull of a tree against a box into the shared frontier.  It
+// starts at the lowest level with at most kFCap / 32 nodes, all of them: their
+// children fit the frontier whatever the box, so the boxes of these nodes
+// themselves are never needed, and the levels above cost no round.
+__device__ void cull(const Params& p, const TreeArg& t, bool fill, Front& sm, int32_t x0, int32_t y0,
                      int32_t x1, int32_t y1, int tid) {
+    constexpr uint32_t kSeeds = kFCap / 32;
+    static_assert(kSeeds <= kThreads, "one thread per seed");
+    int l0 = t.top;
+    while (l0 > 1 && t.level_n[l0 - 1] <= kSeeds) l0--;
+    const bool meets = t.top > 0 && t.root_box.x <= x1 && t.root_box.z >= x0 && t.root_box.y <= y1 && t.root_box.w >= y0;
+    const int seeds = meets ? (int)t.level_n[l0] : 0;
+    if (tid < seeds) sm.fid[0][tid] = (uint32_t)tid;
     if (tid == 0) {
         sm.f_buf = 0;
-        sm.f_level = t.top;
-        sm.f_count = 0;
-        if (t.top > 0 && t.root_box.x <= x1 && t.root_box.z >= x0 && t.root_box.y <= y1 &&
-            t.root_box.w >= y0) {
-            sm.fid[0][0] = 0;
-            sm.fbox[0][0] = t.root_box;
-            sm.f_count = 1;
-        }
+        sm.f_level = l0;
+        sm.f_count = seeds;
     }
     __syncthreads();
     refine(p, t, fill, sm, x0, y0, x1, y1, tid);
@@ -1054,7 +910,7 @@ __device__ void cull(const Params& p, const TreeArg& t, bool fill, Smem& sm, int
 // and turn the ranges into R-tree subtrees at the finest level whose entries
 // fit the frontier.  Every object whose centre lies in the box is under one of
 // the entries; the blocks then proceed exactly as after the R-tree cull.
-__device__ void learned_cull(const Params& p, const TreeArg& t, const LModel& m, int32_t halo, Smem& sm,
+__device__ void learned_cull(const Params& p, const TreeArg& t, const LModel& m, int32_t halo, Front& sm,
                              int32_t bx0, int32_t by0, int32_t bx1, int32_t by1, int tid) {
     __shared__ unsigned long long cnt[kMaxLevels + 1];
     const int64_t lo_g = -(int64_t)kGridHalf, hi_g = (int64_t)kGridHalf - 1;
@@ -1212,15 +1068,6 @@ __device__ void blocks_pass(const Params& p, Smem& sm, const Src& src, const Src
     const int L = 23 - z;
     const int32_t ps = 1 << L;
     const int f_count = sm.f_count, f_level = sm.f_level, fb = sm.f_buf;
-    // certain-cover half-side: the largest q with 2 q^2 <= R^2
-    int32_t q = -1;
-    if (V::kCertain) {
-        const int64_t R2 = (int64_t)R * R;
-        int64_t t = (int64_t)((double)R * 0.70710678118654752);
-        while (t > 0 && 2 * t * t > R2) t--;
-        while (2 * (t + 1) * (t + 1) <= R2) t++;
-        q = (int32_t)t;
-    }
     while (true) {
         int blk = 0;
         if (lane == 0) blk = atomicAdd(&sm.next_block, 1);
@@ -1251,8 +1098,6 @@ __device__ void blocks_pass(const Params& p, Smem& sm, const Src& src, const Src
             s.nk = 4;
         }
         s.ext = (V::kFill ? 0 : R) + s.off;
-        s.narrow = (int64_t)s.ext + s.off <= kNarrow;
-        s.q = q;
         s.U = kFull;
         for (int k = 0; k < 4; k++) s.Uk[k] = k < s.nk ? kFull : 0u;
         if constexpr (V::kOutline) {
@@ -1301,7 +1146,7 @@ __device__ void blocks_pass(const Params& p, Smem& sm, const Src& src, const Src
                     const int ek = __shfl_sync(kFull, e, k);
                     if constexpr (V::kExactWhenTaken) {
                         const int4 bk = sm.fbox[fb][ek];
-                        if (!box_reach_lanes<V::kNarrowReach>(s, bk.x, bk.y, bk.z, bk.w,
+                        if (!box_reach_lanes(s, bk.x, bk.y, bk.z, bk.w,
                                                               __shfl_sync(kFull, cm, k) & s.U, lane))
                             continue;
                     }
@@ -1590,11 +1435,8 @@ __global__ void __launch_bounds__(kThreads, KindTraits<kKind>::kBlocksPerSM) k_r
         const int32_t sy0 = Y0 + strip * rows * ps + (ps >> 1) - off;
         const int32_t sy1 = Y0 + (strip * rows + rows - 1) * ps + (ps >> 1) + off;
         const bool learned = p.use_learned != 0;
-        // Algorithm 1 over points / segments / polygon edges
-        if constexpr (kKind == HV_LAYER_POINTS)
-            stage<PointLeaf, kProf>(p, sm, p.tree, p.obj, nullptr, p.side, p.side_obj, p.side_ids, learned ? &p.lm : nullptr,
-                             p.halo, X0, Y0, strip, col0, col_shift, z, R, mask_mode, sx0 - R, sy0 - R, sx1 + R, sy1 + R, tid);
-        else if constexpr (kKind != kPolyFill)
+        // Algorithm 1 over segments / polygon edges
+        if constexpr (kKind != kPolyFill)
             stage<SegLeaf<kKind == HV_LAYER_LINES>, kProf>(p, sm, p.tree, p.obj, nullptr, p.side, p.side_obj, p.side_ids, learned ? &p.lm : nullptr,
                            p.halo, X0, Y0, strip, col0, col_shift, z, R, mask_mode, sx0 - R, sy0 - R, sx1 + R, sy1 + R, tid);
         // Algorithm 2 over polygon boxes and edges
@@ -1689,6 +1531,8 @@ __global__ void __launch_bounds__(kThreads, KindTraits<kKind>::kBlocksPerSM) k_r
         if (tid < kPN && sm.prof[tid]) atomicAdd(p.phases + tid, sm.prof[tid]);
     }
 }
+
+#include "hv_sweep.cuh"
 
 TreeArg tree_arg(const TreeView& v) {
     TreeArg a;
@@ -1823,7 +1667,7 @@ int launch_render(Layer* L, const hv_tile_req* d_reqs, uint32_t n, int mode, int
         // polygon layers profile their two launches (fill, outline) into two
         // sets of counters
         if (L->kind == HV_LAYER_POINTS)
-            k_render<HV_LAYER_POINTS, true, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+            k_sweep<HV_LAYER_POINTS, true, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         else if (L->kind == HV_LAYER_LINES)
             k_render<HV_LAYER_LINES, true, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         else {
@@ -1834,7 +1678,7 @@ int launch_render(Layer* L, const hv_tile_req* d_reqs, uint32_t n, int mode, int
         }
     } else if (p.parts > 1) {
         if (L->kind == HV_LAYER_POINTS)
-            k_render<HV_LAYER_POINTS, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+            k_sweep<HV_LAYER_POINTS, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         else if (L->kind == HV_LAYER_LINES)
             k_render<HV_LAYER_LINES, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         else {
@@ -1842,7 +1686,7 @@ int launch_render(Layer* L, const hv_tile_req* d_reqs, uint32_t n, int mode, int
             k_render<HV_LAYER_POLYGONS, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         }
     } else if (L->kind == HV_LAYER_POINTS)
-        k_render<HV_LAYER_POINTS, false, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+        k_sweep<HV_LAYER_POINTS, false, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
     else if (L->kind == HV_LAYER_LINES)
         k_render<HV_LAYER_LINES, false, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
     else {

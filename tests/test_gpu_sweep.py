@@ -1,0 +1,103 @@
+"""Points drawn row by row over a strip's sample lattice: layers and requests
+at the edges of that path, byte-equal to the oracle -- leaves with 1 to 33
+points, points on strip, part and grid borders, samples at exactly R and R +- 1
+units, rows on both sides of the 32-bit radius, reaches wider than the 32-column
+window, crowded and sparse leaves, every zoom class, mode, strip height and
+column part."""
+import numpy as np
+import pytest
+
+import oracle
+import oracle_par
+from geom import centre, ps
+from workloads import gen
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2005_12489_gb300 import hv  # noqa: E402
+
+STYLE_T = (230, 40, 20, 0, 30, 90, 200, 0)
+MODES = [hv.HV_MODE_MASK, hv.HV_MODE_COVERAGE, hv.HV_MODE_RGBA]
+HALF = 1 << 30
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    c = hv.hv_create(0)
+    yield c
+    hv.hv_destroy(c)
+
+
+def _check(ctx, pts, reqs, radius=None, batches=(1, 3, 200)):
+    pts = np.ascontiguousarray(pts, dtype=np.int32)
+    reqs = np.array(reqs, dtype=np.uint32)
+    L = hv.hv_layer_load_points(ctx, pts)
+    hv.hv_layer_build_index(L, hv.HV_INDEX_RTREE | hv.HV_INDEX_LEARNED)
+    s = hv.make_style(STYLE_T[:3], STYLE_T[4:7])
+    try:
+        for mode in MODES:
+            ref = oracle_par.render(lambda r: oracle.render_points(pts, r, mode, STYLE_T, R_units=radius), reqs)
+            for index in (hv.HV_INDEX_RTREE, hv.HV_INDEX_LEARNED):
+                for per in batches:      # column parts, 4-row strips, full strips (requests repeated)
+                    rows = np.resize(np.arange(len(reqs)), max(per, len(reqs))) if per > len(reqs) else np.arange(len(reqs))
+                    for k in range(0, len(rows), per):
+                        part = rows[k:k + per]
+                        d = torch.from_numpy(hv.make_requests(reqs[part]).view(np.uint8).copy()).cuda()
+                        out = torch.full((len(part), hv.hv_tile_bytes(mode)), 0xAB, dtype=torch.uint8, device="cuda")
+                        if radius is None:
+                            hv.hv_render_tiles(L, d, len(part), mode, index, s, out, out.numel(), None)
+                        else:
+                            hv.hv_render_buffer(L, d, len(part), mode, index, radius, s, out, out.numel(), None)
+                        assert np.array_equal(out.cpu().numpy(), ref[part]), (mode, index, per)
+        assert hv.hv_layer_take_status(L) == 0
+    finally:
+        hv.hv_layer_free(L)
+
+
+@pytest.mark.parametrize("z", [0, 1, 8, 9, 13, 19])
+def test_samples_at_exactly_R(ctx, z):
+    """Around samples of a tile's corners and strip borders: points at R and
+    R +- 1 units along an axis and on a 3-4-5 slant."""
+    t = (1 << z) // 2
+    pts, reqs = [], []
+    for r16 in (5, 16, 32, 240):
+        R = r16 << (19 - z)
+        reqs.append([z, t, t, r16])
+        for i, j in ((0, 0), (255, 255), (63, 15), (64, 16), (130, 131)):
+            cx, cy = centre(z, t, t, i, j)
+            for o in (0, ps(z) // 4):
+                for d in (-1, 0, 1):
+                    pts += [(cx + o + R + d, cy + o), (cx + o, cy + o - R - d),
+                            (cx + o + 4 * R // 5 + d, cy + o - 3 * R // 5)]
+    pts = np.array([p for p in pts if all(-HALF <= v < HALF for v in p)] + [(0, 0), (-HALF, -HALF), (HALF - 1, HALF - 1)])
+    _check(ctx, pts, reqs)
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 1025])
+def test_leaf_remainders_and_grid_borders(ctx, n):
+    rng = np.random.default_rng(n)
+    edge = rng.choice([-HALF, HALF - 1, 0, -1], size=(n, 2))
+    pts = np.where(rng.random((n, 2)) < 0.5, edge, rng.integers(-HALF, HALF, (n, 2)))
+    _check(ctx, pts, [[0, 0, 0, 16], [0, 0, 0, 1024], [1, 0, 0, 40], [1, 1, 1, 1], [2, 3, 0, 512], [5, 31, 31, 32]])
+
+
+def test_crowded_and_sparse_leaves(ctx):
+    """Clusters far narrower than a pixel, duplicates, and lone points, at
+    radii from a sixteenth of a pixel to 64 px."""
+    rng = np.random.default_rng(9)
+    c = rng.integers(-2 ** 20, 2 ** 20, (40, 2))
+    crowd = (c[rng.integers(0, 40, 60_000)] + rng.integers(-300, 300, (60_000, 2)))
+    pts = np.concatenate([crowd, np.repeat(c, 50, axis=0), rng.integers(-2 ** 22, 2 ** 22, (500, 2))])
+    reqs = gen.density_tiles(pts.astype(np.int32), 6, 7, 16, [1, 16, 33, 130], seed=5)
+    _check(ctx, pts, np.concatenate([reqs, [[9, 256, 256, 1024], [12, 2048, 2048, 700]]]))
+
+
+@pytest.mark.parametrize("radius", [0, 1, 46340, 46341, 3_000_003, 1 << 29])
+def test_ground_radii(ctx, radius):
+    rng = np.random.default_rng(11)
+    pts = rng.integers(-2 ** 24, 2 ** 24, (3000, 2))
+    _check(ctx, pts, [[5, 16, 16, 1], [8, 128, 127, 1], [13, 4096, 4095, 1], [19, 262144, 262143, 1], [0, 0, 0, 1]],
+           radius=radius, batches=(1, 150))
