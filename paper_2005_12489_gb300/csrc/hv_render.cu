@@ -201,8 +201,6 @@ struct Src {
     const int32_t* nodes;        // node array (for the read log)
     const int32_t* const* lvl;   // lvl[l] = first node of level l
     const uint32_t* lvl_n;       // lvl_n[l] = nodes of level l
-    int4* seg_scratch;           // per warp kSegScratch int4 (segment leaves)
-    uint16_t* pair_scratch;      // per warp kPairCap pairs (segment leaves)
 };
 
 // Per-lane state of one 8 x 4 pixel block (lane l = pixel (l & 7, l >> 3)).
@@ -220,19 +218,6 @@ struct Lane {
     int32_t bx0, by0;      // warp-uniform: centre of the block's first pixel
     int L;                 // warp-uniform: log2 of the pixel size
 };
-
-// Fold per-sample coverage masks (bit l: lane l's sample k was covered) into
-// the warp's undecided state.
-__device__ __forceinline__ void apply_cover(Lane& s, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
-                                            int lane) {
-    s.Uk[0] &= ~c0;
-    s.Uk[1] &= ~c1;
-    s.Uk[2] &= ~c2;
-    s.Uk[3] &= ~c3;
-    s.U = s.Uk[0] | s.Uk[1] | s.Uk[2] | s.Uk[3];
-    s.und = ((s.Uk[0] >> lane) & 1u) | (((s.Uk[1] >> lane) & 1u) << 1) | (((s.Uk[2] >> lane) & 1u) << 2) |
-            (((s.Uk[3] >> lane) & 1u) << 3);
-}
 
 // Lanes of the block that have a sample within Chebyshev distance `ext` of
 // the box [x0, x1] x [y0, y1]: a pixel column c qualifies when its centre
@@ -253,112 +238,6 @@ __device__ __forceinline__ uint32_t rect_lanes(const Lane& s, int32_t x0, int32_
     uint32_t col = (0xFFu << c0) & (0xFFu >> (7 - c1));
     uint32_t rows = (0x01010101u << (8 * r0)) & (0x01010101u >> (8 * (3 - r1)));
     return col * rows;
-}
-
-// Does the box [x0, x1] x [y0, y1] come within Euclidean distance R of an
-// undecided sample of one of the lanes in `cand`?  Exact for every sample;
-// stops at the first that qualifies.
-__device__ __forceinline__ bool round_reach(const Lane& s, int32_t x0, int32_t y0, int32_t x1,
-                                            int32_t y1, uint32_t cand) {
-    // box edges relative to the block's first pixel centre, clamped to
-    // +-2^30 (32-bit arithmetic below): a clamped edge lies more than
-    // 2^30 - 2^26 > R from every sample, so it never decides a gap within R
-    const int32_t ax = max(min(x0 - s.bx0, kGridHalf), -kGridHalf), bx = max(min(x1 - s.bx0, kGridHalf), -kGridHalf);
-    const int32_t ay = max(min(y0 - s.by0, kGridHalf), -kGridHalf), by = max(min(y1 - s.by0, kGridHalf), -kGridHalf);
-    while (cand) {
-        int l = __ffs(cand) - 1;
-        cand &= cand - 1;
-        const int32_t sx = (l & 7) << s.L, sy = (l >> 3) << s.L;
-        const uint32_t gxm = (uint32_t)max(max(ax - (sx - s.off), (sx - s.off) - bx), 0);
-        const uint32_t gxp = (uint32_t)max(max(ax - (sx + s.off), (sx + s.off) - bx), 0);
-        const uint32_t gym = (uint32_t)max(max(ay - (sy - s.off), (sy - s.off) - by), 0);
-        const uint32_t gyp = (uint32_t)max(max(ay - (sy + s.off), (sy + s.off) - by), 0);
-        const uint64_t xm = (uint64_t)gxm * gxm, xp = (uint64_t)gxp * gxp;
-        const uint64_t ym = (uint64_t)gym * gym, yp = (uint64_t)gyp * gyp;
-        const uint64_t R2 = (uint64_t)s.R2;
-        const bool h0 = (s.Uk[0] >> l) & 1u && xm + ym <= R2;
-        const bool h1 = (s.Uk[1] >> l) & 1u && xp + ym <= R2;
-        const bool h2 = (s.Uk[2] >> l) & 1u && xm + yp <= R2;
-        const bool h3 = (s.Uk[3] >> l) & 1u && xp + yp <= R2;
-        if (h0 | h1 | h2 | h3) return true;
-    }
-    return false;
-}
-
-// Lanes `cm` can reach and one of their undecided samples really is within
-// reach.  For the fill (R = 0, centres) the Chebyshev test is already exact.
-template <class V>
-__device__ __forceinline__ bool reaches(const Lane& s, uint32_t cm, int32_t x0, int32_t y0, int32_t x1, int32_t y1) {
-    uint32_t cand = cm & s.U;
-    if (!cand) return false;
-    return V::kFill || round_reach(s, x0, y0, x1, y1, cand);
-}
-
-// One box against the lanes' own undecided samples (lanes in `lanes` only,
-// each lane its four samples, no loop): whether the box comes within R of
-// any of them.  The same exact test as round_reach, transposed.
-__device__ __forceinline__ bool box_reach_lanes(const Lane& s, int32_t x0, int32_t y0, int32_t x1, int32_t y1,
-                                                uint32_t lanes, int lane) {
-    bool hit = false;
-    if ((lanes >> lane) & 1u) {
-        const int32_t ax = max(min(x0 - s.bx0, kGridHalf), -kGridHalf), bx = max(min(x1 - s.bx0, kGridHalf), -kGridHalf);
-        const int32_t ay = max(min(y0 - s.by0, kGridHalf), -kGridHalf), by = max(min(y1 - s.by0, kGridHalf), -kGridHalf);
-        const int32_t sx = (lane & 7) << s.L, sy = (lane >> 3) << s.L;
-        const uint32_t gxm = (uint32_t)max(max(ax - (sx - s.off), (sx - s.off) - bx), 0);
-        const uint32_t gxp = (uint32_t)max(max(ax - (sx + s.off), (sx + s.off) - bx), 0);
-        const uint32_t gym = (uint32_t)max(max(ay - (sy - s.off), (sy - s.off) - by), 0);
-        const uint32_t gyp = (uint32_t)max(max(ay - (sy + s.off), (sy + s.off) - by), 0);
-        const uint64_t R2 = (uint64_t)s.R2;
-        const uint64_t xm = (uint64_t)gxm * gxm, xp = (uint64_t)gxp * gxp;
-        const uint64_t ym = (uint64_t)gym * gym, yp = (uint64_t)gyp * gyp;
-        hit = ((s.und & 1u) && xm + ym <= R2) || ((s.und & 2u) && xp + ym <= R2) ||
-              ((s.und & 4u) && xm + yp <= R2) || ((s.und & 8u) && xp + yp <= R2);
-    }
-    return __any_sync(kFull, hit);
-}
-
-// Pixels of the block whose centre lies within E of the segment's line,
-// E = R + 2 off + slack >= R + off * sqrt 2 (a covered sample's pixel centre
-// is that close): in pixel row r the centres (c ps, r ps), relative to the
-// block's first centre, satisfy |c A + K_r| <= B with A = ps dy,
-// K_r = cross((0, r ps) - P, d), B = E |d|, P a point within 2 units of the
-// line (the centre of the piece box: a piece runs corner to corner of it).
-// Single precision with every bound widened by more than its rounding error
-// (relative 2^-20 of the magnitudes involved, plus a column): a superset of
-// the pixels the exact test can cover.
-__device__ __forceinline__ uint32_t line_lanes(const Lane& s, int32_t px, int32_t py, int32_t dx, int32_t dy) {
-    const float fdx = (float)dx, fdy = (float)dy, fpx = (float)px, fpy = (float)py;
-    const float dn = sqrtf(fmaf(fdx, fdx, fdy * fdy));
-    const float E = (float)(s.ext + s.off + 2) + (fabsf(fpx) + fabsf(fpy)) * 0x1p-22f;
-    const float B = E * dn * (1.0f + 0x1p-20f);
-    const float ps = (float)(1 << s.L);
-    const float A = ps * fdy;
-    const float inv = A != 0.f ? 1.0f / A : 0.f;
-    uint32_t m = 0u;
-#pragma unroll
-    for (int r = 0; r < kBH; r++) {
-        const float t1 = -fpx * fdy, t2 = fmaf((float)r, ps, -fpy) * fdx;
-        const float K = t1 - t2;
-        const float mag = fabsf(t1) + fabsf(t2) + B;
-        uint32_t row;
-        if (A == 0.f) {
-            row = fabsf(K) <= B + mag * 0x1p-20f ? 0xFFu : 0u;
-        } else {
-            float lo = (-B - K) * inv, hi = (B - K) * inv;
-            if (inv < 0.f) {
-                const float t = lo;
-                lo = hi;
-                hi = t;
-            }
-            const float err = fmaf(mag * fabsf(inv), 0x1p-20f, 1.0f) + (fabsf(lo) + fabsf(hi)) * 0x1p-20f;
-            lo = fmaxf(lo - err, -1.f);
-            hi = fminf(hi + err, 8.f);
-            const int c0 = max((int)ceilf(lo), 0), c1 = min((int)floorf(hi), 7);
-            row = c0 <= c1 ? (0xFFu << c0) & (0xFFu >> (7 - c1)) : 0u;
-        }
-        m |= row << (8 * r);
-    }
-    return m;
 }
 
 // Pixels of the block whose centre the edge e crosses strictly to the right
@@ -391,186 +270,9 @@ __device__ __forceinline__ uint32_t crossing_columns(int4 e, const Lane& s, int3
     return m;
 }
 
-// ---- leaf visitors -----------------------------------------------------------
-// Points and segments: each lane takes one object of the leaf and evaluates
-// the exact predicate on the undecided samples within its reach; the
-// per-sample hits are OR-reduced over the warp.
-
-// Per warp, a segment leaf's pieces (their screen parameters, below) and its
-// (piece, pixel) pairs in reach are staged
-// in shared memory, and the warp's lanes take the pairs in turn: a leaf whose
-// few pieces in reach each reach many pixels costs ceil(pairs / 32) rounds of
-// exact tests instead of the largest piece's pixel count.
-constexpr int kSegScratch = 64;   // 16-byte slots per warp: two per piece
-constexpr int kPairCap = 128;     // pairs per warp and round of staging
-static_assert(kSegScratch * kWarps <= kFCap, "segment scratch exceeds a frontier buffer");
-static_assert(kPairCap * kWarps * 2 <= kFCap * 4, "pair scratch exceeds a frontier id buffer");
-
-template <bool kLineLayer>
-struct SegLeaf {
-    static constexpr bool kFill = false;
-    static constexpr bool kOutline = !kLineLayer;   // the outline of a polygon layer
-    // frontier entries listed by their Chebyshev reach, tested exactly when
-    // taken (measured faster for segments, slower for points)
-    static constexpr bool kExactWhenTaken = true, kScanChebyshev = true, kChildChebyshev = false;
-    static constexpr bool kOneVisitSite = !kLineLayer;   // polygon outlines
-    __device__ static uint32_t visit(const Params& p, const Src& src, uint32_t leaf, Lane& s, int lane) {
-        if ((uint64_t)leaf * 32 >= src.n) {
-            if (lane == 0) check_failed(p, 4, leaf);
-            return kVisitEmpty;
-        }
-        uint64_t i = (uint64_t)leaf * 32 + lane;
-        log_read(p, kLogLeaf, leaf, lane);
-        // a record is a piece: the whole segment and the box of its piece
-        int4 o = make_int4(0, 0, 0, 0);   // padding: never in reach (empty piece box)
-        int4 pb = make_int4(kEmptyLo, kEmptyLo, kEmptyHi, kEmptyHi);
-        if (i < src.n) {
-            o = __ldg((const int4*)src.obj + 2 * i);
-            pb = __ldg((const int4*)src.obj + 2 * i + 1);
-        }
-        const int32_t sx0 = pb.x, sy0 = pb.y, sx1 = pb.z, sy1 = pb.w;
-        uint32_t pm = rect_lanes(s, sx0, sy0, sx1, sy1) & s.U;
-        if (!__any_sync(kFull, pm != 0)) return kVisitEmpty;
-        const uint32_t U_before = s.U;
-        // a piece box much larger than the pixels: keep the pixels near the line
-        if (__reduce_max_sync(kFull, (uint32_t)__popc(pm)) > 8u)
-            pm &= line_lanes(s, mid32(sx0, sx1) - s.bx0, mid32(sy0, sy1) - s.by0, o.z - o.x, o.w - o.y);
-        // the segment relative to the block's first pixel centre (grid
-        // coordinates lie in [-2^30, 2^30), so the differences fit 32 bits);
-        // 32-bit products when both endpoints are within 2^30 of it, else the
-        // absolute 64-bit test
-        const int32_t ax = o.x - s.bx0, ay = o.y - s.by0, bx = o.z - s.bx0, by = o.w - s.by0;
-        const bool near = max(max(abs(ax), abs(ay)), max(abs(bx), abs(by))) <= kGridHalf;
-        uint32_t c[4] = {0u, 0u, 0u, 0u};
-        if (__any_sync(kFull, pm != 0 && !near)) {
-            // a segment reaching from beyond 2^30 of the block (grid-spanning
-            // edges at low zoom): each lane its own piece, absolute 64-bit tests
-            while (pm) {
-                const int l = __ffs(pm) - 1;
-                pm &= pm - 1;
-                const int32_t px = (l & 7) << s.L, py = (l >> 3) << s.L;
-#pragma unroll
-                for (int k = 0; k < 4; k++) {
-                    if (k < s.nk && ((s.Uk[k] >> l) & 1u)) {
-                        const int32_t sx = s.bx0 + px + ((k & 1) ? s.off : -s.off);
-                        const int32_t sy = s.by0 + py + ((k & 2) ? s.off : -s.off);
-                        if (segment_within(o.x, o.y, o.z, o.w, sx, sy, s.R2)) c[k] |= 1u << l;
-                    }
-                }
-            }
-            return finish(s, c, U_before, lane);
-        }
-        const int warp = threadIdx.x >> 5;
-        int4* const seg = src.seg_scratch + warp * kSegScratch;
-        uint16_t* const pairs = src.pair_scratch + warp * kPairCap;
-        // single-precision screen of the distance test.  Per piece, from exact
-        // int64 values rounded once: the unit direction m = d / |d|, the
-        // line's offset c0 = (d x a) / |d| and the projection offset
-        // e0 = (d . a) / |d|, so that a sample s (relative to the block, its
-        // coordinates exact in single precision) lies at signed distance
-        // m x s - c0 from the line and at m . s - e0 along it from a; the
-        // distance to the closed segment is then |(along - clamp(along, 0,
-        // |d|), across)|.  Every rounding is bounded by 8 units in the last
-        // place of the magnitudes involved (|s| <= 8 ps, |c0|, |e0|, |d|, R);
-        // E1 takes 64 of them plus 2 grid units, and the squared thresholds
-        // another 2^-20: a sample closer than R - E1 is within R, one farther
-        // than R + E1 beyond it, and only the rest is decided exactly.
-        {
-            const int32_t dx = o.z - o.x, dy = o.w - o.y;
-            const int64_t Ls = (int64_t)dx * dx + (int64_t)dy * dy;
-            float mx = 1.f, my = 0.f, c0 = (float)ay, e0 = (float)ax, D = 0.f;   // a point: any direction
-            if (Ls > 0) {
-                D = sqrtf((float)Ls);
-                const float inv = 1.0f / D;
-                mx = (float)dx * inv;
-                my = (float)dy * inv;
-                c0 = (float)((int64_t)dx * ay - (int64_t)dy * ax) * inv;
-                e0 = (float)((int64_t)dx * ax + (int64_t)dy * ay) * inv;
-            }
-            const float fR = (float)(s.ext - s.off);
-            const float E1 = fmaf(0x1p-18f, 32.f * (float)(1 << s.L) + fabsf(c0) + fabsf(e0) + D + fR, 2.f);
-            const float lo = fR - E1, hi = fR + E1;
-            const float lo2 = lo > 0.f ? lo * lo * (1.f - 0x1p-20f) : -1.f;
-            const float hi2 = hi * hi * (1.f + 0x1p-20f);
-            reinterpret_cast<float4*>(seg)[lane] = make_float4(mx, my, c0, e0);
-            reinterpret_cast<float4*>(seg + 32)[lane] = make_float4(D, lo2, hi2, 0.f);
-        }
-        // the lane's pairs are numbered first .. first + popc(pm) - 1
-        const uint32_t cnt = (uint32_t)__popc(pm);
-        uint32_t incl = cnt;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t v = __shfl_up_sync(kFull, incl, d);
-            if (lane >= d) incl += v;
-        }
-        const uint32_t total = __shfl_sync(kFull, incl, 31), first = incl - cnt;
-        const uint32_t tag = (uint32_t)lane << 5;
-        for (uint32_t w0 = 0; w0 < total; w0 += kPairCap) {
-            uint32_t m = pm, g = first - w0;   // unsigned: pairs before the round wrap above kPairCap
-            while (m) {
-                const int l = __ffs(m) - 1;
-                m &= m - 1;
-                if (g < (uint32_t)kPairCap) pairs[g] = (uint16_t)(tag | (uint32_t)l);
-                g++;
-            }
-            __syncwarp();
-            const uint32_t n = min(total - w0, (uint32_t)kPairCap);
-            for (uint32_t j = lane; j < n; j += 32) {
-                const uint32_t e = pairs[j];
-                const int l = e & 31, pc = e >> 5;
-                const float4 A = reinterpret_cast<const float4*>(seg)[pc];
-                const float4 B = reinterpret_cast<const float4*>(seg + 32)[pc];
-                // the pixel's column and row as exact floats (2^23 + c - 2^23)
-                const float col = __int_as_float(0x4B000000 | (l & 7)) - 8388608.f;
-                const float row = __int_as_float(0x4B000000 | (l >> 3)) - 8388608.f;
-                const float fps = (float)(1 << s.L), foff = (float)s.off;
-                const float sxs[2] = {fmaf(col, fps, -foff), fmaf(col, fps, foff)};
-                const float sys[2] = {fmaf(row, fps, -foff), fmaf(row, fps, foff)};
-#pragma unroll
-                for (int k = 0; k < 4; k++) {
-                    if (k < s.nk && ((s.Uk[k] >> l) & 1u)) {
-                        const float sx = sxs[k & 1], sy = sys[k >> 1];
-                        const float across = fmaf(A.x, sy, -fmaf(A.y, sx, A.z));
-                        const float along = fmaf(A.x, sx, fmaf(A.y, sy, -A.w));
-                        const float u = along - fminf(fmaxf(along, 0.f), B.x);
-                        const float q = fmaf(u, u, across * across);
-                        bool hit = q < B.y;
-                        if (!hit && q <= B.z) {
-                            // within the margin: the exact test on the piece's segment
-                            const int4 og = __ldg((const int4*)src.obj + 2 * ((uint64_t)leaf * 32 + pc));
-                            const int32_t gx = og.x - s.bx0, gy = og.y - s.by0, hx = og.z - s.bx0, hy = og.w - s.by0;
-                            const int32_t dx = og.z - og.x, dy = og.w - og.y;
-                            const int32_t isx = ((l & 7) << s.L) + ((k & 1) ? s.off : -s.off);
-                            const int32_t isy = ((l >> 3) << s.L) + ((k & 2) ? s.off : -s.off);
-                            hit = segment_within_rel(gx, gy, hx, hy, dx, dy, (int64_t)dx * dx + (int64_t)dy * dy, -1,
-                                                     INT64_MAX, isx, isy, s.R2);
-                        }
-                        if (hit) c[k] |= 1u << l;
-                    }
-                }
-            }
-            __syncwarp();
-        }
-        return finish(s, c, U_before, lane);
-    }
-
-    // Fold the lanes' hits into the warp's undecided state.
-    __device__ static uint32_t finish(Lane& s, const uint32_t c[4], uint32_t U_before, int lane) {
-        const uint32_t c0 = __reduce_or_sync(kFull, c[0]), c1 = __reduce_or_sync(kFull, c[1]);
-        const uint32_t c2 = __reduce_or_sync(kFull, c[2]), c3 = __reduce_or_sync(kFull, c[3]);
-        apply_cover(s, c0, c1, c2, c3, lane);
-        return (c0 | c1 | c2 | c3) & U_before ? kVisitDecided : kVisitTested;
-    }
-};
-
 // Polygon boxes: a leaf holds 32 polygon boxes; for each box that contains an
 // unfilled pixel centre, count that polygon's own edges crossing the ray.
 struct FillLeaf {
-    static constexpr bool kFill = true;
-    static constexpr bool kOutline = false;
-    // R = 0 at the centres: the Chebyshev test is already exact
-    static constexpr bool kExactWhenTaken = false, kScanChebyshev = false, kChildChebyshev = false;
-    static constexpr bool kOneVisitSite = true;
     __device__ static uint32_t visit(const Params& p, const Src& src, uint32_t leaf, Lane& s, int lane) {
         if ((uint64_t)leaf * 32 >= src.n) {
             if (lane == 0) check_failed(p, 4, leaf);
@@ -652,90 +354,21 @@ template <class V>
 __device__ __forceinline__ uint32_t child_hits(const Params& p, const Src& src,
                                                const int32_t* base, Lane& s, int lane, uint32_t* lm) {
     if (p.log != nullptr)
-        log_read(p, V::kFill ? kLogPolyNode : kLogNode, (uint64_t)(base - src.nodes) >> 7, lane);
+        log_read(p, kLogPolyNode, (uint64_t)(base - src.nodes) >> 7, lane);
     int32_t x0 = __ldg(base + lane), y0 = __ldg(base + 32 + lane);
     int32_t x1 = __ldg(base + 64 + lane), y1 = __ldg(base + 96 + lane);
     uint32_t cm = rect_lanes(s, x0, y0, x1, y1);
     lm[lane] = cm;
-    if constexpr (V::kChildChebyshev)
-        return __ballot_sync(kFull, (cm & s.U) != 0u);
-    else
-        return __ballot_sync(kFull, reaches<V>(s, cm, x0, y0, x1, y1));
+    return __ballot_sync(kFull, (cm & s.U) != 0u);
 }
 
-// Depth-first descent from node `node` at level `level` (>= 1).  The stack
-// keeps, per level, the node whose children are being visited, the children
-// still to visit, and each child's lane reach (re-tested against the
+// Depth-first descent from node `node` at level `level` (0: a leaf, which the
+// one visit below takes too, so that the leaf code exists once in the kernel).
+// The stack keeps, per level, the node whose children are being visited, the
+// children still to visit, and each child's lane reach (re-tested against the
 // shrinking undecided set before every visit).
 template <class V, bool kProf>
 __device__ void descend(const Params& p, Smem& sm, const Src& src, int level, uint32_t node, Lane& s,
-                        int lane, int warp) {
-    uint32_t* stk_node = sm.stk_node[warp];
-    uint32_t* stk_mask = sm.stk_mask[warp];
-    int lvl = level;
-    if (level < 1 || level > kMaxLevels || node >= src.lvl_n[level]) {
-        if (lane == 0) check_failed(p, 2, ((uint64_t)level << 40) | node);
-        return;
-    }
-    uint32_t m0 = child_hits<V>(p, src, src.lvl[lvl] + (uint64_t)node * 128, s, lane,
-                             sm.lanemask[warp][lvl]);
-    prof_add<kProf>(sm, kPNodeVisits, 1, lane);
-    if (s.U == 0) return;
-    stk_node[lvl] = node;
-    stk_mask[lvl] = m0;
-    __syncwarp();
-    while (true) {
-        uint32_t m = stk_mask[lvl];
-        m = __ballot_sync(kFull, ((m >> lane) & 1u) && (sm.lanemask[warp][lvl][lane] & s.U));
-        if (m == 0) {
-            if (lvl == level) break;
-            lvl++;
-            continue;
-        }
-        int c = __ffs(m) - 1;
-        uint32_t child = stk_node[lvl] * 32u + (uint32_t)c;
-        __syncwarp();
-        stk_mask[lvl] = m & (m - 1);
-        __syncwarp();
-        if constexpr (V::kChildChebyshev) {
-            // listed by its Chebyshev reach only: the exact test now
-            const int32_t* nb = src.lvl[lvl] + (uint64_t)stk_node[lvl] * 128;
-            if (!box_reach_lanes(s, __ldg(nb + c), __ldg(nb + 32 + c), __ldg(nb + 64 + c),
-                                                  __ldg(nb + 96 + c), sm.lanemask[warp][lvl][c] & s.U, lane))
-                continue;
-        }
-        if (lvl == 1) {
-            const long long t0 = tick<kProf>();
-            const uint32_t how = V::visit(p, src, child, s, lane);
-            prof_since<kProf>(sm, kPLeaf, t0, lane);
-            prof_add<kProf>(sm, kPLeafVisits, 1, lane);
-            prof_add<kProf>(sm, how == kVisitEmpty ? kPLeafEmpty : kPLeafDecided, how != kVisitTested, lane);
-            if (s.U == 0) return;
-        } else {
-            if (child >= src.lvl_n[lvl - 1]) {
-                if (lane == 0) check_failed(p, 3, ((uint64_t)(lvl - 1) << 40) | child);
-                continue;
-            }
-            lvl--;
-            uint32_t hm = child_hits<V>(p, src, src.lvl[lvl] + (uint64_t)child * 128, s, lane,
-                                     sm.lanemask[warp][lvl]);
-            prof_add<kProf>(sm, kPNodeVisits, 1, lane);
-            if (s.U == 0) return;
-            stk_node[lvl] = child;
-            stk_mask[lvl] = hm;
-            __syncwarp();
-        }
-    }
-}
-
-// The same descent for visitors with kOneVisitSite, also from a leaf (level
-// 0, a frontier of leaves): their leaves are reached only through the one
-// visit below, so the leaf code exists once in the kernel.  The polygon
-// kernels measured faster that way (instruction fetch); points and line
-// layers slower, so they keep the form above and visit a frontier of
-// leaves directly.
-template <class V, bool kProf>
-__device__ void descend_one_site(const Params& p, Smem& sm, const Src& src, int level, uint32_t node, Lane& s,
                         int lane, int warp) {
     uint32_t* stk_node = sm.stk_node[warp];
     uint32_t* stk_mask = sm.stk_mask[warp];
@@ -767,13 +400,6 @@ __device__ void descend_one_site(const Params& p, Smem& sm, const Src& src, int 
             __syncwarp();
             stk_mask[lvl] = m & (m - 1);
             __syncwarp();
-            if constexpr (V::kChildChebyshev) {
-                // listed by its Chebyshev reach only: the exact test now
-                const int32_t* nb = src.lvl[lvl] + (uint64_t)stk_node[lvl] * 128;
-                if (!box_reach_lanes(s, __ldg(nb + c), __ldg(nb + 32 + c), __ldg(nb + 64 + c),
-                                                      __ldg(nb + 96 + c), sm.lanemask[warp][lvl][c] & s.U, lane))
-                    continue;
-            }
             if (lvl > 1) {
                 if (child >= src.lvl_n[lvl - 1]) {
                     if (lane == 0) check_failed(p, 3, ((uint64_t)(lvl - 1) << 40) | child);
@@ -1086,8 +712,7 @@ __device__ void blocks_pass(const Params& p, Smem& sm, const Src& src, const Src
         s.bx0 = X0 + (bx * kBW) * ps + (ps >> 1);
         s.by0 = Y0 + (strip * p.rows + by * kBH) * ps + (ps >> 1);
         s.R2 = (int64_t)R * R;
-        bool centre_only = mask_mode;
-        if constexpr (V::kFill) centre_only = mask_mode || !p.fill_aa;
+        const bool centre_only = mask_mode || !p.fill_aa;
         if (centre_only) {
             s.off = 0;
             s.und = 1u;
@@ -1097,18 +722,9 @@ __device__ void blocks_pass(const Params& p, Smem& sm, const Src& src, const Src
             s.und = 15u;
             s.nk = 4;
         }
-        s.ext = (V::kFill ? 0 : R) + s.off;
+        s.ext = s.off;
         s.U = kFull;
         for (int k = 0; k < 4; k++) s.Uk[k] = k < s.nk ? kFull : 0u;
-        if constexpr (V::kOutline) {
-            if (mask_mode && p.pat_w == 0) {
-                // a MASK pixel whose centre is already filled is decided
-                // (unless a pattern may leave it transparent)
-                const uint32_t open = __ballot_sync(kFull, (sm.res[jl * kTile + i] >> kResFillShift) == 0);
-                s.U = s.Uk[0] = open;
-                s.und = (open >> lane) & 1u;
-            }
-        }
         uint32_t und0 = s.und;
         {
             // this block's column list, or the whole frontier
@@ -1134,65 +750,32 @@ __device__ void blocks_pass(const Params& p, Smem& sm, const Src& src, const Src
                         cm = rect_lanes(s, fbx.x, fbx.y, fbx.z, fbx.w);
                     }
                 }
-                uint32_t mm;
-                if constexpr (V::kScanChebyshev)
-                    mm = __ballot_sync(kFull, (cm & s.U) != 0u);
-                else
-                    mm = __ballot_sync(kFull, reaches<V>(s, cm, fbx.x, fbx.y, fbx.z, fbx.w));
+                uint32_t mm = __ballot_sync(kFull, (cm & s.U) != 0u);
                 prof_add<kProf>(sm, kPFrontierEntries, (unsigned long long)min(32, lcnt - c0), lane);
                 while (mm) {
                     int k = __ffs(mm) - 1;
                     mm &= mm - 1;
                     const int ek = __shfl_sync(kFull, e, k);
-                    if constexpr (V::kExactWhenTaken) {
-                        const int4 bk = sm.fbox[fb][ek];
-                        if (!box_reach_lanes(s, bk.x, bk.y, bk.z, bk.w,
-                                                              __shfl_sync(kFull, cm, k) & s.U, lane))
-                            continue;
-                    }
                     uint32_t id = sm.fid[fb][ek];
                     const long long t0 = tick<kProf>();
-                    if constexpr (V::kOneVisitSite) {
-                        descend_one_site<V, kProf>(p, sm, src, f_level, id, s, lane, warp);
-                    } else if (f_level == 0) {
-                        const uint32_t how = V::visit(p, src, id, s, lane);
-                        prof_since<kProf>(sm, kPLeaf, t0, lane);
-                        prof_add<kProf>(sm, kPLeafVisits, 1, lane);
-                        prof_add<kProf>(sm, how == kVisitEmpty ? kPLeafEmpty : kPLeafDecided, how != kVisitTested,
-                                        lane);
-                    } else {
-                        descend<V, kProf>(p, sm, src, f_level, id, s, lane, warp);
-                    }
+                    descend<V, kProf>(p, sm, src, f_level, id, s, lane, warp);
                     // everything below the frontier (leaves included)
                     prof_since<kProf>(sm, kPDescend, t0, lane);
                     // drop frontier entries that no longer reach an undecided lane
-                    if constexpr (V::kExactWhenTaken)
-                        mm &= __ballot_sync(kFull, ((mm >> lane) & 1u) && (cm & s.U) != 0u);
-                    else
-                        mm &= __ballot_sync(kFull, ((mm >> lane) & 1u) &&
-                                                       reaches<V>(s, cm, fbx.x, fbx.y, fbx.z, fbx.w));
+                    mm &= __ballot_sync(kFull, ((mm >> lane) & 1u) && (cm & s.U) != 0u);
                 }
             }
             // objects longer than the learned index's halo live in a side tree
             if (side_top > 0 && s.U) {
                 const long long t0 = tick<kProf>();
-                if constexpr (V::kOneVisitSite)
-                    descend_one_site<V, kProf>(p, sm, side, side_top, 0, s, lane, warp);
-                else
-                    descend<V, kProf>(p, sm, side, side_top, 0, s, lane, warp);
+                descend<V, kProf>(p, sm, side, side_top, 0, s, lane, warp);
                 prof_since<kProf>(sm, kPDescend, t0, lane);
             }
         }
         uint32_t covered = und0 & ~s.und;
         uint8_t r = sm.res[jl * kTile + i];
-        if (V::kFill) {
-            // the centre (1), or the number of super-samples inside (0..4)
-            if (covered) r |= (s.nk == 1 ? 1u : (uint32_t)__popc(covered)) << kResFillShift;
-        } else if (mask_mode) {
-            if (covered) r |= kResCentre;
-        } else {
-            r |= (uint8_t)covered;
-        }
+        // the centre (1), or the number of super-samples inside (0..4)
+        if (covered) r |= (s.nk == 1 ? 1u : (uint32_t)__popc(covered)) << kResFillShift;
         sm.res[jl * kTile + i] = r;
     }
     prof_since<kProf>(sm, kPBlocksWarp, t_active, lane);
@@ -1212,7 +795,7 @@ __device__ void stage(const Params& p, Smem& sm, const TreeArg& t, const void* o
     if (tid == 0) sm.next_block = 0;
     __syncthreads();
     if (m == nullptr)
-        cull(p, t, V::kFill, sm, bx0, by0, bx1, by1, tid);
+        cull(p, t, true, sm, bx0, by0, bx1, by1, tid);
     else
         learned_cull(p, t, *m, halo, sm, bx0, by0, bx1, by1, tid);
     if (tid == 0) prof_since<kProf>(sm, kPCull, t_cull, 0);
@@ -1222,18 +805,14 @@ __device__ void stage(const Params& p, Smem& sm, const TreeArg& t, const void* o
         // the column lists are rebuilt for every pass, also for an empty
         // frontier (a strip reached only by the side tree), so that the
         // blocks never read the lists of an earlier stage
-        bool sub = !mask_mode;   // super-samples
-        if constexpr (V::kFill) sub = !mask_mode && p.fill_aa;
+        const bool sub = !mask_mode && p.fill_aa;   // super-samples
         const int32_t off = sub ? ((1 << (23 - z)) >> 2) : 0;
         const long long t_bin = tick<kProf>();
-        bin_frontier(sm, X0, 23 - z, (V::kFill ? 0 : R) + off, tid);
+        bin_frontier(sm, X0, 23 - z, off, tid);
         if (tid == 0) prof_since<kProf>(sm, kPBin, t_bin, 0);
         const long long t_blocks = tick<kProf>();
-        // the frontier's idle buffer: scratch for segment leaves
-        int4* const seg_scratch = sm.fbox[1 - sm.f_buf];
-        uint16_t* const pair_scratch = reinterpret_cast<uint16_t*>(sm.fid[1 - sm.f_buf]);
-        Src src{obj, ids, t.n_obj, t.nodes, sm.lvl_base[0], sm.lvl_n[0], seg_scratch, pair_scratch};
-        Src side{sobj, sids, st.n_obj, st.nodes, sm.lvl_base[1], sm.lvl_n[1], seg_scratch, pair_scratch};
+        Src src{obj, ids, t.n_obj, t.nodes, sm.lvl_base[0], sm.lvl_n[0]};
+        Src side{sobj, sids, st.n_obj, st.nodes, sm.lvl_base[1], sm.lvl_n[1]};
         blocks_pass<V, kProf>(p, sm, src, side, side_hit ? st.top : 0, X0, Y0, strip, col0, col_shift, z, R, mask_mode,
                               tid);
         __syncthreads();
@@ -1253,15 +832,6 @@ __device__ void stage(const Params& p, Smem& sm, const TreeArg& t, const void* o
 // the instruction cache; fused, the polygon kernel measured 40% slower.
 constexpr int kPolyFill = 3;
 
-// CTAs per SM: four (64 registers) for every kind, measured best for each
-// since the segment leaves share their pairs over the lanes (the line and
-// outline kernels keep a 12-16 byte spill and still run faster than with
-// three).
-template <int kKind>
-struct KindTraits {
-    static constexpr int kBlocksPerSM = 4;
-};
-
 // The pattern texel of global pixel (gx, gy).
 __device__ __forceinline__ uchar4 fill_texel(const Params& p, uint32_t gx, uint32_t gy) {
     return p.pattern[(gy % (uint32_t)p.pat_h) * (uint32_t)p.pat_w + gx % (uint32_t)p.pat_w];
@@ -1279,7 +849,7 @@ __device__ __forceinline__ uint64_t px_offset(int mode, int j, int c) {
 // cols / 8 bytes in every mode), a bit per pixel (centre fill), or with the
 // anti-aliased fill a byte per pixel holding the number of super-samples
 // inside.  This reads them back into the strip's shared results.
-__device__ void decode_fill(const Params& p, const uint8_t* tile_out, Smem& sm, int strip, int col0, int cols,
+__device__ void decode_fill(const Params& p, const uint8_t* tile_out, uint8_t* res, int strip, int col0, int cols,
                             int tid, bool aa_bytes) {
     const int rows = p.rows;
     if (aa_bytes) {
@@ -1287,7 +857,7 @@ __device__ void decode_fill(const Params& p, const uint8_t* tile_out, Smem& sm, 
         for (int k = tid; k < rows * wpr; k += kThreads) {
             const int jl = k >> wsh, w = k & (wpr - 1);
             const uint32_t v = ((const uint32_t*)(tile_out + px_offset(p.mode, strip * rows + jl, col0)))[w];
-            ((uint32_t*)(sm.res + jl * kTile + col0))[w] = (v & 0x07070707u) << kResFillShift;
+            ((uint32_t*)(res + jl * kTile + col0))[w] = (v & 0x07070707u) << kResFillShift;
         }
         return;
     }
@@ -1295,7 +865,7 @@ __device__ void decode_fill(const Params& p, const uint8_t* tile_out, Smem& sm, 
     for (int k = tid; k < rows * wpr; k += kThreads) {
         const int jl = k >> wsh, w = k & (wpr - 1);
         const uint32_t word = ((const uint32_t*)(tile_out + px_offset(p.mode, strip * rows + jl, col0)))[w];
-        uint32_t* r4 = (uint32_t*)(sm.res + jl * kTile + col0 + 32 * w);
+        uint32_t* r4 = (uint32_t*)(res + jl * kTile + col0 + 32 * w);
 #pragma unroll
         for (int q = 0; q < 8; q++) {
             const uint32_t b = word >> (4 * q);
@@ -1308,7 +878,7 @@ __device__ void decode_fill(const Params& p, const uint8_t* tile_out, Smem& sm, 
 // The outline launch of a polygon layer encodes the strip composed over the
 // fill results: per pixel v outline samples, the fill field (centre, or the
 // anti-aliased count), a pattern texel by the global pixel coordinate.
-__device__ void encode_polygons(const Params& p, const Smem& sm, uint8_t* out, int strip, int col0, int cols,
+__device__ void encode_polygons(const Params& p, const uint8_t* res, uint8_t* out, int strip, int col0, int cols,
                                 uint32_t tile, int tid) {
     const int rows = p.rows;
     const hv_tile_req q = p.reqs[tile];
@@ -1319,7 +889,7 @@ __device__ void encode_polygons(const Params& p, const Smem& sm, uint8_t* out, i
             const int jl = tid >> wsh, c = col0 + 32 * (tid & (wpr - 1));
             uint32_t word = 0;
             for (int b = 0; b < 32; b++) {
-                const uint32_t f = sm.res[jl * kTile + c + b];
+                const uint32_t f = res[jl * kTile + c + b];
                 bool filled = (f >> kResFillShift) != 0;
                 if (filled && p.pat_w) filled = fill_texel(p, gx0 + c + b, gy0 + jl).w != 0;
                 if ((f & kResCentre) || filled) word |= 1u << b;
@@ -1331,7 +901,7 @@ __device__ void encode_polygons(const Params& p, const Smem& sm, uint8_t* out, i
         const int upr = cols / 16, ush = __ffs(upr) - 1;
         for (int u = tid; u < rows * upr; u += kThreads) {
             const int jl = u >> ush, c = col0 + 16 * (u & (upr - 1));
-            const uint8_t* r = sm.res + jl * kTile + c;
+            const uint8_t* r = res + jl * kTile + c;
             uint32_t w4[4];
             for (int k = 0; k < 4; k++) {
                 uint32_t v = 0;
@@ -1354,7 +924,7 @@ __device__ void encode_polygons(const Params& p, const Smem& sm, uint8_t* out, i
             const int jl = u >> ush, c = col0 + 4 * (u & (upr - 1));
             uint32_t w[4];
             for (int b = 0; b < 4; b++) {
-                uint32_t f = sm.res[jl * kTile + c + b];
+                uint32_t f = res[jl * kTile + c + b];
                 uint32_t v = __popc(f & 15u);
                 uint32_t a = (255u * v + 2u) >> 2;
                 // fill count: 0..4 anti-aliased, else 4 for a filled centre
@@ -1393,7 +963,7 @@ __device__ void encode_polygons(const Params& p, const Smem& sm, uint8_t* out, i
 // kSplit: the launch splits strips into column parts (p.parts > 1); the
 // full-width instantiation keeps the column arithmetic compile-time constant.
 template <int kKind, bool kProf, bool kSplit>
-__global__ void __launch_bounds__(kThreads, KindTraits<kKind>::kBlocksPerSM) k_render(const Params p) {
+__global__ void __launch_bounds__(kThreads, 4) k_render(const Params p) {
     __shared__ Smem sm;
     const int tid = threadIdx.x;
     const long long t_start = tick<kProf>();
@@ -1410,11 +980,7 @@ __global__ void __launch_bounds__(kThreads, KindTraits<kKind>::kBlocksPerSM) k_r
     if (tile >= n) return;
     hv_tile_req q = p.reqs[tile];
     bool ok = q.z <= 19 && q.x < (1u << q.z) && q.y < (1u << q.z) && (p.R_units >= 0 || (q.r16 >= 1 && q.r16 <= 1024));
-    if constexpr (kKind == HV_LAYER_POLYGONS)
-        decode_fill(p, p.out + (uint64_t)tile * p.tile_bytes, sm, strip, col0, cols, tid,
-                    p.fill_aa && p.mode != HV_MODE_MASK);
-    else
-        for (int k = tid; k < rows * kTile / 4; k += kThreads) ((uint32_t*)sm.res)[k] = 0u;
+    for (int k = tid; k < rows * kTile / 4; k += kThreads) ((uint32_t*)sm.res)[k] = 0u;
     if (!ok) {
         if (tid == 0 && sp == 0) atomicOr(p.status, 1u);
     }
@@ -1426,21 +992,9 @@ __global__ void __launch_bounds__(kThreads, KindTraits<kKind>::kBlocksPerSM) k_r
         const int32_t ps = 1 << (23 - z);
         const int32_t X0 = (int32_t)(-(int64_t)kGridHalf + (int64_t)q.x * ((int64_t)1 << (31 - z)));
         const int32_t Y0 = (int32_t)(-(int64_t)kGridHalf + (int64_t)q.y * ((int64_t)1 << (31 - z)));
-        // at most 2^29 either way (r16 <= 1024, or the buffer limit)
-        int32_t R = (int32_t)q.r16 << (19 - z);
-        if (p.R_units >= 0) R = p.R_units;
-        const int32_t off = mask_mode ? 0 : (ps >> 2);
-        // the CTA's sample box
-        const int32_t sx0 = X0 + col0 * ps + (ps >> 1) - off, sx1 = X0 + (col0 + cols - 1) * ps + (ps >> 1) + off;
-        const int32_t sy0 = Y0 + strip * rows * ps + (ps >> 1) - off;
-        const int32_t sy1 = Y0 + (strip * rows + rows - 1) * ps + (ps >> 1) + off;
         const bool learned = p.use_learned != 0;
-        // Algorithm 1 over segments / polygon edges
-        if constexpr (kKind != kPolyFill)
-            stage<SegLeaf<kKind == HV_LAYER_LINES>, kProf>(p, sm, p.tree, p.obj, nullptr, p.side, p.side_obj, p.side_ids, learned ? &p.lm : nullptr,
-                           p.halo, X0, Y0, strip, col0, col_shift, z, R, mask_mode, sx0 - R, sy0 - R, sx1 + R, sy1 + R, tid);
         // Algorithm 2 over polygon boxes and edges
-        if constexpr (kKind == kPolyFill) {
+        {
             // the CTA's centres, or its super-samples
             const int32_t fo = (p.fill_aa && p.mode != HV_MODE_MASK) ? (ps >> 2) : 0;
             const int32_t cx0 = X0 + col0 * ps + (ps >> 1) - fo, cx1 = X0 + (col0 + cols - 1) * ps + (ps >> 1) + fo;
@@ -1452,10 +1006,10 @@ __global__ void __launch_bounds__(kThreads, KindTraits<kKind>::kBlocksPerSM) k_r
                             cx1, cy1, tid);
         }
     }
-    // ---- encode the strip (Sec. 4.1 Render Tiles) ----
+    // ---- hand the strip's fill over ----
     const long long t_enc = tick<kProf>();
     uint8_t* out = p.out + (uint64_t)tile * p.tile_bytes;
-    if constexpr (kKind == kPolyFill) {
+    {
         // the fill results for the outline part, per pixel row at the start
         // of the row's part of the CTA's own output (see decode_fill)
         if (p.fill_aa && p.mode != HV_MODE_MASK) {
@@ -1474,46 +1028,6 @@ __global__ void __launch_bounds__(kThreads, KindTraits<kKind>::kBlocksPerSM) k_r
                     if (sm.res[jl * kTile + col0 + 32 * w + b] >> kResFillShift) word |= 1u << b;
                 ((uint32_t*)(out + px_offset(p.mode, strip * rows + jl, col0)))[w] = word;
             }
-        }
-    } else if constexpr (kKind == HV_LAYER_POLYGONS) {
-        encode_polygons(p, sm, out, strip, col0, cols, tile, tid);
-    } else if (p.mode == HV_MODE_MASK) {
-        // word w of row j = pixels 32w .. 32w+31
-        const int wpr = cols / 32, wsh = __ffs(wpr) - 1;
-        if (tid < rows * wpr) {
-            const int jl = tid >> wsh, c = col0 + 32 * (tid & (wpr - 1));
-            uint32_t word = 0;
-            for (int b = 0; b < 32; b++)
-                if (sm.res[jl * kTile + c + b] & kResCentre) word |= 1u << b;
-            *(uint32_t*)(out + px_offset(p.mode, strip * rows + jl, c)) = word;
-        }
-    } else if (p.mode == HV_MODE_COVERAGE) {
-        // one uint4 (16 pixels) per thread and step
-        const int upr = cols / 16, ush = __ffs(upr) - 1;
-        for (int u = tid; u < rows * upr; u += kThreads) {
-            const int jl = u >> ush, c = col0 + 16 * (u & (upr - 1));
-            const uint8_t* r = sm.res + jl * kTile + c;
-            uint32_t w4[4];
-            for (int k = 0; k < 4; k++) {
-                uint32_t v = 0;
-                for (int b = 0; b < 4; b++) v |= (uint32_t)__popc(r[4 * k + b] & 15u) << (8 * b);
-                w4[k] = v;
-            }
-            *(uint4*)(out + px_offset(p.mode, strip * rows + jl, c)) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-        }
-    } else {
-        // one uint4 (4 pixels) per thread and step
-        const int upr = cols / 4, ush = __ffs(upr) - 1;
-        for (int u = tid; u < rows * upr; u += kThreads) {
-            const int jl = u >> ush, c = col0 + 4 * (u & (upr - 1));
-            uint32_t w[4];
-            for (int b = 0; b < 4; b++) {
-                const uint32_t v = __popc(sm.res[jl * kTile + c + b] & 15u);
-                const uint32_t a = (255u * v + 2u) >> 2;
-                w[b] = v ? ((uint32_t)p.line.x | ((uint32_t)p.line.y << 8) | ((uint32_t)p.line.z << 16) | (a << 24))
-                         : 0u;
-            }
-            *(uint4*)(out + px_offset(p.mode, strip * rows + jl, c)) = make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
     if constexpr (kProf) {
@@ -1645,9 +1159,7 @@ int launch_render(Layer* L, const hv_tile_req* d_reqs, uint32_t n, int mode, int
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int per_sm = L->kind == HV_LAYER_POINTS ? KindTraits<HV_LAYER_POINTS>::kBlocksPerSM
-                                                  : KindTraits<HV_LAYER_LINES>::kBlocksPerSM;
-    const uint64_t resident = (uint64_t)sms * per_sm;
+    const uint64_t resident = (uint64_t)sms * 4;
     p.rows = (uint64_t)n * 16 >= 2 * resident ? 16 : ((uint64_t)n * 32 >= 2 * resident ? 8 : 4);
     p.strips = kTile / p.rows;
     // batches too small for the GPU even in 4-row strips also split each
@@ -1669,30 +1181,30 @@ int launch_render(Layer* L, const hv_tile_req* d_reqs, uint32_t n, int mode, int
         if (L->kind == HV_LAYER_POINTS)
             k_sweep<HV_LAYER_POINTS, true, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         else if (L->kind == HV_LAYER_LINES)
-            k_render<HV_LAYER_LINES, true, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+            k_sweep<HV_LAYER_LINES, true, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         else {
             k_render<kPolyFill, true, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
             Params q = p;
             q.phases = p.phases + kPN;
-            k_render<HV_LAYER_POLYGONS, true, false><<<(unsigned)grid, kThreads, 0, stream>>>(q);
+            k_sweep<HV_LAYER_POLYGONS, true, false><<<(unsigned)grid, kThreads, 0, stream>>>(q);
         }
     } else if (p.parts > 1) {
         if (L->kind == HV_LAYER_POINTS)
             k_sweep<HV_LAYER_POINTS, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         else if (L->kind == HV_LAYER_LINES)
-            k_render<HV_LAYER_LINES, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+            k_sweep<HV_LAYER_LINES, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         else {
             k_render<kPolyFill, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
-            k_render<HV_LAYER_POLYGONS, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+            k_sweep<HV_LAYER_POLYGONS, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         }
     } else if (L->kind == HV_LAYER_POINTS)
         k_sweep<HV_LAYER_POINTS, false, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
     else if (L->kind == HV_LAYER_LINES)
-        k_render<HV_LAYER_LINES, false, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+        k_sweep<HV_LAYER_LINES, false, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
     else {
         // the fill first: the outline reads its bits and writes the tile
         k_render<kPolyFill, false, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
-        k_render<HV_LAYER_POLYGONS, false, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+        k_sweep<HV_LAYER_POLYGONS, false, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
     }
     HV_CUDA(cudaGetLastError());
     return HV_OK;

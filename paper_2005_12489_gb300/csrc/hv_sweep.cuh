@@ -15,17 +15,22 @@
 // by strips, 600 tiles of 100M clustered points at 2 px take 2.4 M warp
 // instructions per tile where the 8 x 4 block traversal took 5.7 M: 4,000
 // tiles 23.5 -> 11.8 ms; 341 tiles of 100,000 points at zoom 0-4, 1 px, MASK
-// 414 -> 73 us; one tile of 10M points 35 -> 29 us.
+// 414 -> 73 us; one tile of 10M points 35 -> 29 us.  Segments: 4,000 tiles of 50M
+// segments at 1 px 19.7 -> 5.9 ms; the outlines of 1,000 tiles of 2M polygons
+// 12 -> 8.5 ms (dense low-zoom tiles: 390 leaves of short edges per strip, 22
+// pieces and 71 (piece, row) pairs each).
 //
 // Included by hv_render.cu (one translation unit with the block kernels).
 #pragma once
 
 constexpr int kBitStride = 17;   // words per sample row: 512 columns and a pad word (row-parallel reads then hit 32 banks)
-constexpr int kSweepPerSM = 6;   // CTAs per SM (40 registers); measured against 4 and 5 at k_sweep
 constexpr int kSampleRows = 2 * kStripRows;
 static_assert(kSampleRows <= 32, "one lane per sample row");
 
+template <int kKind>
 struct SweepSmem : Front {
+    // polygon outlines: the fill launch's results, and the composed ones for the encode
+    uint8_t res[kKind == HV_LAYER_POLYGONS ? kStripRows * kTile : 16];
     uint32_t bits[kSampleRows * kBitStride];
     int32_t reach[64];
     uint32_t stk_node[kWarps][kMaxLevels + 1];
@@ -152,10 +157,8 @@ __device__ __forceinline__ void fill_reach(int32_t* reach, const Lattice& g, int
     }
 }
 
-// Is a sample of the row within [x0 - w, x1 + w] open?
-__device__ __forceinline__ bool row_open(const uint32_t* row, const Lattice& g, int32_t x0, int32_t x1, int32_t w) {
-    const int lo = max(g.hw - ((w - x0) >> g.s), 0), hi = min(((x1 + w) >> g.s) + g.hw, 2 * g.hw - 1);
-    if (lo > hi) return false;
+// Is a sample of columns lo..hi of the row open?
+__device__ __forceinline__ bool columns_open(const uint32_t* row, int lo, int hi) {
     const int k1 = hi >> 5;
     uint32_t m = ~0u << (lo & 31);
     for (int k = lo >> 5; k < k1; k++) {
@@ -163,6 +166,12 @@ __device__ __forceinline__ bool row_open(const uint32_t* row, const Lattice& g, 
         m = ~0u;
     }
     return (m & (~0u >> (31 - (hi & 31))) & ~*(volatile const uint32_t*)(row + k1)) != 0u;
+}
+
+// Is a sample of the row within [x0 - w, x1 + w] open?
+__device__ __forceinline__ bool row_open(const uint32_t* row, const Lattice& g, int32_t x0, int32_t x1, int32_t w) {
+    const int lo = max(g.hw - ((w - x0) >> g.s), 0), hi = min(((x1 + w) >> g.s) + g.hw, 2 * g.hw - 1);
+    return lo <= hi && columns_open(row, lo, hi);
 }
 
 // Sample rows (one lane each) with an open sample that an object inside the
@@ -246,6 +255,230 @@ __device__ __forceinline__ bool small_box(const Lattice& g, int32_t x0, int32_t 
     return (uint32_t)(x1 - x0) <= most && (uint32_t)(y1 - y0) <= most;
 }
 
+// ---- segments ---------------------------------------------------------------
+
+// A piece of a segment as its row intervals see it, in sample spacings relative
+// to the lattice point (col, row) in the middle of the part of the piece's
+// box that lies in the strip's reach: the unit direction m (my >= 0), the
+// line's signed offset c0 = m x a and the positions ta <= tb of the segment's
+// ends along m.  E bounds the rounding of everything below as a distance from
+// the segment (infinite: the piece's samples are all decided exactly).
+struct PieceRow {
+    float mx, my, c0, ta, tb, E;
+    uint32_t at;      // col + 1024 | (row + 1024) << 16
+    uint32_t span;    // columns within Chebyshev distance R of the box: first | last << 16
+};
+
+__device__ __forceinline__ float rsqrt_approx(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// The line's offset and the nearer end's position along it (from either end
+// the offset is the same; the far end lies |d| beyond the near one).  Inside
+// the reach every coordinate is at most M = the visible box's size + R / h + 3;
+// a near end within 4 M is taken in single precision, one farther away from
+// exact int64 products rounded once, and ends beyond 8 M are cut off there,
+// where they no longer matter.  Root and quotient are good to 2^-22, so the
+// interval ends that draw_row finds are off by fewer than 16 roundings of
+// 2^-22 M; E = 2^-17 M.  The contact point's position t = (..) / my is the one
+// step that a small my magnifies; its error acts squared over 2 R, and
+// pieces too level for that to stay below E (but not exactly level ones, whose
+// contact points are the ends) are left to the exact test.
+__device__ __forceinline__ PieceRow piece_row(const Lattice& g, int4 o, int32_t x0, int32_t y0, int32_t x1, int32_t y1,
+                                              int clo, int chi) {
+    PieceRow q;
+    const int ex0 = max(x0 >> g.s, -g.hw - 1), ex1 = min(x1 >> g.s, g.hw);
+    const int ey0 = max(y0 >> g.s, -g.hh - 1), ey1 = min(y1 >> g.s, g.hh);
+    // (a box beyond one side of the strip: the middle of what is left, near it)
+    const int mc = max(min((ex0 + ex1) >> 1, g.hw), -g.hw - 1), mr = max(min((ey0 + ey1) >> 1, g.hh), -g.hh - 1);
+    q.at = (uint32_t)(mc + g.hw + 1024) | ((uint32_t)(mr + g.hh + 1024) << 16);
+    q.span = (uint32_t)clo | ((uint32_t)chi << 16);
+    const float scale = __int_as_float((127 - g.s) << 23);   // 1 / h
+    const float rho = (float)g.R * scale;
+    const float Y = (float)max(ey1 - ey0, 0) + rho + 3.f;
+    const float M = fmaxf((float)max(ex1 - ex0, 0) + rho + 3.f, Y);
+    q.E = 0x1p-17f * M;
+    if (o.w < o.y || (o.w == o.y && o.z < o.x)) o = make_int4(o.z, o.w, o.x, o.y);
+    // relative to the middle, wrapping: a value that wraps is still beyond 2^29
+    const uint32_t ox = (uint32_t)g.xc + (uint32_t)(mc << g.s), oy = (uint32_t)g.yc + (uint32_t)(mr << g.s);
+    const int32_t ax = (int32_t)((uint32_t)o.x - ox), ay = (int32_t)((uint32_t)o.y - oy);
+    const int32_t bx = (int32_t)((uint32_t)o.z - ox), by = (int32_t)((uint32_t)o.w - oy);
+    const int32_t dx = o.z - o.x, dy = o.w - o.y;
+    const float fx = (float)dx * scale, fy = (float)dy * scale;
+    const float L2 = fmaf(fx, fx, fy * fy);
+    const float inv = L2 > 0.f ? rsqrt_approx(L2) : 0.f, D = L2 * inv;
+    q.mx = L2 > 0.f ? fx * inv : 1.f;
+    q.my = fy * inv;
+    const uint32_t fa = (uint32_t)max(abs(ax), abs(ay)), fb = (uint32_t)max(abs(bx), abs(by));
+    bool from_a = fa <= fb;
+    float near_t;
+    const uint32_t fn = min(fa, fb);
+    if (fn < (1u << 29) && (float)fn * scale <= 4.f * M) {
+        const float nx = (float)(from_a ? ax : bx) * scale, ny = (float)(from_a ? ay : by) * scale;
+        q.c0 = q.mx * ny - q.my * nx;
+        near_t = fmaf(q.mx, nx, q.my * ny);
+    } else {
+        const int64_t wx = (int64_t)g.xc + ((int64_t)mc << g.s), wy = (int64_t)g.yc + ((int64_t)mr << g.s);
+        const int64_t pa = max(llabs(o.x - wx), llabs(o.y - wy)), pb = max(llabs(o.z - wx), llabs(o.w - wy));
+        from_a = pa <= pb;
+        const int64_t nx = (from_a ? o.x : o.z) - wx, ny = (from_a ? o.y : o.w) - wy;
+        // |d| < 2^31 and |n| <= 1.5 * 2^30 keep the sums below 2^63 (beyond: exact tests)
+        const float k = inv * scale;
+        q.c0 = (float)(dx * ny - dy * nx) * scale * k;
+        near_t = (float)(dx * nx + dy * ny) * scale * k;
+        if (min(pa, pb) > 3ll << 29) q.E = __int_as_float(0x7f800000);
+    }
+    q.ta = from_a ? near_t : near_t - D;
+    q.tb = from_a ? near_t + D : near_t;
+    q.ta = fmaxf(fminf(q.ta, 8.f * M), -8.f * M);
+    q.tb = fmaxf(fminf(q.tb, 8.f * M), -8.f * M);
+    const float G = Y + fabsf(q.c0) + rho;
+    if (q.my > 0.f && q.my * q.my * rho * M * 0x1p25f < 4.f * G * G) q.E = __int_as_float(0x7f800000);
+    return q;
+}
+
+// Exact test of one sample (column i of row r), unless it is set already.
+__device__ __forceinline__ void test_sample(uint32_t* bits, const Lattice& g, const int4* seg, int i, int r) {
+    uint32_t* word = bits + r * kBitStride + (i >> 5);
+    if ((*(volatile uint32_t*)word >> (i & 31)) & 1u) return;
+    const int4 o = __ldg(seg);
+    if (segment_within(o.x, o.y, o.z, o.w, g.xc + (i - g.hw) * (1 << g.s), g.yc + (r - g.hh) * (1 << g.s), g.R2))
+        atomicOr(word, 1u << (i & 31));
+}
+
+// The capsule of radius r around a segment meets a row in one interval.  Its
+// left end belongs to the disc around the contact point t = (y - c0 mx - r mx)
+// / my, cut off at the segment's ends (the leftmost point in the row of that
+// disc if it reaches the row; if it does not, neither does the capsule), and
+// the right end likewise with + r mx.
+//
+// draw_row_slow: the rows that graze the capsule, where an end moves by much
+// more than a rounding for one, and pieces without a finite E.  Columns inside
+// the interval of radius R - E are covered, columns outside that of R + E are
+// not, and those between take the exact test.
+__device__ __noinline__ void draw_row_slow(uint32_t* bits, const Lattice& g, const PieceRow q, const int4* seg, int r) {
+    const int col = (int)(q.at & 0xffffu) - 1024, row = (int)(q.at >> 16) - 1024;
+    const int clo = (int)(q.span & 0xffffu) - col, chi = (int)(q.span >> 16) - col;
+    const float rho = (float)g.R * __int_as_float((127 - g.s) << 23);
+    const float ym = (float)(r - row) - q.c0 * q.mx, xm = q.c0 * q.my, inv = rcp_approx(q.my);
+    int lo[2], hi[2];
+    bool met[2];
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+        const float rad = k ? rho - q.E : rho + q.E, r2 = rad * rad, rm = rad * q.mx;
+        const float tl = fminf(fmaxf((ym - rm) * inv, q.ta), q.tb), tr = fminf(fmaxf((ym + rm) * inv, q.ta), q.tb);
+        const float dl = fmaf(-tl, q.my, ym), dr = fmaf(-tr, q.my, ym);
+        // (a graze: the half-chord's square is rounding alone, widened outside)
+        const float wide = k ? 0.f : rad * q.E;
+        const float al = fmaf(-dl, dl, r2) + wide, ar = fmaf(-dr, dr, r2) + wide;
+        lo[k] = max(__float2int_ru(fmaf(tl, q.mx, -xm) - sqrt_approx(fmaxf(al, 0.f))), clo);
+        hi[k] = min(__float2int_rd(fmaf(tr, q.mx, -xm) + sqrt_approx(fmaxf(ar, 0.f))), chi);
+        met[k] = k ? rad > 0.f && fminf(al, ar) >= 0.f : fmaxf(al, ar) >= 0.f;
+    }
+    if (!met[0] || lo[0] > hi[0]) return;
+    lo[1] = max(lo[1], lo[0]);
+    hi[1] = min(hi[1], hi[0]);
+    if (met[1] && lo[1] <= hi[1])
+        set_columns(bits + r * kBitStride, lo[1] + col, hi[1] + col);
+    else
+        lo[1] = hi[0] + 1, hi[1] = hi[0];
+    for (int c = lo[0]; c <= hi[0]; c++) {
+        if (c == lo[1]) c = hi[1] + 1;
+        if (c <= hi[0]) test_sample(bits, g, seg, c + col, r);
+    }
+}
+
+// Set the samples of row r within R of the segment.  Where both discs meet the
+// row well inside (half-chords w with w^2 >= 8 R E), a distance error of E
+// moves an end by E R / w, and by at most an eighth more for the curvature:
+// a column nearer to the end than 1.25 E R / w takes the exact test, every
+// other column is decided by its side of the end.
+__device__ __forceinline__ void draw_row(uint32_t* bits, const Lattice& g, const PieceRow& q, const int4* seg, int r) {
+    const int col = (int)(q.at & 0xffffu) - 1024, row = (int)(q.at >> 16) - 1024;
+    const float rho = (float)g.R * __int_as_float((127 - g.s) << 23);
+    const float ym = (float)(r - row) - q.c0 * q.mx, xm = q.c0 * q.my, inv = rcp_approx(q.my);
+    const float r2 = rho * rho, rm = rho * q.mx, rE = rho * q.E;
+    const float tl = fminf(fmaxf((ym - rm) * inv, q.ta), q.tb), tr = fminf(fmaxf((ym + rm) * inv, q.ta), q.tb);
+    const float dl = fmaf(-tl, q.my, ym), dr = fmaf(-tr, q.my, ym);
+    const float al = fmaf(-dl, dl, r2), ar = fmaf(-dr, dr, r2);
+    if (!(fminf(al, ar) >= 8.f * rE) || q.E >= rho) {
+        // beyond R + E of the row both half-chords are imaginary
+        if (!(fmaxf(al, ar) < -8.f * rE - 2.f * q.E * q.E)) draw_row_slow(bits, g, q, seg, r);
+        return;
+    }
+    const float wl = sqrt_approx(al), wr = sqrt_approx(ar);
+    const float xl = fmaf(tl, q.mx, -xm) - wl, xr = fmaf(tr, q.mx, -xm) + wr;
+    const float el = 1.25f * rE * rcp_approx(wl), er = 1.25f * rE * rcp_approx(wr);
+    const float nl = rintf(xl), nr = rintf(xr);
+    const bool vl = fabsf(xl - nl) <= el, vr = fabsf(xr - nr) <= er;
+    const int il = (int)nl, ir = (int)nr;
+    const int clo = (int)(q.span & 0xffffu) - col, chi = (int)(q.span >> 16) - col;
+    // a doubtful column is left out of the interval and tested
+    const int lo = max(il + (vl || nl < xl ? 1 : 0), clo), hi = min(ir - (vr || nr > xr ? 1 : 0), chi);
+    if (lo <= hi) set_columns(bits + r * kBitStride, lo + col, hi + col);
+    if (vl && il >= clo && il <= chi) test_sample(bits, g, seg, il + col, r);
+    if (vr && ir >= clo && ir <= chi) test_sample(bits, g, seg, ir + col, r);
+}
+
+// A segment leaf: 32 pieces, each with a run of open rows that it reaches.
+// The (piece, row) pairs are numbered through by a prefix sum over the lanes
+// and the lanes take them in turn (each finds its piece by a binary search
+// over the sums), so a leaf costs ceil(pairs / 32) rounds whatever the pieces'
+// heights.
+__device__ __forceinline__ void draw_segments(const Params& p, const Src& src, uint32_t* bits, const Lattice& g,
+                                              uint32_t leaf, uint32_t rows, int lane) {
+    const uint64_t i = (uint64_t)leaf * 32 + lane;
+    int4 o = make_int4(0, 0, 0, 0), pb = make_int4(kEmptyLo, kEmptyLo, kEmptyHi, kEmptyHi);
+    const int4* rec = (const int4*)src.obj + 2 * i;
+    if (i < src.n) {
+        o = __ldg(rec);
+        pb = __ldg(rec + 1);
+    }
+    const int32_t x0 = rel32(pb.x, g.xc), y0 = rel32(pb.y, g.yc), x1 = rel32(pb.z, g.xc), y1 = rel32(pb.w, g.yc);
+    const int r0 = max(g.hh - ((g.R - y0) >> g.s), 0), r1 = min(((y1 + g.R) >> g.s) + g.hh, 2 * g.hh - 1);
+    const int clo = max(g.hw - ((g.R - x0) >> g.s), 0), chi = min(((x1 + g.R) >> g.s) + g.hw, 2 * g.hw - 1);
+    uint32_t mine = 0u;
+    if (i < src.n && r0 <= r1 && clo <= chi) mine = rows & (~0u << r0) & (~0u >> (31 - r1));
+    // from the first to the last open row
+    const int first = __ffs(mine) - 1, count = mine ? 32 - __clz(mine) - first : 0;
+    int sum = count;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int v = __shfl_up_sync(kFull, sum, d);
+        if (lane >= d) sum += v;
+    }
+    const int total = __shfl_sync(kFull, sum, 31);
+    if (total == 0) return;
+    const PieceRow own = piece_row(g, o, x0, y0, x1, y1, clo, chi);
+    const int start = sum - count;   // the lane's first pair
+    for (int base = 0; base < total; base += 32) {
+        const int j = base + lane;
+        // the last piece that starts at or before pair j (pieces without rows
+        // start where the next one does)
+        int k = 0;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1)
+            if (__shfl_sync(kFull, start, k + d) <= j) k += d;
+        const int r = __shfl_sync(kFull, first, k) + j - __shfl_sync(kFull, start, k);
+        PieceRow q;
+        q.mx = __shfl_sync(kFull, own.mx, k), q.my = __shfl_sync(kFull, own.my, k);
+        q.c0 = __shfl_sync(kFull, own.c0, k), q.E = __shfl_sync(kFull, own.E, k);
+        q.ta = __shfl_sync(kFull, own.ta, k), q.tb = __shfl_sync(kFull, own.tb, k);
+        q.at = __shfl_sync(kFull, own.at, k), q.span = __shfl_sync(kFull, own.span, k);
+        if (j < total) draw_row(bits, g, q, (const int4*)src.obj + 2 * ((uint64_t)leaf * 32 + k), r);
+        __syncwarp();
+    }
+}
+
+// ---- traversal ----------------------------------------------------------------
+
 // One frontier entry (its box [bx0, bx1] in x, rows: its open rows): a
 // depth-first descent of its subtree down to the points of its leaves.  Per
 // step the lanes hold 32 boxes -- the children of an inner node, or the points
@@ -256,8 +489,8 @@ __device__ __forceinline__ bool small_box(const Lattice& g, int32_t x0, int32_t 
 // and below it only the rows with such a sample matter.  (One drawing site and
 // one reach test for leaves and nodes keep the loop small for the instruction
 // cache.)
-template <bool kNarrowR, bool kProf>
-__device__ __forceinline__ void sweep_points(const Params& p, SweepSmem& sm, const Src& src, const Lattice& g,
+template <int kKind, bool kNarrowR, bool kProf>
+__device__ __forceinline__ void sweep_entry(const Params& p, SweepSmem<kKind>& sm, const Src& src, const Lattice& g,
                                              int level, uint32_t id, uint32_t rows, int32_t bx0, int32_t bx1,
                                              int lane, int warp) {
     if (level < 0 || level > kMaxLevels || id >= src.lvl_n[level]) {
@@ -274,9 +507,13 @@ __device__ __forceinline__ void sweep_points(const Params& p, SweepSmem& sm, con
     int32_t cx0 = 0, cy0 = 0, cx1 = 0, cy1 = 0;   // its child boxes
     long long t0 = 0;
     while (true) {
-        int32_t x0, y0, x1, y1;
-        bool draw;
-        if (lvl == 0) {
+        int32_t x0 = 0, y0 = 0, x1 = 0, y1 = 0;
+        bool draw = false;
+        if (lvl == 0 && kKind != HV_LAYER_POINTS) {
+            log_read(p, kLogLeaf, node, lane);
+            t0 = tick<kProf>();
+            draw_segments(p, src, sm.bits, g, node, rows, lane);
+        } else if (lvl == 0) {
             log_read(p, kLogLeaf, node, lane);
             t0 = tick<kProf>();
             const uint64_t i = (uint64_t)node * 32 + lane;
@@ -294,12 +531,14 @@ __device__ __forceinline__ void sweep_points(const Params& p, SweepSmem& sm, con
             draw = ax0 <= ax1;   // not a padding box
         }
         const bool valid = draw;
-        draw = draw && small_box(g, x0, y0, x1, y1);
-        const int c0 = g.hw - ((g.R - bx0) >> g.s);
-        if (((bx1 + g.R) >> g.s) + g.hw - c0 < 32 && __popc(rows) <= reach_rows) {
-            if (__any_sync(kFull, draw)) splat_window<kNarrowR>(sm.bits, g, x0, y0, x1, y1, c0, draw, rows, lane);
-        } else if (draw) {
-            splat<kNarrowR>(sm.bits, g, x0, y0, x1, y1, rows);
+        if constexpr (kKind == HV_LAYER_POINTS) {
+            draw = draw && small_box(g, x0, y0, x1, y1);
+            const int c0 = g.hw - ((g.R - bx0) >> g.s);
+            if (((bx1 + g.R) >> g.s) + g.hw - c0 < 32 && __popc(rows) <= reach_rows) {
+                if (__any_sync(kFull, draw)) splat_window<kNarrowR>(sm.bits, g, x0, y0, x1, y1, c0, draw, rows, lane);
+            } else if (draw) {
+                splat<kNarrowR>(sm.bits, g, x0, y0, x1, y1, rows);
+            }
         }
         __syncwarp();
         if (lvl == 0) {
@@ -365,8 +604,8 @@ __device__ __forceinline__ void sweep_points(const Params& p, SweepSmem& sm, con
 
 // Every frontier entry of the strip, taken by the warps in turn, and the side
 // tree (objects longer than the learned index's halo) as one more entry.
-template <bool kNarrowR, bool kProf>
-__device__ void sweep_pass(const Params& p, SweepSmem& sm, const Src& src, const Src& side, const TreeArg& st,
+template <int kKind, bool kNarrowR, bool kProf>
+__device__ void sweep_pass(const Params& p, SweepSmem<kKind>& sm, const Src& src, const Src& side, const TreeArg& st,
                            bool side_hit, const Lattice& g, int tid) {
     const int lane = tid & 31, warp = tid >> 5;
     const int f_count = sm.f_count, f_level = sm.f_level, fb = sm.f_buf;
@@ -385,8 +624,8 @@ __device__ void sweep_pass(const Params& p, SweepSmem& sm, const Src& src, const
         const uint32_t rows = open_rows(bits, sm.reach, g, x0, rel32(b.y, g.yc), x1, rel32(b.w, g.yc), lane);
         if (rows == 0) continue;
         const long long t0 = tick<kProf>();
-        sweep_points<kNarrowR, kProf>(p, sm, from_side ? side : src, g, from_side ? st.top : f_level,
-                                      from_side ? 0u : sm.fid[fb][e], rows, x0, x1, lane, warp);
+        sweep_entry<kKind, kNarrowR, kProf>(p, sm, from_side ? side : src, g, from_side ? st.top : f_level,
+                                            from_side ? 0u : sm.fid[fb][e], rows, x0, x1, lane, warp);
         prof_since<kProf>(sm, kPDescend, t0, lane);
     }
     prof_since<kProf>(sm, kPBlocksWarp, t_active, lane);
@@ -397,12 +636,19 @@ __device__ __forceinline__ uint32_t pixel_count(uint32_t top, uint32_t bottom, i
     return (uint32_t)(__popc((top >> (2 * q)) & 3u) + __popc((bottom >> (2 * q)) & 3u));
 }
 
-// Six CTAs per SM: 11.5 ms for 4,000 tiles of 100M points against 11.9 with
-// five and 12.6 with four (40 registers with a small spill; the dependent steps
-// of a row leave issue slots that more warps fill).
+// CTAs per SM.  Points: six, 11.5 ms for 4,000 tiles of 100M points against 11.9
+// with five and 12.6 with four (40 registers with a small spill; the dependent
+// steps of a row leave issue slots that more warps fill).  Segments: four, 24
+// tiles of 5M segments 68 us, 1,000 polygon tiles 12.0 ms, against 72 us and
+// 12.4 ms with five (4,000 line tiles 5.9 against 5.7 ms).
+template <int kKind>
+struct SweepTraits {
+    static constexpr int kPerSM = kKind == HV_LAYER_POINTS ? 6 : 4;
+};
+
 template <int kKind, bool kProf, bool kSplit>
-__global__ void __launch_bounds__(kThreads, kSweepPerSM) k_sweep(const Params p) {
-    __shared__ SweepSmem sm;
+__global__ void __launch_bounds__(kThreads, SweepTraits<kKind>::kPerSM) k_sweep(const Params p) {
+    __shared__ SweepSmem<kKind> sm;
     const int tid = threadIdx.x;
     const long long t_start = tick<kProf>();
     if constexpr (kProf) {
@@ -418,11 +664,28 @@ __global__ void __launch_bounds__(kThreads, kSweepPerSM) k_sweep(const Params p)
     const hv_tile_req q = p.reqs[tile];
     const bool ok = q.z <= 19 && q.x < (1u << q.z) && q.y < (1u << q.z) && (p.R_units >= 0 || (q.r16 >= 1 && q.r16 <= 1024));
     for (int k = tid; k < kSampleRows * kBitStride; k += kThreads) sm.bits[k] = 0u;
+    uint8_t* const out = p.out + (uint64_t)tile * p.tile_bytes;
+    const bool mask_mode = p.mode == HV_MODE_MASK;
+    if constexpr (kKind == HV_LAYER_POLYGONS) {
+        decode_fill(p, out, sm.res, strip, col0, cols, tid, p.fill_aa && !mask_mode);
+        __syncthreads();
+        // a MASK pixel whose centre is already filled is decided (unless a
+        // pattern may leave it transparent)
+        if (mask_mode && p.pat_w == 0) {
+            const int wpr = cols / 32, wsh = __ffs(wpr) - 1;
+            if (tid < rows * wpr) {
+                const int jl = tid >> wsh, w = tid & (wpr - 1);
+                uint32_t word = 0u;
+                for (int b = 0; b < 32; b++)
+                    if (sm.res[jl * kTile + col0 + 32 * w + b] >> kResFillShift) word |= 1u << b;
+                sm.bits[jl * kBitStride + w] = word;
+            }
+        }
+    }
     if (!ok && tid == 0 && sp == 0) atomicOr(p.status, 1u);
     if (tid == 0) sm.next_entry = 0;
     __syncthreads();
     if (tid == 0) prof_since<kProf>(sm, kPPrologue, t_start, 0);
-    const bool mask_mode = p.mode == HV_MODE_MASK;
     if (ok) {
         const int z = q.z, L = 23 - z;
         const int32_t ps = 1 << L;
@@ -458,20 +721,34 @@ __global__ void __launch_bounds__(kThreads, kSweepPerSM) k_sweep(const Params p)
         if (sm.f_count > 0 || side_hit) {
             const long long t_pass = tick<kProf>();
             if (tid == 0) prof_add<kProf>(sm, kPBlocks, (unsigned long long)(rows / kBH) * (cols / kBW), 0);
-            Src src{p.obj, nullptr, p.tree.n_obj, p.tree.nodes, sm.lvl_base[0], sm.lvl_n[0], nullptr, nullptr};
-            Src side{p.side_obj, p.side_ids, p.side.n_obj, p.side.nodes, sm.lvl_base[1], sm.lvl_n[1], nullptr, nullptr};
-            if (g.narrow)
-                sweep_pass<true, kProf>(p, sm, src, side, p.side, side_hit, g, tid);
+            Src src{p.obj, nullptr, p.tree.n_obj, p.tree.nodes, sm.lvl_base[0], sm.lvl_n[0]};
+            Src side{p.side_obj, p.side_ids, p.side.n_obj, p.side.nodes, sm.lvl_base[1], sm.lvl_n[1]};
+            // (segments draw the same way at every radius)
+            if (kKind != HV_LAYER_POINTS || g.narrow)
+                sweep_pass<kKind, true, kProf>(p, sm, src, side, p.side, side_hit, g, tid);
             else
-                sweep_pass<false, kProf>(p, sm, src, side, p.side, side_hit, g, tid);
+                sweep_pass<kKind, false, kProf>(p, sm, src, side, p.side, side_hit, g, tid);
             __syncthreads();
             if (tid == 0) prof_since<kProf>(sm, kPBlocksCta, t_pass, 0);
         }
     }
     // ---- encode the strip (Sec. 4.1 Render Tiles) ----
     const long long t_enc = tick<kProf>();
-    uint8_t* out = p.out + (uint64_t)tile * p.tile_bytes;
-    if (mask_mode) {
+    if constexpr (kKind == HV_LAYER_POLYGONS) {
+        // the covered samples join the fill results, a byte per pixel
+        for (int k = tid; k < rows * cols; k += kThreads) {
+            const int jl = k / cols, c = k % cols;
+            uint32_t v;
+            if (mask_mode)
+                v = (sm.bits[jl * kBitStride + (c >> 5)] >> (c & 31)) & 1u ? kResCentre : 0u;
+            else
+                v = ((sm.bits[2 * jl * kBitStride + (c >> 4)] >> (2 * (c & 15))) & 3u) |
+                    (((sm.bits[(2 * jl + 1) * kBitStride + (c >> 4)] >> (2 * (c & 15))) & 3u) << 2);
+            sm.res[jl * kTile + col0 + c] |= (uint8_t)v;
+        }
+        __syncthreads();
+        encode_polygons(p, sm.res, out, strip, col0, cols, tile, tid);
+    } else if (mask_mode) {
         // the sample bits are the output: word w of row j = pixels 32w .. 32w+31
         const int wpr = cols / 32, wsh = __ffs(wpr) - 1;
         if (tid < rows * wpr) {

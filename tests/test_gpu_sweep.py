@@ -1,9 +1,11 @@
-"""Points drawn row by row over a strip's sample lattice: layers and requests
-at the edges of that path, byte-equal to the oracle -- leaves with 1 to 33
-points, points on strip, part and grid borders, samples at exactly R and R +- 1
-units, rows on both sides of the 32-bit radius, reaches wider than the 32-column
-window, crowded and sparse leaves, every zoom class, mode, strip height and
-column part."""
+"""Points and segments drawn row by row over a strip's sample lattice: layers
+and requests at the edges of that path, byte-equal to the oracle in every mode,
+strip height and column part -- points: leaves with 1 to 33 points, strip, part
+and grid borders, samples at exactly R and R +- 1 units, rows on both sides of
+the 32-bit radius, reaches wider than the 32-column window, crowded and sparse
+leaves; segments: level, upright, almost level and slanted ones, zero lengths,
+ends far outside the strip and the grid's whole width, leaves with few and
+with many (piece, row) pairs."""
 import numpy as np
 import pytest
 
@@ -31,15 +33,18 @@ def ctx():
     hv.hv_destroy(c)
 
 
-def _check(ctx, pts, reqs, radius=None, batches=(1, 3, 200)):
+def _check(ctx, pts, reqs, radius=None, batches=(1, 3, 200), lines=False):
     pts = np.ascontiguousarray(pts, dtype=np.int32)
     reqs = np.array(reqs, dtype=np.uint32)
-    L = hv.hv_layer_load_points(ctx, pts)
+    off = np.arange(0, len(pts) + 1, 2, dtype=np.uint64)   # lines: a segment per vertex pair
+    L = hv.hv_layer_load_linestrings(ctx, pts, off) if lines else hv.hv_layer_load_points(ctx, pts)
     hv.hv_layer_build_index(L, hv.HV_INDEX_RTREE | hv.HV_INDEX_LEARNED)
     s = hv.make_style(STYLE_T[:3], STYLE_T[4:7])
     try:
         for mode in MODES:
-            ref = oracle_par.render(lambda r: oracle.render_points(pts, r, mode, STYLE_T, R_units=radius), reqs)
+            ref = oracle_par.render(
+                lambda r: oracle.render_lines(pts, off, r, mode, STYLE_T, R_units=radius) if lines
+                else oracle.render_points(pts, r, mode, STYLE_T, R_units=radius), reqs)
             for index in (hv.HV_INDEX_RTREE, hv.HV_INDEX_LEARNED):
                 for per in batches:      # column parts, 4-row strips, full strips (requests repeated)
                     rows = np.resize(np.arange(len(reqs)), max(per, len(reqs))) if per > len(reqs) else np.arange(len(reqs))
@@ -101,3 +106,32 @@ def test_ground_radii(ctx, radius):
     pts = rng.integers(-2 ** 24, 2 ** 24, (3000, 2))
     _check(ctx, pts, [[5, 16, 16, 1], [8, 128, 127, 1], [13, 4096, 4095, 1], [19, 262144, 262143, 1], [0, 0, 0, 1]],
            radius=radius, batches=(1, 150))
+
+
+def _fan(rng, n, spread, size):
+    """n segments (2n, 2): slopes from level to upright with near misses of
+    both, lengths over three decades, some of length 0, swapped ends."""
+    a = rng.integers(-spread, spread, (n, 2)).astype(np.float64)
+    th = np.choose(rng.integers(0, 5, n), [np.zeros(n), np.full(n, np.pi / 2), rng.uniform(0, 2 * np.pi, n),
+                                           10.0 ** rng.uniform(-7, -1, n), np.pi / 2 - 10.0 ** rng.uniform(-7, -1, n)])
+    d = size * 10.0 ** rng.uniform(-3, 0, n) * (rng.random(n) > 0.05)
+    b = a + np.stack([d * np.cos(th), d * np.sin(th)], 1)
+    flip = (rng.random(n) < 0.5)[:, None]
+    seg = np.stack([np.where(flip, b, a), np.where(flip, a, b)], 1)
+    return np.clip(np.round(seg), -HALF, HALF - 1).astype(np.int32).reshape(-1, 2)
+
+
+@pytest.mark.parametrize("spread, size", [(2 ** 12, 2 ** 11), (2 ** 18, 2 ** 20), (2 ** 24, 2 ** 29), (2 ** 29, 2 ** 30)])
+def test_segments_of_every_slope(ctx, spread, size):
+    rng = np.random.default_rng(spread)
+    seg = _fan(rng, 1500, spread, size)
+    zs = [z for z in (0, 3, 9, 13, 19) if (1 << (31 - z)) < 4096 * spread]
+    _check(ctx, seg, [[z, (1 << z) // 2 - k, (1 << z) // 2 - (1 - k), r] for z in zs for k in (0, 1) if z
+                      for r in (1, 8, 40)] + [[0, 0, 0, 16], [2, 1, 2, 1024]], lines=True, batches=(1, 120))
+
+
+@pytest.mark.parametrize("radius", [0, 7, 100_003, 1 << 27])
+def test_segments_at_ground_radii(ctx, radius):
+    seg = _fan(np.random.default_rng(5), 400, 2 ** 22, 2 ** 23)
+    _check(ctx, seg, [[7, 64, 63, 1], [11, 1024, 1024, 1], [16, 32768, 32767, 1]], radius=radius, lines=True,
+           batches=(1, 150))
