@@ -15,16 +15,9 @@
 // column parts, one CTA each).  The CTA first culls the R-tree (or, with the
 // learned index, the subtrees of the key ranges the model finds) against the
 // strip's box expanded by R, breadth first, into a frontier of at most kFCap
-// nodes in shared memory (the deepest level that fits).  Points are then
-// drawn object by object into a bit per sample of the strip (hv_sweep.cuh).
-// For segments and polygons the frontier is binned by 8-pixel block column,
-// and each warp takes 8 x 4 pixel blocks (one pixel per lane, up to four
-// samples per lane): it tests its column's frontier entries against its
-// still-undecided samples, descends the intersecting subtrees depth first (a
-// ballot over the 32 child boxes decides which children to visit), evaluates
-// the exact predicate on the records of each visited leaf, and stops as soon
-// as every sample of the block is decided.  Results go to a per-pixel byte
-// array in shared memory; the epilogue encodes the strip (MASK bits,
+// nodes in shared memory (the deepest level that fits).  Its warps then take
+// the frontier's subtrees in turn and draw their objects into a bit per sample
+// of the strip (hv_sweep.cuh); the epilogue encodes the bits (MASK bits,
 // COVERAGE bytes or RGBA) with coalesced 16-byte stores.
 #include "hv_device.cuh"
 #include "hv_internal.h"
@@ -37,10 +30,8 @@ namespace {
 constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
 constexpr int kStripRows = 16;   // the largest strip; a launch picks 4, 8 or 16 rows
-constexpr int kBW = 8, kBH = 4;
-constexpr int kBlocksX = kTile / kBW;
+constexpr int kBW = 8, kBH = 4;   // the pixel blocks that the phase profile counts
 constexpr int kFCap = 512;
-constexpr int kBucketCap = 2048;   // keeps the static shared memory under 48 KiB
 constexpr int kCullCells = 64;     // learned cull: at most this many Hilbert cells per strip
 constexpr int kCullSub = kThreads / kCullCells;   // threads per cell
 static_assert(kCullSub >= 2 && kCullSub <= 32 && (kCullSub & (kCullSub - 1)) == 0, "cell threads within a warp");
@@ -68,7 +59,6 @@ struct Params {
     int strips;                 // strips per tile (256 / rows)
     int cols;                   // pixel columns per CTA: 256, or 128 / 64 for batches too small to fill the GPU
     int parts;                  // CTAs per strip (256 / cols)
-    int col_shift;              // log2(cols / 8): block columns per CTA as a shift
     const uint32_t* n_dev;      // if set, the batch size is min(*n_dev, n) (graph launches)
     int mode;
     int kind;
@@ -127,10 +117,6 @@ __device__ __forceinline__ long long tick() {
     return 0;
 }
 
-// outcome of a leaf visit (counted by the phase profile): no record in reach
-// of an undecided sample, records tested without deciding one, a sample decided
-constexpr uint32_t kVisitEmpty = 0, kVisitTested = 1, kVisitDecided = 2;
-
 // kinds of logged reads
 constexpr uint32_t kLogNode = 0, kLogLeaf = 1, kLogPolyNode = 2, kLogPolyLeaf = 3, kLogPoly = 4;
 
@@ -151,10 +137,8 @@ __device__ __noinline__ void check_failed(const Params& p, uint32_t code, uint64
     atomicOr(p.status, 2u);
 }
 
-// The frontier is built in two buffers that the cull alternates; the pass
-// over the blocks reads only the final one (f_buf), and the other serves the
-// warps as scratch for segment leaves (Src::seg_scratch, pair_scratch) until
-// the barrier that ends the pass.
+// The frontier is built in two buffers that the cull alternates; the sweep
+// reads the final one (f_buf).
 struct Front {
     int4 fbox[2][kFCap];
     uint32_t fid[2][kFCap];
@@ -163,20 +147,6 @@ struct Front {
     int f_count, f_level, f_buf, next_count;
     int lvl_count[kMaxLevels + 1];
     unsigned long long prof[kPN];   // phase profile of the CTA (kProf only)
-};
-
-struct Smem : Front {
-    uint8_t res[kStripRows * kTile];
-    uint32_t stk_node[kWarps][kMaxLevels + 1];
-    uint32_t stk_mask[kWarps][kMaxLevels + 1];
-    uint32_t lanemask[kWarps][kMaxLevels + 1][32];
-    // the frontier binned by 8-pixel block column: bucket c lists the entries
-    // that can reach blocks of column c
-    uint16_t bucket[kBucketCap];
-    int bucket_off[kBlocksX + 1];
-    int bucket_cur[kBlocksX];
-    int binned;
-    int next_block;
 };
 
 // Add the cycles since t0 (or a count) to a phase counter of the CTA (one
@@ -202,229 +172,6 @@ struct Src {
     const int32_t* const* lvl;   // lvl[l] = first node of level l
     const uint32_t* lvl_n;       // lvl_n[l] = nodes of level l
 };
-
-// Per-lane state of one 8 x 4 pixel block (lane l = pixel (l & 7, l >> 3)).
-// Sample k of a lane sits at (cx -+ off, cy -+ off): bit 0 of k picks +x,
-// bit 1 picks +y.  MASK mode and the fill use one sample, the centre.
-struct Lane {
-    int32_t cx, cy;        // pixel centre
-    int32_t off;           // super-sample offset (0 in MASK mode and for fill)
-    int32_t ext;           // reach of a lane's samples: R + off (Chebyshev)
-    int64_t R2;
-    uint32_t und;          // this lane's undecided samples (bit k: sample k)
-    uint32_t Uk[4];        // warp-uniform: lanes whose sample k is undecided
-    uint32_t U;            // warp-uniform: lanes with an undecided sample
-    int nk;                // samples per lane (1 or 4)
-    int32_t bx0, by0;      // warp-uniform: centre of the block's first pixel
-    int L;                 // warp-uniform: log2 of the pixel size
-};
-
-// Lanes of the block that have a sample within Chebyshev distance `ext` of
-// the box [x0, x1] x [y0, y1]: a pixel column c qualifies when its centre
-// lies in [x0 - ext, x1 + ext], i.e. ceil((x0-ext-bx0)/ps) <= c <=
-// floor((x1+ext-bx0)/ps), and likewise for rows.  A necessary condition for
-// any object inside the box to cover any of that lane's samples.
-__device__ __forceinline__ uint32_t rect_lanes(const Lane& s, int32_t x0, int32_t y0, int32_t x1,
-                                               int32_t y1) {
-    // empty boxes and padding records lie outside the grid
-    if (x0 > x1 || y0 > y1 || x0 < -kGridHalf || y0 < -kGridHalf) return 0u;
-    // differences from the block origin fit 32 bits once clamped to +-2^30
-    // (the reach is below 2^30, so farther boxes stay out of range)
-    const int32_t ax = max(x0 - s.bx0, -kGridHalf) - s.ext, bx = min(x1 - s.bx0, kGridHalf) + s.ext;
-    const int32_t ay = max(y0 - s.by0, -kGridHalf) - s.ext, by = min(y1 - s.by0, kGridHalf) + s.ext;
-    const int32_t c0 = max(-((-ax) >> s.L), 0), c1 = min(bx >> s.L, 7);
-    const int32_t r0 = max(-((-ay) >> s.L), 0), r1 = min(by >> s.L, 3);
-    if (c0 > c1 || r0 > r1) return 0u;
-    uint32_t col = (0xFFu << c0) & (0xFFu >> (7 - c1));
-    uint32_t rows = (0x01010101u << (8 * r0)) & (0x01010101u >> (8 * (3 - r1)));
-    return col * rows;
-}
-
-// Pixels of the block whose centre the edge e crosses strictly to the right
-// (Algorithm 2's ray test, half-open straddle in y): per pixel row the
-// orientation num(c) = dx (y - ly) - (x_c - lx) dy of the edge ordered by y
-// falls as the column c grows, so the crossed columns are a prefix 0..t-1,
-// t found by a three-step binary search with exact 64-bit products.
-// (ox, oy) offsets the samples from the pixel centres (the anti-aliased
-// fill's super-samples); the column search is the same.
-__device__ __forceinline__ uint32_t crossing_columns(int4 e, const Lane& s, int32_t ox = 0, int32_t oy = 0) {
-    int32_t lx = e.x, ly = e.y, hx = e.z, hy = e.w;
-    if (ly > hy) {
-        lx = e.z; ly = e.w; hx = e.x; hy = e.y;
-    }
-    if (ly == hy) return 0u;   // a level edge straddles no scanline
-    const int32_t ex = hx - lx, ey = hy - ly;
-    uint32_t m = 0u;
-#pragma unroll
-    for (int r = 0; r < kBH; r++) {
-        const int32_t y = s.by0 + (r << s.L) + oy;
-        if (y < ly || y >= hy) continue;
-        const int64_t n0 = (int64_t)ex * (y - ly) - ((int64_t)s.bx0 + ox - lx) * ey;
-        // column c is crossed iff n0 > c ps ey
-        int t = n0 > (int64_t)(3 << s.L) * ey ? 4 : 0;
-        if (n0 > (int64_t)((t + 1) << s.L) * ey) t += 2;
-        if (n0 > (int64_t)(t << s.L) * ey) t += 1;
-        if (t == 7 && n0 > (int64_t)(7 << s.L) * ey) t = 8;
-        m |= ((1u << t) - 1u) << (8 * r);
-    }
-    return m;
-}
-
-// Polygon boxes: a leaf holds 32 polygon boxes; for each box that contains an
-// unfilled pixel centre, count that polygon's own edges crossing the ray.
-struct FillLeaf {
-    __device__ static uint32_t visit(const Params& p, const Src& src, uint32_t leaf, Lane& s, int lane) {
-        if ((uint64_t)leaf * 32 >= src.n) {
-            if (lane == 0) check_failed(p, 4, leaf);
-            return kVisitEmpty;
-        }
-        uint64_t i = (uint64_t)leaf * 32 + lane;
-        log_read(p, kLogPolyLeaf, leaf, lane);
-        int4 b = make_int4(kEmptyLo, kEmptyLo, kEmptyHi, kEmptyHi);
-        uint32_t id = 0;
-        if (i < src.n) {
-            b = __ldg((const int4*)src.obj + i);
-            id = __ldg(src.ids + i);
-        }
-        uint32_t pm = rect_lanes(s, b.x, b.y, b.z, b.w);
-        uint32_t m = __ballot_sync(kFull, (pm & s.U) != 0);
-        uint32_t outcome = m ? kVisitTested : kVisitEmpty;
-        const uint32_t U_before = s.U;
-        while (m) {
-            int k = __ffs(m) - 1;
-            m &= m - 1;
-            int32_t bx0 = __shfl_sync(kFull, b.x, k), by0 = __shfl_sync(kFull, b.y, k);
-            int32_t bx1 = __shfl_sync(kFull, b.z, k), by1 = __shfl_sync(kFull, b.w, k);
-            uint32_t pid = __shfl_sync(kFull, id, k);
-            // a sample of the lane (the centre, or a super-sample within off
-            // of it) may lie in the box
-            bool active = s.und && s.cx + s.off >= bx0 && s.cx - s.off <= bx1 && s.cy + s.off >= by0 &&
-                          s.cy - s.off <= by1;
-            if (__ballot_sync(kFull, active) == 0) continue;
-            log_read(p, kLogPoly, pid, lane);
-            if (pid >= p.n_poly) {
-                if (lane == 0) check_failed(p, 5, pid);
-                continue;
-            }
-            uint64_t e0 = __ldg(p.poly_edge_off + pid), e1 = __ldg(p.poly_edge_off + pid + 1);
-            if (e0 > e1 || e1 > p.n_edges) {
-                if (lane == 0) check_failed(p, 6, ((uint64_t)pid << 24) | (e1 & 0xffffff));
-                continue;
-            }
-            // each lane takes an edge; the crossed pixels of all the edges,
-            // XOR-reduced, are every pixel's parity at once (per sample)
-            uint32_t inside = 0u;
-            if (s.nk == 1) {
-                uint32_t par = 0u;
-                for (uint64_t base = e0; base < e1; base += 32) {
-                    uint32_t cm = 0u;
-                    if (base + lane < e1) cm = crossing_columns(__ldg(p.poly_edges + base + lane), s);
-                    par ^= __reduce_xor_sync(kFull, cm);
-                }
-                inside = (par >> lane) & 1u;
-            } else {
-                // super-sample k sits at -+off in x (bit 0) and y (bit 1)
-                uint32_t par[4] = {0u, 0u, 0u, 0u};
-                for (uint64_t base = e0; base < e1; base += 32) {
-                    int4 e = make_int4(0, 0, 0, 0);   // a level edge crosses nothing
-                    if (base + lane < e1) e = __ldg(p.poly_edges + base + lane);
-#pragma unroll
-                    for (int k = 0; k < 4; k++)
-                        par[k] ^= __reduce_xor_sync(kFull, crossing_columns(e, s, (k & 1) ? s.off : -s.off,
-                                                                            (k & 2) ? s.off : -s.off));
-                }
-#pragma unroll
-                for (int k = 0; k < 4; k++) inside |= ((par[k] >> lane) & 1u) << k;
-            }
-            if (active) s.und &= ~inside;
-            uint32_t U2 = __ballot_sync(kFull, s.und != 0);
-            if (U2 != s.U) {
-                s.U = U2;
-                s.Uk[0] = U2;
-                m &= __ballot_sync(kFull, (pm & U2) != 0);
-            }
-        }
-        return s.U != U_before ? kVisitDecided : outcome;
-    }
-};
-
-// Child boxes of one inner node: lane c computes the lanes child c can
-// reach, keeps it in `lm`, and the ballot selects the children to visit.
-template <class V>
-__device__ __forceinline__ uint32_t child_hits(const Params& p, const Src& src,
-                                               const int32_t* base, Lane& s, int lane, uint32_t* lm) {
-    if (p.log != nullptr)
-        log_read(p, kLogPolyNode, (uint64_t)(base - src.nodes) >> 7, lane);
-    int32_t x0 = __ldg(base + lane), y0 = __ldg(base + 32 + lane);
-    int32_t x1 = __ldg(base + 64 + lane), y1 = __ldg(base + 96 + lane);
-    uint32_t cm = rect_lanes(s, x0, y0, x1, y1);
-    lm[lane] = cm;
-    return __ballot_sync(kFull, (cm & s.U) != 0u);
-}
-
-// Depth-first descent from node `node` at level `level` (0: a leaf, which the
-// one visit below takes too, so that the leaf code exists once in the kernel).
-// The stack keeps, per level, the node whose children are being visited, the
-// children still to visit, and each child's lane reach (re-tested against the
-// shrinking undecided set before every visit).
-template <class V, bool kProf>
-__device__ void descend(const Params& p, Smem& sm, const Src& src, int level, uint32_t node, Lane& s,
-                        int lane, int warp) {
-    uint32_t* stk_node = sm.stk_node[warp];
-    uint32_t* stk_mask = sm.stk_mask[warp];
-    int lvl = level;
-    if (level < 0 || level > kMaxLevels || (level > 0 && node >= src.lvl_n[level])) {
-        if (lane == 0) check_failed(p, 2, ((uint64_t)level << 40) | node);
-        return;
-    }
-    uint32_t leaf = node;
-    if (level > 0) {
-        uint32_t m0 = child_hits<V>(p, src, src.lvl[lvl] + (uint64_t)node * 128, s, lane, sm.lanemask[warp][lvl]);
-        prof_add<kProf>(sm, kPNodeVisits, 1, lane);
-        if (s.U == 0) return;
-        stk_node[lvl] = node;
-        stk_mask[lvl] = m0;
-        __syncwarp();
-    }
-    while (true) {
-        if (lvl > 0) {
-            uint32_t m = stk_mask[lvl];
-            m = __ballot_sync(kFull, ((m >> lane) & 1u) && (sm.lanemask[warp][lvl][lane] & s.U));
-            if (m == 0) {
-                if (lvl == level) break;
-                lvl++;
-                continue;
-            }
-            int c = __ffs(m) - 1;
-            uint32_t child = stk_node[lvl] * 32u + (uint32_t)c;
-            __syncwarp();
-            stk_mask[lvl] = m & (m - 1);
-            __syncwarp();
-            if (lvl > 1) {
-                if (child >= src.lvl_n[lvl - 1]) {
-                    if (lane == 0) check_failed(p, 3, ((uint64_t)(lvl - 1) << 40) | child);
-                    continue;
-                }
-                lvl--;
-                uint32_t hm = child_hits<V>(p, src, src.lvl[lvl] + (uint64_t)child * 128, s, lane,
-                                            sm.lanemask[warp][lvl]);
-                prof_add<kProf>(sm, kPNodeVisits, 1, lane);
-                if (s.U == 0) return;
-                stk_node[lvl] = child;
-                stk_mask[lvl] = hm;
-                __syncwarp();
-                continue;
-            }
-            leaf = child;
-        }
-        const long long t0 = tick<kProf>();
-        const uint32_t how = V::visit(p, src, leaf, s, lane);
-        prof_since<kProf>(sm, kPLeaf, t0, lane);
-        prof_add<kProf>(sm, kPLeafVisits, 1, lane);
-        prof_add<kProf>(sm, how == kVisitEmpty ? kPLeafEmpty : kPLeafDecided, how != kVisitTested, lane);
-        if (s.U == 0 || level == 0) return;
-    }
-}
 
 // Level bases of a tree into shared memory slot `slot` (0: the tree being
 // traversed, 1: its side tree).
@@ -632,195 +379,6 @@ __device__ void learned_cull(const Params& p, const TreeArg& t, const LModel& m,
     refine(p, t, false, sm, bx0, by0, bx1, by1, tid);
 }
 
-// Column range [c0, c1] of 8-pixel block columns an entry box can reach: a
-// column's samples span x in [X0 + 8c ps + ps/2 - off, X0 + (8c+7) ps + ps/2
-// + off], widened by R.
-__device__ __forceinline__ void entry_columns(int4 b, int32_t X0, int L, int32_t reach, int* c0, int* c1) {
-    const int64_t base = (int64_t)X0 + ((int64_t)1 << L >> 1);
-    int64_t lo = (int64_t)b.x - reach - base - 7 * ((int64_t)1 << L);
-    int64_t hi = (int64_t)b.z + reach - base;
-    int64_t a = -((-lo) >> (L + 3)), e = hi >> (L + 3);
-    *c0 = (int)(a < 0 ? 0 : (a > kBlocksX ? kBlocksX : a));
-    *c1 = (int)(e > kBlocksX - 1 ? kBlocksX - 1 : (e < -1 ? -1 : e));
-}
-
-// Bin the frontier by block column (falls back to the whole frontier when
-// the lists would overflow).
-__device__ void bin_frontier(Smem& sm, int32_t X0, int L, int32_t reach, int tid) {
-    const int f_count = sm.f_count, fb = sm.f_buf;
-    if (tid < kBlocksX) {
-        sm.bucket_off[tid] = 0;
-        sm.bucket_cur[tid] = 0;
-    }
-    __syncthreads();
-    for (int e = tid; e < f_count; e += kThreads) {
-        int c0, c1;
-        entry_columns(sm.fbox[fb][e], X0, L, reach, &c0, &c1);
-        for (int c = c0; c <= c1; c++) atomicAdd(&sm.bucket_off[c], 1);
-    }
-    __syncthreads();
-    if (tid == 0) {
-        int sum = 0;
-        for (int c = 0; c < kBlocksX; c++) {
-            int n = sm.bucket_off[c];
-            sm.bucket_off[c] = sum;
-            sum += n;
-        }
-        sm.bucket_off[kBlocksX] = sum;
-        sm.binned = sum <= kBucketCap;
-    }
-    __syncthreads();
-    if (sm.binned) {
-        for (int e = tid; e < f_count; e += kThreads) {
-            int c0, c1;
-            entry_columns(sm.fbox[fb][e], X0, L, reach, &c0, &c1);
-            for (int c = c0; c <= c1; c++) {
-                int pos = sm.bucket_off[c] + atomicAdd(&sm.bucket_cur[c], 1);
-                if (pos < sm.bucket_off[c + 1]) sm.bucket[pos] = (uint16_t)e;
-            }
-        }
-    }
-    __syncthreads();
-}
-
-// Process every pixel block of the strip: against the culled frontier (R-tree)
-// or through the learned lookup.
-template <class V, bool kProf>
-__device__ void blocks_pass(const Params& p, Smem& sm, const Src& src, const Src& side, int side_top, int32_t X0,
-                            int32_t Y0, int strip, int col0, int col_shift, int z, int32_t R, bool mask_mode,
-                            int tid) {
-    int lane = tid & 31, warp = tid >> 5;
-    const long long t_active = tick<kProf>();
-    const int L = 23 - z;
-    const int32_t ps = 1 << L;
-    const int f_count = sm.f_count, f_level = sm.f_level, fb = sm.f_buf;
-    while (true) {
-        int blk = 0;
-        if (lane == 0) blk = atomicAdd(&sm.next_block, 1);
-        blk = __shfl_sync(kFull, blk, 0);
-        // the CTA's blocks: 2^col_shift block columns from col0, rows / 4 block rows
-        if (blk >= (p.rows / kBH) << col_shift) break;
-        prof_add<kProf>(sm, kPBlocks, 1, lane);
-        int bx = col0 / kBW + (blk & ((1 << col_shift) - 1)), by = blk >> col_shift;
-        int i = bx * kBW + (lane & 7);
-        int jl = by * kBH + (lane >> 3);
-        int j = strip * p.rows + jl;
-        Lane s;
-        s.L = L;
-        s.cx = X0 + i * ps + (ps >> 1);
-        s.cy = Y0 + j * ps + (ps >> 1);
-        s.bx0 = X0 + (bx * kBW) * ps + (ps >> 1);
-        s.by0 = Y0 + (strip * p.rows + by * kBH) * ps + (ps >> 1);
-        s.R2 = (int64_t)R * R;
-        const bool centre_only = mask_mode || !p.fill_aa;
-        if (centre_only) {
-            s.off = 0;
-            s.und = 1u;
-            s.nk = 1;
-        } else {
-            s.off = ps >> 2;
-            s.und = 15u;
-            s.nk = 4;
-        }
-        s.ext = s.off;
-        s.U = kFull;
-        for (int k = 0; k < 4; k++) s.Uk[k] = k < s.nk ? kFull : 0u;
-        uint32_t und0 = s.und;
-        {
-            // this block's column list, or the whole frontier
-            const bool binned = sm.binned;
-            int lbeg = binned ? sm.bucket_off[bx] : 0;
-            int lcnt = binned ? sm.bucket_off[bx + 1] - lbeg : f_count;
-            if (binned && (lbeg < 0 || lcnt < 0 || lbeg + lcnt > kBucketCap)) {
-                if (lane == 0) check_failed(p, 7, ((uint64_t)bx << 32) | (uint32_t)lbeg);
-                lbeg = 0;
-                lcnt = 0;
-            }
-            for (int c0 = 0; c0 < lcnt && s.U; c0 += 32) {
-                int e = -1;
-                uint32_t cm = 0;
-                int4 fbx = make_int4(kEmptyLo, kEmptyLo, kEmptyHi, kEmptyHi);
-                if (c0 + lane < lcnt) {
-                    e = binned ? (int)sm.bucket[lbeg + c0 + lane] : c0 + lane;
-                    if (e >= f_count) {
-                        check_failed(p, 1, ((uint64_t)bx << 32) | (uint32_t)e);
-                        e = -1;
-                    } else {
-                        fbx = sm.fbox[fb][e];
-                        cm = rect_lanes(s, fbx.x, fbx.y, fbx.z, fbx.w);
-                    }
-                }
-                uint32_t mm = __ballot_sync(kFull, (cm & s.U) != 0u);
-                prof_add<kProf>(sm, kPFrontierEntries, (unsigned long long)min(32, lcnt - c0), lane);
-                while (mm) {
-                    int k = __ffs(mm) - 1;
-                    mm &= mm - 1;
-                    const int ek = __shfl_sync(kFull, e, k);
-                    uint32_t id = sm.fid[fb][ek];
-                    const long long t0 = tick<kProf>();
-                    descend<V, kProf>(p, sm, src, f_level, id, s, lane, warp);
-                    // everything below the frontier (leaves included)
-                    prof_since<kProf>(sm, kPDescend, t0, lane);
-                    // drop frontier entries that no longer reach an undecided lane
-                    mm &= __ballot_sync(kFull, ((mm >> lane) & 1u) && (cm & s.U) != 0u);
-                }
-            }
-            // objects longer than the learned index's halo live in a side tree
-            if (side_top > 0 && s.U) {
-                const long long t0 = tick<kProf>();
-                descend<V, kProf>(p, sm, side, side_top, 0, s, lane, warp);
-                prof_since<kProf>(sm, kPDescend, t0, lane);
-            }
-        }
-        uint32_t covered = und0 & ~s.und;
-        uint8_t r = sm.res[jl * kTile + i];
-        // the centre (1), or the number of super-samples inside (0..4)
-        if (covered) r |= (s.nk == 1 ? 1u : (uint32_t)__popc(covered)) << kResFillShift;
-        sm.res[jl * kTile + i] = r;
-    }
-    prof_since<kProf>(sm, kPBlocksWarp, t_active, lane);
-}
-
-// One stage (Algorithm 1 over points / segments / edges, or Algorithm 2 over
-// polygon boxes) for the strip: cull through the R-tree or the learned
-// index, then every block.
-template <class V, bool kProf>
-__device__ void stage(const Params& p, Smem& sm, const TreeArg& t, const void* obj, const uint32_t* ids,
-                      const TreeArg& st, const void* sobj, const uint32_t* sids, const LModel* m, int32_t halo,
-                      int32_t X0, int32_t Y0, int strip, int col0, int col_shift, int z, int32_t R, bool mask_mode,
-                      int32_t bx0, int32_t by0, int32_t bx1, int32_t by1, int tid) {
-    const long long t_cull = tick<kProf>();
-    set_levels(sm, 0, t, tid);
-    set_levels(sm, 1, st, tid);
-    if (tid == 0) sm.next_block = 0;
-    __syncthreads();
-    if (m == nullptr)
-        cull(p, t, true, sm, bx0, by0, bx1, by1, tid);
-    else
-        learned_cull(p, t, *m, halo, sm, bx0, by0, bx1, by1, tid);
-    if (tid == 0) prof_since<kProf>(sm, kPCull, t_cull, 0);
-    int4 sb = st.root_box;
-    bool side_hit = st.top > 0 && sb.x <= bx1 && sb.z >= bx0 && sb.y <= by1 && sb.w >= by0;
-    if (sm.f_count > 0 || side_hit) {
-        // the column lists are rebuilt for every pass, also for an empty
-        // frontier (a strip reached only by the side tree), so that the
-        // blocks never read the lists of an earlier stage
-        const bool sub = !mask_mode && p.fill_aa;   // super-samples
-        const int32_t off = sub ? ((1 << (23 - z)) >> 2) : 0;
-        const long long t_bin = tick<kProf>();
-        bin_frontier(sm, X0, 23 - z, off, tid);
-        if (tid == 0) prof_since<kProf>(sm, kPBin, t_bin, 0);
-        const long long t_blocks = tick<kProf>();
-        Src src{obj, ids, t.n_obj, t.nodes, sm.lvl_base[0], sm.lvl_n[0]};
-        Src side{sobj, sids, st.n_obj, st.nodes, sm.lvl_base[1], sm.lvl_n[1]};
-        blocks_pass<V, kProf>(p, sm, src, side, side_hit ? st.top : 0, X0, Y0, strip, col0, col_shift, z, R, mask_mode,
-                              tid);
-        __syncthreads();
-        if (tid == 0) prof_since<kProf>(sm, kPBlocksCta, t_blocks, 0);
-    }
-    __syncthreads();
-}
-
 // Kernel parts: one per layer kind, and polygon layers in two launches --
 // first the fill (kPolyFill: Algorithm 2), which leaves the strip's fill bits
 // as a bit mask (MASK layout, 32 bytes per pixel row) at the start of the
@@ -828,8 +386,7 @@ __device__ void stage(const Params& p, Smem& sm, const TreeArg& t, const void* o
 // part: Algorithm 1 over the edges), which reads those bits back, decides
 // the samples and encodes the composed strip over them.  Each CTA reads and
 // writes only its own strip's part of the output, so the bits never meet
-// another CTA's writes.  Apart, each part's traversal stays small enough for
-// the instruction cache; fused, the polygon kernel measured 40% slower.
+// another CTA's writes.
 constexpr int kPolyFill = 3;
 
 // The pattern texel of global pixel (gx, gy).
@@ -960,92 +517,6 @@ __device__ void encode_polygons(const Params& p, const uint8_t* res, uint8_t* ou
     }
 }
 
-// kSplit: the launch splits strips into column parts (p.parts > 1); the
-// full-width instantiation keeps the column arithmetic compile-time constant.
-template <int kKind, bool kProf, bool kSplit>
-__global__ void __launch_bounds__(kThreads, 4) k_render(const Params p) {
-    __shared__ Smem sm;
-    const int tid = threadIdx.x;
-    const long long t_start = tick<kProf>();
-    if constexpr (kProf) {
-        if (tid < kPN) sm.prof[tid] = 0;
-    }
-    const int rows = p.rows;
-    const int parts = kSplit ? p.parts : 1, cols = kTile / parts, col_shift = kSplit ? p.col_shift : 5;
-    // CTA -> tile, strip of rows pixel rows, part of cols pixel columns
-    const uint32_t tile = blockIdx.x / (p.strips * parts);
-    const int sp = (int)(blockIdx.x % (p.strips * parts));
-    const int strip = sp / parts, col0 = (sp % parts) * cols;
-    const uint32_t n = p.n_dev ? min(*p.n_dev, p.n) : p.n;
-    if (tile >= n) return;
-    hv_tile_req q = p.reqs[tile];
-    bool ok = q.z <= 19 && q.x < (1u << q.z) && q.y < (1u << q.z) && (p.R_units >= 0 || (q.r16 >= 1 && q.r16 <= 1024));
-    for (int k = tid; k < rows * kTile / 4; k += kThreads) ((uint32_t*)sm.res)[k] = 0u;
-    if (!ok) {
-        if (tid == 0 && sp == 0) atomicOr(p.status, 1u);
-    }
-    __syncthreads();
-    if (tid == 0) prof_since<kProf>(sm, kPPrologue, t_start, 0);
-    const bool mask_mode = p.mode == HV_MODE_MASK;
-    if (ok) {
-        const int z = q.z;
-        const int32_t ps = 1 << (23 - z);
-        const int32_t X0 = (int32_t)(-(int64_t)kGridHalf + (int64_t)q.x * ((int64_t)1 << (31 - z)));
-        const int32_t Y0 = (int32_t)(-(int64_t)kGridHalf + (int64_t)q.y * ((int64_t)1 << (31 - z)));
-        const bool learned = p.use_learned != 0;
-        // Algorithm 2 over polygon boxes and edges
-        {
-            // the CTA's centres, or its super-samples
-            const int32_t fo = (p.fill_aa && p.mode != HV_MODE_MASK) ? (ps >> 2) : 0;
-            const int32_t cx0 = X0 + col0 * ps + (ps >> 1) - fo, cx1 = X0 + (col0 + cols - 1) * ps + (ps >> 1) + fo;
-            const int32_t cy0 = Y0 + strip * rows * ps + (ps >> 1) - fo;
-            const int32_t cy1 = Y0 + (strip * rows + rows - 1) * ps + (ps >> 1) + fo;
-            stage<FillLeaf, kProf>(p, sm, p.mtree, p.mbr_obj, p.mbr_ids, p.mside, p.mside_obj, p.mside_ids,
-                            learned ? &p.mlm : nullptr, p.mhalo, X0, Y0, strip, col0, col_shift, z, 0, mask_mode,
-                            cx0, cy0,
-                            cx1, cy1, tid);
-        }
-    }
-    // ---- hand the strip's fill over ----
-    const long long t_enc = tick<kProf>();
-    uint8_t* out = p.out + (uint64_t)tile * p.tile_bytes;
-    {
-        // the fill results for the outline part, per pixel row at the start
-        // of the row's part of the CTA's own output (see decode_fill)
-        if (p.fill_aa && p.mode != HV_MODE_MASK) {
-            const int wpr = cols / 4, wsh = __ffs(wpr) - 1;
-            for (int k = tid; k < rows * wpr; k += kThreads) {
-                const int jl = k >> wsh, w = k & (wpr - 1);
-                ((uint32_t*)(out + px_offset(p.mode, strip * rows + jl, col0)))[w] =
-                    (((const uint32_t*)(sm.res + jl * kTile + col0))[w] >> kResFillShift) & 0x07070707u;
-            }
-        } else {
-            const int wpr = cols / 32, wsh = __ffs(wpr) - 1;
-            if (tid < rows * wpr) {
-                const int jl = tid >> wsh, w = tid & (wpr - 1);
-                uint32_t word = 0;
-                for (int b = 0; b < 32; b++)
-                    if (sm.res[jl * kTile + col0 + 32 * w + b] >> kResFillShift) word |= 1u << b;
-                ((uint32_t*)(out + px_offset(p.mode, strip * rows + jl, col0)))[w] = word;
-            }
-        }
-    }
-    if constexpr (kProf) {
-        __syncthreads();
-        if (tid == 0) {
-            const unsigned long long now = (unsigned long long)clock64();
-            sm.prof[kPEncode] += now - (unsigned long long)t_enc;
-            sm.prof[kPTotal] += now - (unsigned long long)t_start;
-            sm.prof[kPCtas] = 1;
-            // CTA-wide phases hold every warp of the CTA
-            const int cta_phases[6] = {kPTotal, kPPrologue, kPCull, kPBin, kPBlocksCta, kPEncode};
-            for (int k = 0; k < 6; k++) sm.prof[cta_phases[k]] *= kWarps;
-        }
-        __syncthreads();
-        if (tid < kPN && sm.prof[tid]) atomicAdd(p.phases + tid, sm.prof[tid]);
-    }
-}
-
 #include "hv_sweep.cuh"
 
 TreeArg tree_arg(const TreeView& v) {
@@ -1168,7 +639,6 @@ int launch_render(Layer* L, const hv_tile_req* d_reqs, uint32_t n, int mode, int
     if (p.rows == 4 && !prof)
         while (p.parts < 4 && (uint64_t)n * p.strips * p.parts * 2 <= resident) p.parts *= 2;
     p.cols = kTile / p.parts;
-    p.col_shift = p.parts == 1 ? 5 : (p.parts == 2 ? 4 : 3);
     uint64_t grid = (uint64_t)n * p.strips * p.parts;
     if (grid > 0x7fffffffull) {
         set_error("too many tiles in one call");
@@ -1183,7 +653,7 @@ int launch_render(Layer* L, const hv_tile_req* d_reqs, uint32_t n, int mode, int
         else if (L->kind == HV_LAYER_LINES)
             k_sweep<HV_LAYER_LINES, true, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         else {
-            k_render<kPolyFill, true, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+            k_sweep<kPolyFill, true, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
             Params q = p;
             q.phases = p.phases + kPN;
             k_sweep<HV_LAYER_POLYGONS, true, false><<<(unsigned)grid, kThreads, 0, stream>>>(q);
@@ -1194,7 +664,7 @@ int launch_render(Layer* L, const hv_tile_req* d_reqs, uint32_t n, int mode, int
         else if (L->kind == HV_LAYER_LINES)
             k_sweep<HV_LAYER_LINES, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         else {
-            k_render<kPolyFill, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+            k_sweep<kPolyFill, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
             k_sweep<HV_LAYER_POLYGONS, false, true><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         }
     } else if (L->kind == HV_LAYER_POINTS)
@@ -1203,7 +673,7 @@ int launch_render(Layer* L, const hv_tile_req* d_reqs, uint32_t n, int mode, int
         k_sweep<HV_LAYER_LINES, false, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
     else {
         // the fill first: the outline reads its bits and writes the tile
-        k_render<kPolyFill, false, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
+        k_sweep<kPolyFill, false, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
         k_sweep<HV_LAYER_POLYGONS, false, false><<<(unsigned)grid, kThreads, 0, stream>>>(p);
     }
     HV_CUDA(cudaGetLastError());

@@ -135,3 +135,56 @@ def test_segments_at_ground_radii(ctx, radius):
     seg = _fan(np.random.default_rng(5), 400, 2 ** 22, 2 ** 23)
     _check(ctx, seg, [[7, 64, 63, 1], [11, 1024, 1024, 1], [16, 32768, 32767, 1]], radius=radius, lines=True,
            batches=(1, 150))
+
+
+def _rings(rng):
+    """Polygons for the fill: a comb of 401 vertices across many tiles, squares
+    on sample positions and word borders, nested rings, slivers, one as wide
+    as the grid, and overlapping stars."""
+    P = []
+    x = np.repeat(np.linspace(-3e6, 3e6, 200), 2)
+    y = np.tile([-2e6, 2e6, 2e6, -2e6], 100) + rng.integers(-5, 5, 400)
+    P.append([np.concatenate([np.stack([x, y], 1), [[0, 2.5e6]]])])
+    for z, i, j, k in ((9, 0, 0, 32), (11, 31, 15, 33), (13, 224, 240, 32), (10, 255, 255, 3)):
+        cx, cy = centre(z, (1 << z) // 2, (1 << z) // 2, i, j)
+        d = k * ps(z)
+        sq = np.array([[0, 0], [d, 0], [d, d], [0, d]])
+        P.append([sq + (cx, cy), sq // 2 + (cx + d // 4, cy + d // 4)])
+        P.append([sq + (cx + ps(z) // 4, cy - ps(z) // 4)])
+    P.append([np.array([[-HALF, -5], [HALF - 1, 3], [HALF - 1, 90_000], [-HALF, 70_000]])])
+    P.append([np.array([[-HALF, -HALF], [HALF - 1, -HALF], [0, -HALF // 2]])])
+    for _ in range(60):
+        c, m = rng.integers(-2 ** 22, 2 ** 22, 2), int(rng.integers(3, 90))
+        a = np.sort(rng.uniform(0, 2 * np.pi, m))
+        r = 2.0 ** rng.uniform(8, 22) * rng.uniform(0.3, 1, m)
+        P.append([c + np.stack([r * np.cos(a), r * np.sin(a)], 1)])
+    rings = [np.clip(np.floor(r), -HALF, HALF - 1).astype(np.int32) for p in P for r in p]
+    ro = np.concatenate([[0], np.cumsum([len(r) for r in rings])]).astype(np.uint64)
+    po = np.concatenate([[0], np.cumsum([len(p) for p in P])]).astype(np.uint64)
+    return np.concatenate(rings), ro, po
+
+
+@pytest.mark.parametrize("aa", [False, True])
+def test_fill_of_every_width(ctx, aa):
+    xy, ro, po = _rings(np.random.default_rng(8))
+    L = hv.hv_layer_load_polygons(ctx, xy, ro, po)
+    hv.hv_layer_build_index(L, hv.HV_INDEX_RTREE | hv.HV_INDEX_LEARNED)
+    reqs = np.array([[0, 0, 0, 8], [1, 0, 1, 16], [8, 128, 127, 8]] +
+                    [[z, (1 << z) // 2 - a, (1 << z) // 2 - b, 4] for z in (9, 11, 13, 16) for a in (0, 1) for b in (0, 1)],
+                    dtype=np.uint32)
+    s, fill = hv.make_style(STYLE_T[:3], STYLE_T[4:7]), hv.make_fill_style(aa=aa)
+    try:
+        for mode in MODES:
+            ref = oracle_par.render(lambda r: oracle.render_polygons(xy, ro, po, r, mode, STYLE_T, aa=aa), reqs)
+            for index in (hv.HV_INDEX_RTREE, hv.HV_INDEX_LEARNED):
+                for per in (1, 3, 150):
+                    rows = np.resize(np.arange(len(reqs)), max(per, len(reqs)))
+                    for k in range(0, len(rows), per):
+                        part = rows[k:k + per]
+                        d = torch.from_numpy(hv.make_requests(reqs[part]).view(np.uint8).copy()).cuda()
+                        out = torch.full((len(part), hv.hv_tile_bytes(mode)), 0xAB, dtype=torch.uint8, device="cuda")
+                        hv.hv_render_tiles_styled(L, d, len(part), mode, index, s, fill, out, out.numel(), None)
+                        assert np.array_equal(out.cpu().numpy(), ref[part]), (mode, index, per)
+        assert hv.hv_layer_take_status(L) == 0
+    finally:
+        hv.hv_layer_free(L)
