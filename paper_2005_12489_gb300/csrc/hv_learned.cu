@@ -110,140 +110,251 @@ __global__ void k_to_bf16(const float* src, __nv_bfloat16* dst, uint64_t n) {
     if (i < n) dst[i] = __float2bfloat16(src[i]);
 }
 
-__device__ __forceinline__ float warp_sum_f(float v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    return v;
+// The piece of the key at position i: i / P, or (equal keys across a piece's
+// end) the last piece whose first key is not above it.
+__device__ __forceinline__ uint32_t piece_of(const LModel& m, uint64_t i, uint64_t k) {
+    const uint32_t j = (uint32_t)(i / m.P);
+    return j + 1 < m.n_seg && __ldg(m.kb + j + 1) <= k ? learn_piece(m, k) : j;
 }
 
-// One training step on kBatch sampled keys: forward with the fp32 master
-// weights, squared error against the residual of the linear piece, backward;
-// gradients warp-reduced, then accumulated in shared and global memory.
-__global__ void k_train(LModel m, const float* w, const float* emb, float* gw, float* gemb, int step, uint32_t seed) {
-    __shared__ float sg[kLearnNW];
+// One training step on kBatch sampled keys, one per thread: forward with the
+// fp32 master weights, squared error against the residual of the linear
+// piece, backward.  Every weight's gradient is a sum over samples of a product
+// of two of the sample's values (an input, activation or error, or one), so the
+// block keeps those values as rows of shared memory, a column per sample, and
+// each thread forms a few gradients as dot products of two rows (fp32, four
+// partial sums), then adds them to the global ones: 256 products where a warp
+// reduction per gradient and sample took ten shuffles and adds.  The weights
+// are read from shared memory, the sample's values stay in registers.
+// (65,536 samples took 123 us by warp reductions with the activations in local
+// memory.)
+constexpr int kTrainThreads = 128;
+constexpr int kRowIn = 0, kRowH1 = kRowIn + kLearnIn, kRowD1 = kRowH1 + kLearnH, kRowH2 = kRowD1 + kLearnH,
+              kRowD2 = kRowH2 + kLearnH, kRowDo = kRowD2 + kLearnH, kRowOne = kRowDo + 1, kRows = kRowOne + 1;
+constexpr int kRowStride = kTrainThreads + 4;   // rows 4 banks apart: 8 rows' float4s meet 32 banks
+static_assert(kBatch % kTrainThreads == 0, "one sample per thread");
+static_assert((kRows * kRowStride + kLearnNW) * 4 <= 48 * 1024, "static shared memory");
+
+__global__ void __launch_bounds__(kTrainThreads, 4) k_train(LModel m, const float* w, const float* emb, float* gw, float* gemb,
+                                                         int step, uint32_t seed) {
     constexpr int H = kLearnH;
-    constexpr int nw = kLearnNW;
-    for (int i = threadIdx.x; i < nw; i += blockDim.x) sg[i] = 0.f;
-    __syncthreads();
-    uint64_t gid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    __shared__ __align__(16) float rows[kRows * kRowStride];
+    __shared__ __align__(16) float sw[kLearnNW];
+    const int tid = threadIdx.x;
+    for (int i = tid; i < kLearnNW; i += kTrainThreads) sw[i] = w[i];
+    uint64_t gid = blockIdx.x * (uint64_t)blockDim.x + tid;
     uint64_t h = ((uint64_t)seed << 32) ^ ((uint64_t)step * 0x9E3779B97F4A7C15ull) ^ (gid * 0xD1B54A32D192ED03ull);
     h ^= h >> 31; h *= 0x94D049BB133111EBull; h ^= h >> 29;
-    uint64_t i = h % m.n;
-    uint64_t k = m.keys[i];
-    uint32_t j = learn_piece(m, k);
-    uint64_t kbj = m.kb[j];
-    float x = (float)(k - kbj);
-    float lin = m.pc[j] + m.pa[j] * x;
-    float target = ((float)((double)i - (double)j * m.P) - lin) / (float)m.P;
+    const uint64_t i = h % m.n;
+    const uint64_t k = m.keys[i];
+    const uint32_t j = piece_of(m, i, k);
+    const float x = (float)(k - m.kb[j]);
+    const float target = ((float)((double)i - (double)j * m.P) - learn_line(m, j, x)) / (float)m.P;
     float in[kLearnIn];
     in[0] = fminf(fmaxf(x * m.pinv[j], 0.f), 1.f);
-    for (int q = 0; q < 4; q++) in[1 + q] = emb[(uint64_t)j * 4 + q];
-    const float* W1 = w;
-    const float* B1 = W1 + H * kLearnIn;
-    const float* W2 = B1 + H;
-    const float* B2 = W2 + H * H;
-    const float* W3 = B2 + H;
-    const float* B3 = W3 + H;
-    float h1[H], h2[H], d2[H], d1[H];
+    const float4 e4 = *(const float4*)(emb + (uint64_t)j * 4);
+    in[1] = e4.x, in[2] = e4.y, in[3] = e4.z, in[4] = e4.w;
+    __syncthreads();
+    const NetF32 net{sw};
+    float* col = rows + tid;   // the sample's column
+    float v[H];                // h1, then d1
+#pragma unroll
     for (int r = 0; r < H; r++) {
-        float acc = B1[r];
-        for (int q = 0; q < kLearnIn; q++) acc = fmaf(W1[r * kLearnIn + q], in[q], acc);
-        h1[r] = fmaxf(acc, 0.f);
+        float acc = net.b1(r);
+#pragma unroll
+        for (int q = 0; q < kLearnIn; q++) acc = fmaf(net.w1(r, q), in[q], acc);
+        v[r] = fmaxf(acc, 0.f);
+        col[(kRowH1 + r) * kRowStride] = v[r];
     }
+    float out = net.b3();
+    // (a few rows of W2 at a time: unrolled whole, the loads ahead spill)
+#pragma unroll 2
     for (int r = 0; r < H; r++) {
-        float acc = B2[r];
-        for (int q = 0; q < H; q++) acc = fmaf(W2[r * H + q], h1[q], acc);
-        h2[r] = fmaxf(acc, 0.f);
+        float acc = net.b2(r);
+        const float4* w4 = (const float4*)(sw + kLearnW2 + r * H);
+#pragma unroll
+        for (int q = 0; q < H / 4; q++) {
+            const float4 u = w4[q];
+            acc = fmaf(u.x, v[4 * q], acc);
+            acc = fmaf(u.y, v[4 * q + 1], acc);
+            acc = fmaf(u.z, v[4 * q + 2], acc);
+            acc = fmaf(u.w, v[4 * q + 3], acc);
+        }
+        acc = fmaxf(acc, 0.f);
+        col[(kRowH2 + r) * kRowStride] = acc;
+        out = fmaf(net.w3(r), acc, out);
     }
-    float out = B3[0];
-    for (int q = 0; q < H; q++) out = fmaf(W3[q], h2[q], out);
-    float dout = 2.f * (out - target) / (float)kBatch;
-    for (int r = 0; r < H; r++) d2[r] = h2[r] > 0.f ? dout * W3[r] : 0.f;
-    for (int q = 0; q < H; q++) {
-        float acc = 0.f;
-        for (int r = 0; r < H; r++) acc = fmaf(d2[r], W2[r * H + q], acc);
-        d1[q] = h1[q] > 0.f ? acc : 0.f;
+    const float dout = 2.f * (out - target) / (float)kBatch;
+#pragma unroll
+    for (int q = 0; q < H; q++) v[q] = 0.f;
+#pragma unroll 2
+    for (int r = 0; r < H; r++) {
+        const float d2 = col[(kRowH2 + r) * kRowStride] > 0.f ? dout * net.w3(r) : 0.f;
+        col[(kRowD2 + r) * kRowStride] = d2;
+        const float4* w4 = (const float4*)(sw + kLearnW2 + r * H);
+#pragma unroll
+        for (int q = 0; q < H / 4; q++) {
+            const float4 u = w4[q];
+            v[4 * q] = fmaf(d2, u.x, v[4 * q]);
+            v[4 * q + 1] = fmaf(d2, u.y, v[4 * q + 1]);
+            v[4 * q + 2] = fmaf(d2, u.z, v[4 * q + 2]);
+            v[4 * q + 3] = fmaf(d2, u.w, v[4 * q + 3]);
+        }
     }
     // embedding gradient (input features 1..4): a piece's embedding sees about
     // one sample per step, so it takes the per-sample gradient, not the batch
     // mean the shared weights take
-    for (int q = 1; q < kLearnIn; q++) {
-        float acc = 0.f;
-        for (int r = 0; r < H; r++) acc = fmaf(d1[r], W1[r * kLearnIn + q], acc);
-        atomicAdd(gemb + (uint64_t)j * 4 + (q - 1), acc * (float)kBatch);
+    float ge[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int q = 0; q < H; q++) {
+        const float d1 = col[(kRowH1 + q) * kRowStride] > 0.f ? v[q] : 0.f;
+        col[(kRowD1 + q) * kRowStride] = d1;
+#pragma unroll
+        for (int f = 0; f < 4; f++) ge[f] = fmaf(d1, net.w1(q, 1 + f), ge[f]);
     }
-    int lane = threadIdx.x & 31;
-    int idx = 0;
-#define HV_ACC(val)                                  \
-    {                                                \
-        float v_ = warp_sum_f(val);                  \
-        if (lane == 0) atomicAdd(sg + idx, v_);      \
-        idx++;                                       \
-    }
-#pragma unroll 1
-    for (int r = 0; r < H; r++)
-        for (int q = 0; q < kLearnIn; q++) HV_ACC(d1[r] * in[q]);
-#pragma unroll 1
-    for (int r = 0; r < H; r++) HV_ACC(d1[r]);
-#pragma unroll 1
-    for (int r = 0; r < H; r++)
-        for (int q = 0; q < H; q++) HV_ACC(d2[r] * h1[q]);
-    for (int r = 0; r < H; r++) HV_ACC(d2[r]);
-    for (int q = 0; q < H; q++) HV_ACC(dout * h2[q]);
-    HV_ACC(dout);
-#undef HV_ACC
+#pragma unroll
+    for (int q = 0; q < kLearnIn; q++) col[(kRowIn + q) * kRowStride] = in[q];
+    col[kRowDo * kRowStride] = dout;
+    col[kRowOne * kRowStride] = 1.f;
+#pragma unroll
+    for (int f = 0; f < 4; f++) atomicAdd(gemb + (uint64_t)j * 4 + f, ge[f] * (float)kBatch);
     __syncthreads();
-    for (int t = threadIdx.x; t < nw; t += blockDim.x) atomicAdd(gw + t, sg[t]);
-}
-
-__global__ void k_adam(float* w, float* g, float* mo, float* ve, int nw, int step, float lr) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nw) return;
-    const float b1 = 0.9f, b2 = 0.999f;
-    float gi = g[i];
-    mo[i] = b1 * mo[i] + (1 - b1) * gi;
-    ve[i] = b2 * ve[i] + (1 - b2) * gi * gi;
-    float mh = mo[i] / (1 - powf(b1, (float)(step + 1)));
-    float vh = ve[i] / (1 - powf(b2, (float)(step + 1)));
-    w[i] -= lr * mh / (sqrtf(vh) + 1e-8f);
-    g[i] = 0.f;
-}
-
-__global__ void k_sgd(float* w, float* g, uint64_t n, float lr) {
-    uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    w[i] -= lr * g[i];
-    g[i] = 0.f;
-}
-
-// Per-piece error bound over every stored key, measured with the inference
-// code the lookups use.
-__global__ void k_eps(LModel m, uint32_t* eps, unsigned long long* sum_err) {
-    uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    float e = 0.f;
-    if (i < m.n) {
-        uint64_t k = m.keys[i];
-        uint32_t j = learn_piece(m, k);
-        float within = learn_predict(m, j, k);
-        int64_t c = (int64_t)j * m.P + (int64_t)floorf(within);
-        int64_t d = (int64_t)i - c;
-        if (d < 0) d = -d;
-        atomicMax(eps + j, (uint32_t)(d > 0xfffffff0ll ? 0xfffffff0ll : d));
-        e = fabsf(within - (float)((int64_t)i - (int64_t)j * m.P));
+    for (int o = tid; o < kLearnNW; o += kTrainThreads) {
+        // the two rows whose product's sum is gradient o
+        int a, b;
+        if (o < kLearnB1) a = kRowD1 + o / kLearnIn, b = kRowIn + o % kLearnIn;
+        else if (o < kLearnW2) a = kRowD1 + (o - kLearnB1), b = kRowOne;
+        else if (o < kLearnB2) a = kRowD2 + (o - kLearnW2) / H, b = kRowH1 + (o - kLearnW2) % H;
+        else if (o < kLearnW3) a = kRowD2 + (o - kLearnB2), b = kRowOne;
+        else if (o < kLearnB3) a = kRowDo, b = kRowH2 + (o - kLearnW3);
+        else a = kRowDo, b = kRowOne;
+        const float4* pa = (const float4*)(rows + a * kRowStride);
+        const float4* pb = (const float4*)(rows + b * kRowStride);
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+        for (int c = 0; c < kTrainThreads / 4; c++) {
+            const float4 u = pa[c], v = pb[c];
+            s.x = fmaf(u.x, v.x, s.x);
+            s.y = fmaf(u.y, v.y, s.y);
+            s.z = fmaf(u.z, v.z, s.z);
+            s.w = fmaf(u.w, v.w, s.w);
+        }
+        atomicAdd(gw + o, (s.x + s.y) + (s.z + s.w));
     }
-    // mean absolute error, for reporting
-    unsigned long long s = (unsigned long long)e;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(sum_err, s);
 }
 
-// max and sum of the per-piece bounds (out[0] = max, out[1] = sum)
+// End of a step: Adam on the network's weights (the first kLearnNW threads) and
+// SGD on the embeddings, in one launch.
+__global__ void k_update(float* w, float* g, float* mo, float* ve, int step, float lr, float* emb, float* gemb,
+                         uint64_t n_emb, float lr_emb) {
+    uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    if (i < (uint64_t)kLearnNW) {
+        const float b1 = 0.9f, b2 = 0.999f;
+        float gi = g[i];
+        mo[i] = b1 * mo[i] + (1 - b1) * gi;
+        ve[i] = b2 * ve[i] + (1 - b2) * gi * gi;
+        float mh = mo[i] / (1 - powf(b1, (float)(step + 1)));
+        float vh = ve[i] / (1 - powf(b2, (float)(step + 1)));
+        w[i] -= lr * mh / (sqrtf(vh) + 1e-8f);
+        g[i] = 0.f;
+        return;
+    }
+    i -= kLearnNW;
+    if (i < n_emb) {
+        emb[i] -= lr_emb * gemb[i];
+        gemb[i] = 0.f;
+    }
+}
+
+// Error of one prediction: the position error that a lookup's window has to
+// cover, and the offset error (whole units) for the reported mean.
+__device__ __forceinline__ void prediction_error(const LModel& m, uint64_t i, uint32_t j, float within, uint32_t* pos,
+                                                 uint32_t* off) {
+    const int64_t c = (int64_t)j * m.P + (int64_t)floorf(within);
+    int64_t d = (int64_t)i - c;
+    if (d < 0) d = -d;
+    *pos = (uint32_t)(d > 0xfffffff0ll ? 0xfffffff0ll : d);
+    *off = (uint32_t)fminf(fabsf(within - (float)((int64_t)i - (int64_t)j * m.P)), 4294967040.f);
+}
+
+// Per-piece error bounds (and summed errors) over every stored key, of the
+// lines alone and, with kMlp, of lines and network, in one pass with the steps
+// that the lookups take.  One warp per piece: the piece's parameters and
+// the network are read once (the weights as floats in shared memory) and its
+// maximum and sum are formed in registers; only keys equal to the next
+// piece's first key belong elsewhere and go there by themselves.  (Without
+// kMlp there is nothing to choose between pieces and sum_l is one number.)
+template <bool kMlp>
+__global__ void __launch_bounds__(256) k_eps(LModel m, uint32_t* eps_l, uint32_t* eps_m, unsigned long long* sum_l,
+                                             unsigned long long* sum_m) {
+    __shared__ float sw[kLearnNW];
+    if (kMlp) {
+        for (int i = threadIdx.x; i < kLearnNW; i += blockDim.x) sw[i] = __bfloat162float(m.w[i]);
+        __syncthreads();
+    }
+    const uint64_t j0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (j0 >= m.n_seg) return;
+    const uint64_t i0 = j0 * m.P, i1 = i0 + m.P < m.n ? i0 + m.P : m.n;
+    const uint64_t next = j0 + 1 < m.n_seg ? m.kb[j0 + 1] : ~0ull;
+    uint32_t el = 0, em = 0;
+    unsigned long long sl = 0, sm = 0;
+    const NetF32 net{sw};
+    for (uint64_t i = i0 + lane; i < i1; i += 32) {
+        const uint64_t k = __ldg(m.keys + i);
+        const bool own = k < next;
+        const uint32_t j = own ? (uint32_t)j0 : learn_piece(m, k);
+        const float x = (float)(k - __ldg(m.kb + j));
+        const float line = learn_line(m, j, x);
+        uint32_t pos, off;
+        prediction_error(m, i, j, line, &pos, &off);
+        if (own) {
+            el = max(el, pos);
+            sl += off;
+        } else {
+            atomicMax(eps_l + j, pos);
+            atomicAdd(sum_l + (kMlp ? j : 0), (unsigned long long)off);
+        }
+        if (kMlp) {
+            float in[kLearnIn];
+            learn_input(m, j, x, in);
+            prediction_error(m, i, j, fmaf((float)m.P, learn_net(net, in), line), &pos, &off);
+            if (own) {
+                em = max(em, pos);
+                sm += off;
+            } else {
+                atomicMax(eps_m + j, pos);
+                atomicAdd(sum_m + j, (unsigned long long)off);
+            }
+        }
+    }
+    el = __reduce_max_sync(kFull, el);
+    if (kMlp) em = __reduce_max_sync(kFull, em);
+    for (int o = 16; o > 0; o >>= 1) {
+        sl += __shfl_xor_sync(kFull, sl, o);
+        if (kMlp) sm += __shfl_xor_sync(kFull, sm, o);
+    }
+    if (lane == 0) {
+        atomicMax(eps_l + j0, el);
+        atomicAdd(sum_l + (kMlp ? j0 : 0), sl);
+        if (kMlp) {
+            atomicMax(eps_m + j0, em);
+            atomicAdd(sum_m + j0, sm);
+        }
+    }
+}
+
 // Keep the MLP term for a piece only where it narrows the piece's bound.
-__global__ void k_choose(const uint32_t* eps_lin, uint32_t* eps, uint8_t* use, uint32_t n_seg) {
+__global__ void k_choose(const uint32_t* eps_lin, uint32_t* eps, uint8_t* use, uint32_t n_seg,
+                         const unsigned long long* sum_lin, unsigned long long* sum) {
     uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n_seg) return;
     bool u = eps[j] < eps_lin[j];
     use[j] = u ? 1 : 0;
-    if (!u) eps[j] = eps_lin[j];
+    if (!u) {
+        eps[j] = eps_lin[j];
+        sum[j] = sum_lin[j];
+    }
 }
 
 __global__ void k_count_u8(const uint8_t* a, uint32_t n, unsigned long long* out) {
@@ -258,15 +369,21 @@ __global__ void k_fill_u8(uint8_t* a, uint32_t n, uint8_t v) {
     if (j < n) a[j] = v;
 }
 
-__global__ void k_max_u32(const uint32_t* a, uint32_t n, unsigned long long* out) {
+// Over the pieces: out[0] = sum of the summed errors, out[1] = largest bound,
+// out[2] = sum of the bounds.
+__global__ void k_bounds(const uint32_t* eps, const unsigned long long* sum, uint32_t n, unsigned long long* out) {
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t v = i < n ? a[i] : 0u;
+    uint32_t v = i < n ? eps[i] : 0u;
     uint32_t mx = __reduce_max_sync(kFull, v);
-    unsigned long long sm = v;
-    for (int o = 16; o > 0; o >>= 1) sm += __shfl_xor_sync(kFull, sm, o);
+    unsigned long long sm = v, er = sum && i < n ? sum[i] : 0ull;
+    for (int o = 16; o > 0; o >>= 1) {
+        sm += __shfl_xor_sync(kFull, sm, o);
+        er += __shfl_xor_sync(kFull, er, o);
+    }
     if ((threadIdx.x & 31) == 0) {
-        atomicMax(out, (unsigned long long)mx);
-        atomicAdd(out + 1, sm);
+        atomicAdd(out, er);
+        atomicMax(out + 1, (unsigned long long)mx);
+        atomicAdd(out + 2, sm);
     }
 }
 
@@ -355,42 +472,43 @@ static int build_one(Ctx* c, Learned* L, const uint64_t* keys, uint64_t n, const
     LModel m;
     m.keys = keys; m.n = n; m.kb = kb; m.pa = pa; m.pc = pc; m.pinv = pinv; m.eps = eps; m.rt = rt;
     m.emb = nullptr; m.w = nullptr; m.use_mlp = nullptr; m.n_seg = n_seg; m.P = P; m.hidden = 0;
-    // error of the linear pieces alone
     unsigned long long* scratch;
     HV_TRY(dev_alloc(c, (void**)&scratch, 64));
+    struct Free {
+        Ctx* c;
+        void* p;
+        ~Free() { dev_free(c, p, 64); }
+    } free_scratch{c, scratch};
+    HV_CUDA(cudaMemset(scratch, 0, 64));
+    uint8_t* use;
+    uint32_t* eps_l;
+    HV_TRY(A.get((void**)&use, n_seg));
+    HV_TRY(A.get((void**)&eps_l, (uint64_t)n_seg * 4));
+    k_fill_u8<<<blocks_for(n_seg, 256), 256>>>(use, n_seg, 0);
+    HV_CUDA(cudaMemset(eps_l, 0, (uint64_t)n_seg * 4));
+    m.use_mlp = use;
     // max bound, mean |error|, and the sum of per-piece bounds (the average
     // search window, what a lookup pays)
-    auto measure = [&](const LModel& mm, uint32_t* max_eps, double* mean, double* sum_eps) -> int {
-        cudaMemset(eps, 0, (uint64_t)n_seg * 4);
-        cudaMemset(scratch, 0, 64);
-        k_eps<<<blocks_for(n, 256), 256>>>(mm, eps, scratch);
-        k_max_u32<<<blocks_for(n_seg, 256), 256>>>(eps, n_seg, scratch + 1);
-        unsigned long long h[3];
-        cudaError_t e = cudaMemcpy(h, scratch, 24, cudaMemcpyDeviceToHost);
+    auto bounds = [&](const uint32_t* e_piece, const unsigned long long* s_piece, uint32_t* max_eps, double* mean,
+                      double* sum_eps) -> int {
+        cudaMemset(scratch, 0, 24);
+        k_bounds<<<blocks_for(n_seg, 256), 256>>>(e_piece, s_piece, n_seg, scratch);
+        unsigned long long h[4];
+        cudaError_t e = cudaMemcpy(h, scratch, 32, cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) { set_error("learned error pass: %s", cudaGetErrorString(e)); return HV_ECUDA; }
-        *mean = (double)h[0] / (double)n;
+        *mean = (double)(s_piece ? h[0] : h[3]) / (double)n;
         *max_eps = (uint32_t)h[1];
         *sum_eps = (double)h[2];
         return HV_OK;
     };
     uint32_t eps_lin = 0, eps_mlp = 0, eps_fin = 0;
     double mean_lin = 0, mean_mlp = 0, sum_lin = 0, sum_mlp = 0, mean_fin = 0, sum_fin = 0;
-    uint8_t* use;
-    uint32_t* eps_l;
-    HV_TRY(A.get((void**)&use, n_seg));
-    HV_TRY(A.get((void**)&eps_l, (uint64_t)n_seg * 4));
-    k_fill_u8<<<blocks_for(n_seg, 256), 256>>>(use, n_seg, 0);
-    m.use_mlp = use;
-    int rc = measure(m, &eps_lin, &mean_lin, &sum_lin);
-    if (rc != HV_OK) { dev_free(c, scratch, 64); return rc; }
-    HV_CUDA(cudaMemcpy(eps_l, eps, (uint64_t)n_seg * 4, cudaMemcpyDeviceToDevice));
-    eps_fin = eps_lin; mean_fin = mean_lin; sum_fin = sum_lin;
     // MLP residual, trained on the device
     cudaEvent_t t0, t1;
     cudaEventCreate(&t0);
     cudaEventCreate(&t1);
     cudaEventRecord(t0);
-    int nw = H * kLearnIn + H + H * H + H + H + 1;
+    int nw = kLearnNW;
     float *w, *gw, *mo, *ve, *emb, *gemb;
     __nv_bfloat16 *wb, *embb;
     bool ok = A.get((void**)&w, nw * 4) == HV_OK && A.get((void**)&gw, nw * 4) == HV_OK &&
@@ -398,6 +516,7 @@ static int build_one(Ctx* c, Learned* L, const uint64_t* keys, uint64_t n, const
               A.get((void**)&emb, (uint64_t)n_seg * 16) == HV_OK && A.get((void**)&gemb, (uint64_t)n_seg * 16) == HV_OK &&
               A.get((void**)&wb, nw * 2) == HV_OK && A.get((void**)&embb, (uint64_t)n_seg * 8) == HV_OK;
     uint32_t pieces_mlp = 0;
+    const uint32_t piece_blocks = blocks_for((uint64_t)n_seg * 32, 256);
     if (ok && steps > 0 && H > 0) {
         cudaMemset(gw, 0, nw * 4);
         cudaMemset(mo, 0, nw * 4);
@@ -408,26 +527,29 @@ static int build_one(Ctx* c, Learned* L, const uint64_t* keys, uint64_t n, const
         LModel tm = m;
         tm.hidden = H;
         for (int s = 0; s < steps; s++) {
-            k_train<<<kBatch / 256, 256>>>(tm, w, emb, gw, gemb, s, seed);
-            k_adam<<<blocks_for(nw, 256), 256>>>(w, gw, mo, ve, nw, s, 2e-3f);
-            k_sgd<<<blocks_for((uint64_t)n_seg * 4, 256), 256>>>(emb, gemb, (uint64_t)n_seg * 4, 0.02f);
+            k_train<<<kBatch / kTrainThreads, kTrainThreads>>>(tm, w, emb, gw, gemb, s, seed);
+            k_update<<<blocks_for(nw + (uint64_t)n_seg * 4, 256), 256>>>(w, gw, mo, ve, s, 2e-3f, emb, gemb,
+                                                                         (uint64_t)n_seg * 4, 0.02f);
         }
         k_to_bf16<<<blocks_for(nw, 256), 256>>>(w, wb, nw);
         k_to_bf16<<<blocks_for((uint64_t)n_seg * 4, 256), 256>>>(emb, embb, (uint64_t)n_seg * 4);
         HV_CUDA(cudaGetLastError());
-        // every piece with the MLP term ...
+        // the bounds of every piece without and with the MLP term ...
         LModel mm = m;
         mm.hidden = H;
         mm.w = wb;
         mm.emb = embb;
-        k_fill_u8<<<blocks_for(n_seg, 256), 256>>>(use, n_seg, 1);
-        rc = measure(mm, &eps_mlp, &mean_mlp, &sum_mlp);
-        if (rc != HV_OK) { dev_free(c, scratch, 64); return rc; }
-        // ... then each piece keeps the model with the narrower bound, and the
-        // bounds are measured again with the combined model
-        k_choose<<<blocks_for(n_seg, 256), 256>>>(eps_l, eps, use, n_seg);
-        rc = measure(mm, &eps_fin, &mean_fin, &sum_fin);
-        if (rc != HV_OK) { dev_free(c, scratch, 64); return rc; }
+        HV_CUDA(cudaMemset(eps, 0, (uint64_t)n_seg * 4));
+        // (the embeddings' gradient array, no longer needed, holds the summed errors)
+        unsigned long long *sum_l = (unsigned long long*)gemb, *sum_m = sum_l + n_seg;
+        HV_CUDA(cudaMemset(gemb, 0, (uint64_t)n_seg * 16));
+        k_eps<true><<<piece_blocks, 256>>>(mm, eps_l, eps, sum_l, sum_m);
+        HV_TRY(bounds(eps_l, sum_l, &eps_lin, &mean_lin, &sum_lin));
+        HV_TRY(bounds(eps, sum_m, &eps_mlp, &mean_mlp, &sum_mlp));
+        // ... then each piece keeps the model with the narrower bound, and that
+        // model's errors are the combined model's
+        k_choose<<<blocks_for(n_seg, 256), 256>>>(eps_l, eps, use, n_seg, sum_l, sum_m);
+        HV_TRY(bounds(eps, sum_m, &eps_fin, &mean_fin, &sum_fin));
         unsigned long long* cntd = scratch + 4;
         HV_CUDA(cudaMemset(cntd, 0, 8));
         k_count_u8<<<blocks_for(n_seg, 256), 256>>>(use, n_seg, cntd);
@@ -435,6 +557,10 @@ static int build_one(Ctx* c, Learned* L, const uint64_t* keys, uint64_t n, const
         HV_CUDA(cudaMemcpy(&hc, cntd, 8, cudaMemcpyDeviceToHost));
         pieces_mlp = (uint32_t)hc;
         if (pieces_mlp) m = mm;
+    } else {
+        // (one sum over all pieces: nothing to choose between)
+        k_eps<false><<<piece_blocks, 256>>>(m, eps_l, nullptr, scratch + 3, nullptr);
+        HV_TRY(bounds(eps_l, nullptr, &eps_lin, &mean_lin, &sum_lin));
     }
     cudaEventRecord(t1);
     cudaEventSynchronize(t1);
@@ -444,11 +570,10 @@ static int build_one(Ctx* c, Learned* L, const uint64_t* keys, uint64_t n, const
     cudaEventDestroy(t1);
     L->train_ms += ms;
     if (!pieces_mlp) {
-        k_fill_u8<<<blocks_for(n_seg, 256), 256>>>(use, n_seg, 0);
-        rc = measure(m, &eps_fin, &mean_fin, &sum_fin);  // the linear bounds alone
-        if (rc != HV_OK) { dev_free(c, scratch, 64); return rc; }
+        // the linear bounds alone
+        HV_CUDA(cudaMemcpy(eps, eps_l, (uint64_t)n_seg * 4, cudaMemcpyDeviceToDevice));
+        eps_fin = eps_lin; mean_fin = mean_lin; sum_fin = sum_lin;
     }
-    dev_free(c, scratch, 64);
     v.seg_a = pa;
     v.seg_b = pc;
     v.seg_k0 = kb;
@@ -502,7 +627,7 @@ static int build_one(Ctx* c, Learned* L, const uint64_t* keys, uint64_t n, const
         if (n_out) {
             int4* oo;
             uint32_t* oid;
-            rc = dev_alloc(c, (void**)&oo, n_out * 16);
+            int rc = dev_alloc(c, (void**)&oo, n_out * 16);
             if (rc == HV_OK) rc = dev_alloc(c, (void**)&oid, n_out * 4);
             if (rc != HV_OK) { dev_free(c, flag, n * 4); dev_free(c, cnt, 16); return rc; }
             cudaMemset(cnt + 1, 0, 8);

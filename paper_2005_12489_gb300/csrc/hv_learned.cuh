@@ -60,50 +60,79 @@ __device__ __forceinline__ uint32_t learn_piece(const LModel& m, uint64_t k) {
     return (uint32_t)a;
 }
 
-// MLP residual in units of P (fp32 accumulation over bf16 weights).
-__device__ __forceinline__ float learn_mlp(const LModel& m, uint32_t j, float t) {
+// The residual network on one input, given its layers as functions of their
+// indices: w1(r, q), b1(r), w2(r, q), b2(r), w3(q), b3.  Every caller takes the
+// same steps in the same order, so a prediction has the same bits wherever the
+// weights are read from.
+template <class Net>
+__device__ __forceinline__ float learn_net(const Net& net, const float in[kLearnIn]) {
     constexpr int H = kLearnH;
-    const __nv_bfloat16* w = m.w;
-    float in[kLearnIn];
-    in[0] = t;
-#pragma unroll
-    for (int q = 0; q < 4; q++) in[1 + q] = __bfloat162float(m.emb[(uint64_t)j * 4 + q]);
     float h1[H], h2[H];
-    const __nv_bfloat16* W1 = w;
-    const __nv_bfloat16* B1 = W1 + H * kLearnIn;
-    const __nv_bfloat16* W2 = B1 + H;
-    const __nv_bfloat16* B2 = W2 + H * H;
-    const __nv_bfloat16* W3 = B2 + H;
-    const __nv_bfloat16* B3 = W3 + H;
 #pragma unroll
     for (int r = 0; r < H; r++) {
-        float acc = __bfloat162float(B1[r]);
+        float acc = net.b1(r);
 #pragma unroll
-        for (int q = 0; q < kLearnIn; q++) acc = fmaf(__bfloat162float(W1[r * kLearnIn + q]), in[q], acc);
+        for (int q = 0; q < kLearnIn; q++) acc = fmaf(net.w1(r, q), in[q], acc);
         h1[r] = fmaxf(acc, 0.f);
     }
 #pragma unroll
     for (int r = 0; r < H; r++) {
-        float acc = __bfloat162float(B2[r]);
+        float acc = net.b2(r);
 #pragma unroll
-        for (int q = 0; q < H; q++) acc = fmaf(__bfloat162float(W2[r * H + q]), h1[q], acc);
+        for (int q = 0; q < H; q++) acc = fmaf(net.w2(r, q), h1[q], acc);
         h2[r] = fmaxf(acc, 0.f);
     }
-    float out = __bfloat162float(B3[0]);
+    float out = net.b3();
 #pragma unroll
-    for (int q = 0; q < H; q++) out = fmaf(__bfloat162float(W3[q]), h2[q], out);
+    for (int q = 0; q < H; q++) out = fmaf(net.w3(q), h2[q], out);
     return out;
+}
+
+// Offsets of the layers in the flat weight array.
+constexpr int kLearnB1 = kLearnH * kLearnIn, kLearnW2 = kLearnB1 + kLearnH, kLearnB2 = kLearnW2 + kLearnH * kLearnH,
+              kLearnW3 = kLearnB2 + kLearnH, kLearnB3 = kLearnW3 + kLearnH;
+
+struct NetBf16 {   // bf16 weights in global memory
+    const __nv_bfloat16* w;
+    __device__ float w1(int r, int q) const { return __bfloat162float(w[r * kLearnIn + q]); }
+    __device__ float b1(int r) const { return __bfloat162float(w[kLearnB1 + r]); }
+    __device__ float w2(int r, int q) const { return __bfloat162float(w[kLearnW2 + r * kLearnH + q]); }
+    __device__ float b2(int r) const { return __bfloat162float(w[kLearnB2 + r]); }
+    __device__ float w3(int q) const { return __bfloat162float(w[kLearnW3 + q]); }
+    __device__ float b3() const { return __bfloat162float(w[kLearnB3]); }
+};
+
+struct NetF32 {    // weights as floats (shared memory)
+    const float* w;
+    __device__ float w1(int r, int q) const { return w[r * kLearnIn + q]; }
+    __device__ float b1(int r) const { return w[kLearnB1 + r]; }
+    __device__ float w2(int r, int q) const { return w[kLearnW2 + r * kLearnH + q]; }
+    __device__ float b2(int r) const { return w[kLearnB2 + r]; }
+    __device__ float w3(int q) const { return w[kLearnW3 + q]; }
+    __device__ float b3() const { return w[kLearnB3]; }
+};
+
+// Offset predicted by the piece's line, x = key - first key.
+__device__ __forceinline__ float learn_line(const LModel& m, uint32_t j, float x) {
+    return fmaf(__ldg(m.pa + j), x, __ldg(m.pc + j));
+}
+
+// Network input: the key's place in its piece and the piece's embedding.
+__device__ __forceinline__ void learn_input(const LModel& m, uint32_t j, float x, float in[kLearnIn]) {
+    in[0] = fminf(fmaxf(x * __ldg(m.pinv + j), 0.f), 1.f);
+#pragma unroll
+    for (int q = 0; q < 4; q++) in[1 + q] = __bfloat162float(m.emb[(uint64_t)j * 4 + q]);
 }
 
 // Predicted offset of key k from the first position of piece j (the
 // position is j * P plus this, added in integer arithmetic).
 __device__ __forceinline__ float learn_predict(const LModel& m, uint32_t j, uint64_t k) {
-    uint64_t kbj = __ldg(m.kb + j);
-    float x = (float)(k - kbj);
-    float pos = __ldg(m.pc + j) + __ldg(m.pa + j) * x;
+    const float x = (float)(k - __ldg(m.kb + j));
+    float pos = learn_line(m, j, x);
     if (m.hidden > 0 && __ldg(m.use_mlp + j)) {
-        float t = fminf(fmaxf(x * __ldg(m.pinv + j), 0.f), 1.f);
-        pos += (float)m.P * learn_mlp(m, j, t);
+        float in[kLearnIn];
+        learn_input(m, j, x, in);
+        pos = fmaf((float)m.P, learn_net(NetBf16{m.w}, in), pos);
     }
     return pos;
 }

@@ -232,3 +232,34 @@ def test_empty_layer_learned(ctx):
         assert not got.any()
     finally:
         hv.hv_layer_free(L)
+
+
+@pytest.mark.parametrize("n, segments", [(1, 0), (511, 0), (513, 0), (2000, 2000), (2000, 667), (70_001, 3), (5000, 10)])
+def test_bounds_and_lookups_at_piece_borders(ctx, n, segments):
+    """Pieces of one key, of a few, with a short last one, and runs of equal keys
+    across piece borders: lookups are the lower bound for stored keys, their
+    neighbours and both ends, and the reported bound covers every piece's."""
+    rng = np.random.default_rng(n + segments)
+    pts = rng.integers(-2 ** 24, 2 ** 24, (n, 2)).astype(np.int32)
+    if n > 1:
+        pts[n // 3:2 * n // 3] = pts[0]
+    L = hv.hv_layer_load_points(ctx, pts)
+    try:
+        opts = hv.hv_build_opts()
+        opts.learned_segments = segments
+        opts.max_error = 1 << 30
+        hv.hv_layer_build_index(L, hv.HV_INDEX_RTREE | hv.HV_INDEX_LEARNED, opts)
+        info = hv.info_dict(L)
+        assert info["learned_error"] <= info["learned_error_linear"]
+        assert 0 <= info["learned_mean_window"] <= info["learned_mean_window_linear"]
+        assert info["learned_mean_window"] <= info["learned_error"]
+        keys = torch.zeros(n, dtype=torch.int64, device="cuda")
+        hv.hv_layer_keys(L, 0, keys, n)
+        k = keys.cpu().numpy()
+        q = np.unique(np.concatenate([k, k + 1, np.maximum(k - 1, 0), [0, (1 << 62) - 1]]))
+        dq = torch.from_numpy(q).cuda()
+        pos = torch.zeros(len(q), dtype=torch.int64, device="cuda")
+        hv.hv_learned_lookup(L, 0, dq, len(q), pos)
+        assert np.array_equal(pos.cpu().numpy(), np.searchsorted(k, q))
+    finally:
+        hv.hv_layer_free(L)
