@@ -82,12 +82,18 @@ int prepare_polygons(Ctx* c, const int2* d_xy, uint64_t n_vert, const uint64_t* 
 
 namespace {
 
-__global__ void k_check_coords(const int32_t* xy, uint64_t n, uint32_t* bad) {
-    uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (i < n) {
-        int32_t v = xy[i];
-        if (v < -kGridHalf || v > kGridHalf - 1) atomicOr(bad, 1u);
+// Two vertices (16 bytes) per thread; xy starts on an allocation.
+__global__ void k_check_coords(const int2* xy, uint64_t n, uint32_t* bad) {
+    const uint64_t i = 2 * (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x);
+    if (i >= n) return;
+    int4 v;
+    if (i + 1 < n) {
+        v = *(const int4*)(xy + i);
+    } else {
+        const int2 a = xy[i];
+        v = make_int4(a.x, a.y, a.x, a.y);
     }
+    if (min(min(v.x, v.y), min(v.z, v.w)) < -kGridHalf || max(max(v.x, v.y), max(v.z, v.w)) > kGridHalf - 1) atomicOr(bad, 1u);
 }
 
 // Copy `n` vertices (host or device) into a fresh device array and check the
@@ -103,8 +109,7 @@ int upload_vertices(Ctx* c, const int32_t* xy, uint64_t n, int2** out) {
         int rc = dev_alloc(c, (void**)&bad, 4);
         if (rc != HV_OK) { dev_free(c, *out, n * 8); *out = nullptr; return rc; }
         cudaMemset(bad, 0, 4);
-        uint64_t cnt = 2 * n;
-        k_check_coords<<<(unsigned)((cnt + 255) / 256), 256>>>((const int32_t*)*out, cnt, bad);
+        k_check_coords<<<(unsigned)((n + 511) / 512), 256>>>(*out, n, bad);
         uint32_t h = 0;
         e = cudaMemcpy(&h, bad, 4, cudaMemcpyDeviceToHost);
         dev_free(c, bad, 4);

@@ -49,6 +49,18 @@ __global__ void k_keys(const typename O::T* obj, uint64_t n, uint64_t* keys, uin
     idx[i] = (uint32_t)i;
 }
 
+// Keys of points, two per thread (16-byte loads and stores; both arrays start
+// on an allocation).
+__global__ void k_point_keys(const int2* obj, uint64_t n, uint64_t* keys) {
+    const uint64_t i = 2 * (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x);
+    if (i + 1 < n) {
+        const int4 o = *(const int4*)(obj + i);
+        *(ulonglong2*)(keys + i) = make_ulonglong2(hilbert_key(o.x, o.y), hilbert_key(o.z, o.w));
+    } else if (i < n) {
+        keys[i] = hilbert_key(obj[i].x, obj[i].y);
+    }
+}
+
 template <class T>
 __global__ void k_gather(const T* src, const uint32_t* idx, uint64_t n, T* dst) {
     uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
@@ -58,6 +70,22 @@ __global__ void k_gather(const T* src, const uint32_t* idx, uint64_t n, T* dst) 
 __device__ __forceinline__ int4 warp_union(int4 b) {
     return make_int4(__reduce_min_sync(kFull, b.x), __reduce_min_sync(kFull, b.y),
                      __reduce_max_sync(kFull, b.z), __reduce_max_sync(kFull, b.w));
+}
+
+// The points of sorted keys and (if asked for) the boxes of their leaves: one
+// warp per leaf, so that the points are not read again for their boxes.
+__global__ void k_key_points(const uint64_t* keys, uint64_t n, int2* obj, int4* box) {
+    const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    if ((i & ~31ull) >= n) return;
+    int4 b = make_int4(kEmptyLo, kEmptyLo, kEmptyHi, kEmptyHi);
+    if (i < n) {
+        const int2 o = hilbert_point(keys[i]);
+        obj[i] = o;
+        b = PointObj::box(o);
+    }
+    if (box == nullptr) return;
+    b = warp_union(b);
+    if ((i & 31) == 0) box[i >> 5] = b;
 }
 
 // Leaf boxes: one warp per leaf of 32 consecutive objects.
@@ -125,12 +153,12 @@ int sort_objects(Ctx* c, typename O::T** obj, uint64_t n, uint64_t** keys_out, u
     if (rc != HV_OK) { dev_free(c, k_out, n * 8); return rc; }
     k_keys<O><<<grid_for(n, 256), 256>>>(*obj, n, k_in, i_in);
     size_t temp_bytes = 0;
-    cub::DeviceRadixSort::SortPairs(nullptr, temp_bytes, k_in, k_out, i_in, i_out, (int64_t)n, 0, 62);
+    cub::DeviceRadixSort::SortPairs(nullptr, temp_bytes, k_in, k_out, i_in, i_out, (uint32_t)n, 0, 62);
     void* temp;
     rc = tmp.get(&temp, temp_bytes);
     if (rc != HV_OK) { dev_free(c, k_out, n * 8); return rc; }
     cudaError_t e = cub::DeviceRadixSort::SortPairs(temp, temp_bytes, k_in, k_out, i_in, i_out,
-                                                    (int64_t)n, 0, 62);
+                                                    (uint32_t)n, 0, 62);
     if (e != cudaSuccess) {
         dev_free(c, k_out, n * 8);
         set_error("radix sort failed: %s", cudaGetErrorString(e));
@@ -155,9 +183,46 @@ int sort_objects(Ctx* c, typename O::T** obj, uint64_t n, uint64_t** keys_out, u
     return HV_OK;
 }
 
-// Build the inner levels over sorted objects.
+// Sort points by Hilbert key.  A point's key determines the point (the curve
+// visits every grid position once), so the keys alone are sorted, without a
+// permutation and a gather through it, and the points are read off the sorted
+// keys afterwards (k_key_points): *obj is left as room for them.  The sort's
+// second buffer is the points' own array, as wide as the keys; one
+// allocation of n keys is all that grows with n but the sort's counters.
+// If the sort fails the points are gone: *obj is released and set to NULL.
+int sort_points(Ctx* c, int2** obj, uint64_t n, uint64_t** keys_out) {
+    uint64_t* keys;
+    HV_TRY(dev_alloc(c, (void**)&keys, n * 8));
+    Tmp tmp(c);
+    cub::DoubleBuffer<uint64_t> buf(keys, (uint64_t*)*obj);
+    size_t temp_bytes = 0;
+    void* temp = nullptr;
+    cudaError_t e = cub::DeviceRadixSort::SortKeys(nullptr, temp_bytes, buf, (uint32_t)n, 0, 62);
+    int rc = HV_ECUDA;
+    if (e == cudaSuccess)
+        rc = tmp.get(&temp, temp_bytes);
+    else
+        set_error("radix sort failed: %s", cudaGetErrorString(e));
+    if (rc != HV_OK) { dev_free(c, keys, n * 8); return rc; }
+    k_point_keys<<<grid_for((n + 1) / 2, 256), 256>>>(*obj, n, keys);
+    e = cub::DeviceRadixSort::SortKeys(temp, temp_bytes, buf, (uint32_t)n, 0, 62);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) {
+        set_error("radix sort failed: %s", cudaGetErrorString(e));
+        dev_free(c, keys, n * 8);
+        dev_free(c, *obj, n * 8);
+        *obj = nullptr;
+        return HV_ECUDA;
+    }
+    *keys_out = buf.Current();
+    *obj = (int2*)buf.Alternate();
+    return HV_OK;
+}
+
+// Build the inner levels over sorted objects.  point_keys: the sorted keys of a
+// point layer whose points are still to be read off them.
 template <class O>
-int build_levels(Ctx* c, const typename O::T* obj, uint64_t n, Tree* t) {
+int build_levels(Ctx* c, typename O::T* obj, uint64_t n, Tree* t, const uint64_t* point_keys = nullptr) {
     *t = Tree();
     t->view.n_obj = n;
     if (n == 0) return HV_OK;
@@ -180,7 +245,10 @@ int build_levels(Ctx* c, const typename O::T* obj, uint64_t n, Tree* t) {
     HV_TRY(dev_alloc(c, (void**)&t->nodes, total * 512));
     t->nodes_bytes = total * 512;
     t->n_nodes = total;
-    k_leaf_boxes<O><<<grid_for(n_leaf * 32, 256), 256>>>(obj, n, n_leaf, box_a);
+    if (point_keys)
+        k_key_points<<<grid_for(n, 256), 256>>>(point_keys, n, (int2*)obj, box_a);
+    else
+        k_leaf_boxes<O><<<grid_for(n_leaf * 32, 256), 256>>>(obj, n, n_leaf, box_a);
     uint64_t off = 0, n_child = n_leaf;
     for (int l = 1; l <= top; l++) {
         t->view.level_off[l] = off;
@@ -293,31 +361,45 @@ __global__ void k_piece_count(const int4* segs, uint64_t n, int shift, uint32_t*
     cnt[i] = (uint32_t)(m < kMaxPieces ? m : kMaxPieces);
 }
 
-__device__ __forceinline__ int64_t floordiv64(int64_t a, int64_t b) {
-    int64_t q = a / b;
-    return (a % b != 0 && ((a < 0) != (b < 0))) ? q - 1 : q;
-}
+// Positions k d / m, k = 0 .. m, rounded down, one after the other: d = q m + r
+// with 0 <= r < m, each step adds q and carries one whenever the summed
+// remainders pass m.  (|d| < 2^31: coordinates lie in [-2^30, 2^30).)
+struct Steps {
+    int32_t q, r, at, sum;
+    int32_t m;
+    __device__ Steps(int32_t d, int32_t m_) : at(0), sum(0), m(m_) {
+        q = d / m;
+        r = d - q * m;
+        if (r < 0) q--, r += m;
+    }
+    __device__ void next() {
+        at += q;
+        sum += r;
+        if (sum >= m) at++, sum -= m;
+    }
+};
 
 // Piece k of m covers the parameter interval [k/m, (k+1)/m]; along each axis
 // the segment moves monotonically, so the piece lies between its two end
-// positions, rounded outwards to the grid.
+// positions, rounded outwards to the grid.  (With a 64-bit division per
+// end and axis 5M segments took 0.72 ms.)
 __global__ void k_emit_pieces(const int4* segs, uint64_t n, const uint32_t* cnt, const uint64_t* off,
                               Piece* out) {
     uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    int4 s = segs[i];
-    int64_t m = cnt[i];
-    int64_t dx = (int64_t)s.z - s.x, dy = (int64_t)s.w - s.y;
-    uint64_t o = off[i];
-    for (int64_t k = 0; k < m; k++) {
-        int64_t xa = floordiv64(dx * k, m), xb = floordiv64(dx * (k + 1), m);
-        int64_t ya = floordiv64(dy * k, m), yb = floordiv64(dy * (k + 1), m);
+    const int4 s = segs[i];
+    const int32_t m = (int32_t)cnt[i];
+    const uint64_t o = off[i];
+    const int32_t sx0 = min(s.x, s.z), sx1 = max(s.x, s.z), sy0 = min(s.y, s.w), sy1 = max(s.y, s.w);
+    Steps x(s.z - s.x, m), y(s.w - s.y, m);
+    for (int32_t k = 0; k < m; k++) {
+        const int32_t xa = s.x + x.at, ya = s.y + y.at;
+        x.next();
+        y.next();
+        const int32_t xb = s.x + x.at, yb = s.y + y.at;
         // exact positions lie in [floor, floor + 1)
-        int64_t x0 = s.x + (xa < xb ? xa : xb), x1 = s.x + (xa > xb ? xa : xb) + 1;
-        int64_t y0 = s.y + (ya < yb ? ya : yb), y1 = s.y + (ya > yb ? ya : yb) + 1;
-        int4 b = make_int4((int32_t)max(x0, (int64_t)min(s.x, s.z)), (int32_t)max(y0, (int64_t)min(s.y, s.w)),
-                           (int32_t)min(x1, (int64_t)max(s.x, s.z)), (int32_t)min(y1, (int64_t)max(s.y, s.w)));
-        out[o + k] = Piece{s, b};
+        out[o + k] = Piece{s, make_int4(max(min(xa, xb), sx0), max(min(ya, yb), sy0),
+                                        min(max(xa, xb) + 1, sx1), min(max(ya, yb) + 1, sy1))};
     }
 }
 
@@ -377,10 +459,21 @@ void free_tree(Ctx* c, Tree* t) {
 
 int build_tree_points(Layer* L) {
     Ctx* c = L->ctx;
-    if (L->n_obj) {
-        HV_TRY(sort_objects<PointObj>(c, (int2**)&L->obj, L->n_obj, &L->keys, nullptr));
+    const uint64_t n = L->n_obj;
+    if (n) {
+        if (!L->obj) { set_error("the layer lost its points in a failed index build"); return HV_ESTATE; }
+        HV_TRY(sort_points(c, (int2**)&L->obj, n, &L->keys));
     }
-    HV_TRY(build_levels<PointObj>(c, (const int2*)L->obj, L->n_obj, &L->tree));
+    const int rc = build_levels<PointObj>(c, (int2*)L->obj, n, &L->tree, L->keys);
+    if (rc != HV_OK) {
+        // the layer keeps its points (in their order), for another attempt
+        if (n) k_key_points<<<grid_for(n, 256), 256>>>(L->keys, n, (int2*)L->obj, nullptr);
+        cudaDeviceSynchronize();
+        free_tree(c, &L->tree);
+        dev_free(c, L->keys, n * 8);
+        L->keys = nullptr;
+        return rc;
+    }
     HV_CUDA(cudaDeviceSynchronize());
     return HV_OK;
 }
@@ -397,7 +490,7 @@ static int build_piece_tree(Layer* L, const int4* segs, uint64_t n_seg) {
     L->obj_bytes = n * sizeof(Piece);
     L->n_obj = n;
     if (n) HV_TRY(sort_objects<PieceObj>(c, (Piece**)&L->obj, n, &L->keys, nullptr));
-    HV_TRY(build_levels<PieceObj>(c, (const Piece*)L->obj, n, &L->tree));
+    HV_TRY(build_levels<PieceObj>(c, (Piece*)L->obj, n, &L->tree));
     return HV_OK;
 }
 

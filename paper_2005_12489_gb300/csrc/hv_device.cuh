@@ -11,27 +11,73 @@ constexpr int32_t kGridHalf = 1 << 30;
 constexpr int32_t kEmptyLo = 0x7fffffff;          // min-corner of an empty box
 constexpr int32_t kEmptyHi = (int32_t)0x80000000; // max-corner of an empty box
 
+// Interleave with zeros: bit i moves to bit 2 i (and back).
+__host__ __device__ inline uint64_t spread_bits(uint32_t v) {
+    uint64_t x = v;
+    x = (x | (x << 16)) & 0x0000ffff0000ffffull;
+    x = (x | (x << 8)) & 0x00ff00ff00ff00ffull;
+    x = (x | (x << 4)) & 0x0f0f0f0f0f0f0f0full;
+    x = (x | (x << 2)) & 0x3333333333333333ull;
+    return (x | (x << 1)) & 0x5555555555555555ull;
+}
+__host__ __device__ inline uint32_t squeeze_bits(uint64_t x) {
+    x &= 0x5555555555555555ull;
+    x = (x | (x >> 1)) & 0x3333333333333333ull;
+    x = (x | (x >> 2)) & 0x0f0f0f0f0f0f0f0full;
+    x = (x | (x >> 4)) & 0x00ff00ff00ff00ffull;
+    x = (x | (x >> 8)) & 0x0000ffff0000ffffull;
+    return (uint32_t)(x | (x >> 16));
+}
+
 // Hilbert curve index of (x, y) on a 2^31 grid (x, y shifted to [0, 2^31)),
-// the classic quadrant-rotation construction; 62-bit result.
+// the quadrant-rotation curve; 62-bit result.
+//
+// Read top down, level i sees the bits (X, Y) of x and y, exchanged if s and
+// complemented if c: rx = X ^ s (X ^ Y) ^ c, ry likewise; its digit is (3 rx) ^
+// ry, and a digit with ry = 0 flips s, and c too if rx = 1.  Over GF(2) the
+// step from one level's (s, c) to the next's is affine: with X = Y it is s ^ c ^
+// !Y, c; else c ^ !Y, s ^ !Y.  So the states of all levels at once are a prefix
+// composition of the levels' maps (s' = a s ^ b c ^ e, c' = d s ^ g c ^ f), a bit
+// per level and word, in five doubling steps: about 150 instructions where the
+// loop over 31 levels takes 370.
 __host__ __device__ inline uint64_t hilbert_key(int32_t gx, int32_t gy) {
-    uint32_t x = (uint32_t)(gx + kGridHalf);
-    uint32_t y = (uint32_t)(gy + kGridHalf);
-    uint64_t d = 0;
-    for (uint32_t s = 1u << 30; s > 0; s >>= 1) {
-        uint32_t rx = (x & s) ? 1u : 0u;
-        uint32_t ry = (y & s) ? 1u : 0u;
-        d += (uint64_t)s * (uint64_t)s * (uint64_t)((3u * rx) ^ ry);
-        if (ry == 0) {
-            if (rx == 1) {
-                x = ~x;
-                y = ~y;
-            }
-            uint32_t t = x;
-            x = y;
-            y = t;
-        }
+    // level 30 in bit 31
+    const uint32_t X = (uint32_t)(gx + kGridHalf) << 1, Y = (uint32_t)(gy + kGridHalf) << 1;
+    const uint32_t q = X ^ Y, n = ~Y;
+    // the map of the level above (the top one's is the identity)
+    uint32_t a = (~q >> 1) | 0x80000000u, b = ~0u >> 1, e = n >> 1;
+    uint32_t d = q >> 1, g = (~q >> 1) | 0x80000000u, f = (n & q) >> 1;
+#pragma unroll
+    for (int k = 1; k < 32; k <<= 1) {
+        const uint32_t top = ~(~0u >> k);
+        const uint32_t a2 = (a >> k) | top, b2 = b >> k, e2 = e >> k;
+        const uint32_t d2 = d >> k, g2 = (g >> k) | top, f2 = f >> k;
+        const uint32_t na = (a & a2) ^ (b & d2), nb = (a & b2) ^ (b & g2), ne = (a & e2) ^ (b & f2) ^ e;
+        const uint32_t nd = (d & a2) ^ (g & d2), ng = (d & b2) ^ (g & g2), nf = (d & e2) ^ (g & f2) ^ f;
+        a = na, b = nb, e = ne, d = nd, g = ng, f = nf;
     }
-    return d;
+    // from s = c = 0 above the top level the state is (e, f)
+    const uint32_t flip = (q & e) ^ f, rx = X ^ flip, ry = Y ^ flip;
+    return (spread_bits(rx >> 1) << 1) | spread_bits((rx ^ ry) >> 1);
+}
+
+// The grid point of a Hilbert index.  The digits give every level's flips of s
+// and c directly, so the states are two prefix XORs.
+__host__ __device__ inline int2 hilbert_point(uint64_t key) {
+    const uint32_t rx = squeeze_bits(key >> 1), ry = rx ^ squeeze_bits(key);
+    uint32_t s = ~ry & 0x7fffffffu, c = s & rx;
+    s >>= 1;
+    c >>= 1;
+#pragma unroll
+    for (int k = 1; k < 32; k <<= 1) {
+        s ^= s >> k;
+        c ^= c >> k;
+    }
+    const uint32_t u = rx ^ c, v = ry ^ c, w = (u ^ v) & s;
+    int2 p;
+    p.x = (int32_t)(u ^ w) - kGridHalf;
+    p.y = (int32_t)(v ^ w) - kGridHalf;
+    return p;
 }
 
 // Centre of a box, rounded down, computed without overflow.
