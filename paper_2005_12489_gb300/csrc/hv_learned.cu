@@ -24,6 +24,21 @@ constexpr int kBatch = 1 << 16;
 
 uint32_t blocks_for(uint64_t n, int t) { return (uint32_t)((n + t - 1) / t); }
 
+// A launch that may start before the grid ahead of it in the stream has ended
+// (it waits in the kernel).
+template <class... P, class... A>
+cudaError_t launch_early(void (*kernel)(P...), uint32_t blocks, uint32_t threads, A... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 struct Alloc {
     Learned* l;
     Ctx* c;
@@ -128,6 +143,13 @@ __device__ __forceinline__ uint32_t piece_of(const LModel& m, uint64_t i, uint64
 // are read from shared memory, the sample's values stay in registers.
 // (65,536 samples took 123 us by warp reductions with the activations in local
 // memory.)
+//
+// The two launches of a step start early (programmatic dependent launches):
+// each lets the next grid in at once and waits for the one before where it first
+// needs its results.  Drawing the sample and the line's residual -- dependent
+// random reads that no step changes -- then runs under the previous step's
+// kernels, and the launches themselves cost no gap.  Every thread waits before
+// it ends, so a grid that has waited follows all that came before it.
 constexpr int kTrainThreads = 128;
 constexpr int kRowIn = 0, kRowH1 = kRowIn + kLearnIn, kRowD1 = kRowH1 + kLearnH, kRowH2 = kRowD1 + kLearnH,
               kRowD2 = kRowH2 + kLearnH, kRowDo = kRowD2 + kLearnH, kRowOne = kRowDo + 1, kRows = kRowOne + 1;
@@ -141,7 +163,7 @@ __global__ void __launch_bounds__(kTrainThreads, 4) k_train(LModel m, const floa
     __shared__ __align__(16) float rows[kRows * kRowStride];
     __shared__ __align__(16) float sw[kLearnNW];
     const int tid = threadIdx.x;
-    for (int i = tid; i < kLearnNW; i += kTrainThreads) sw[i] = w[i];
+    cudaTriggerProgrammaticLaunchCompletion();
     uint64_t gid = blockIdx.x * (uint64_t)blockDim.x + tid;
     uint64_t h = ((uint64_t)seed << 32) ^ ((uint64_t)step * 0x9E3779B97F4A7C15ull) ^ (gid * 0xD1B54A32D192ED03ull);
     h ^= h >> 31; h *= 0x94D049BB133111EBull; h ^= h >> 29;
@@ -152,6 +174,8 @@ __global__ void __launch_bounds__(kTrainThreads, 4) k_train(LModel m, const floa
     const float target = ((float)((double)i - (double)j * m.P) - learn_line(m, j, x)) / (float)m.P;
     float in[kLearnIn];
     in[0] = fminf(fmaxf(x * m.pinv[j], 0.f), 1.f);
+    cudaGridDependencySynchronize();   // from here on: the weights of the previous step
+    for (int q = tid; q < kLearnNW; q += kTrainThreads) sw[q] = w[q];
     const float4 e4 = *(const float4*)(emb + (uint64_t)j * 4);
     in[1] = e4.x, in[2] = e4.y, in[3] = e4.z, in[4] = e4.w;
     __syncthreads();
@@ -247,6 +271,8 @@ __global__ void __launch_bounds__(kTrainThreads, 4) k_train(LModel m, const floa
 // SGD on the embeddings, in one launch.
 __global__ void k_update(float* w, float* g, float* mo, float* ve, int step, float lr, float* emb, float* gemb,
                          uint64_t n_emb, float lr_emb) {
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
     uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     if (i < (uint64_t)kLearnNW) {
         const float b1 = 0.9f, b2 = 0.999f;
@@ -527,9 +553,10 @@ static int build_one(Ctx* c, Learned* L, const uint64_t* keys, uint64_t n, const
         LModel tm = m;
         tm.hidden = H;
         for (int s = 0; s < steps; s++) {
-            k_train<<<kBatch / kTrainThreads, kTrainThreads>>>(tm, w, emb, gw, gemb, s, seed);
-            k_update<<<blocks_for(nw + (uint64_t)n_seg * 4, 256), 256>>>(w, gw, mo, ve, s, 2e-3f, emb, gemb,
-                                                                         (uint64_t)n_seg * 4, 0.02f);
+            HV_CUDA(launch_early(k_train, kBatch / kTrainThreads, kTrainThreads, tm, (const float*)w, (const float*)emb,
+                                 gw, gemb, s, seed));
+            HV_CUDA(launch_early(k_update, blocks_for(nw + (uint64_t)n_seg * 4, 256), 256, w, gw, mo, ve, s, 2e-3f, emb,
+                                 gemb, (uint64_t)n_seg * 4, 0.02f));
         }
         k_to_bf16<<<blocks_for(nw, 256), 256>>>(w, wb, nw);
         k_to_bf16<<<blocks_for((uint64_t)n_seg * 4, 256), 256>>>(emb, embb, (uint64_t)n_seg * 4);
