@@ -282,7 +282,7 @@ __device__ void cull(const Params& p, const TreeArg& t, bool fill, Front& sm, in
 // sorted order), find each cell's position range through the learned model,
 // and turn the ranges into R-tree subtrees at the finest level whose entries
 // fit the frontier.  Every object whose centre lies in the box is under one of
-// the entries; the blocks then proceed exactly as after the R-tree cull.
+// the entries; the sweep then proceeds exactly as after the R-tree cull.
 __device__ void learned_cull(const Params& p, const TreeArg& t, const LModel& m, int32_t halo, Front& sm,
                              int32_t bx0, int32_t by0, int32_t bx1, int32_t by1, int tid) {
     __shared__ unsigned long long cnt[kMaxLevels + 1];
@@ -624,14 +624,21 @@ int launch_render(Layer* L, const hv_tile_req* d_reqs, uint32_t n, int mode, int
         p.phases = (unsigned long long*)log->phases;
     }
     const bool prof = p.phases != nullptr;
-    // strip height: 16 rows (16 CTAs per tile) when the batch fills the GPU,
-    // 8 or 4 rows for small batches so that a few tiles still spread over
-    // many SMs (lower latency)
+    // Strip height: 16 rows (16 CTAs per tile) when the batch fills the GPU, 8 or
+    // 4 rows for small batches so that the densest strips, which end last, are
+    // shared over more SMs.  Smaller strips repeat the cull.  Measured at z 8-14 on
+    // three layers each: points and polygons gain from 8 rows up to 151 tiles
+    // (90 tiles: 117 -> 99 us and 208 -> 174 us; 250 tiles would lose: 177 -> 191
+    // us for points), points from 4 rows up to 75 tiles (45 tiles: 75 -> 68 us), polygons
+    // only up to 37 (60 tiles: 150 -> 175 us).  Segments, whose strips cost
+    // little more than their cull, change at 76 and 38 tiles (60 tiles in 4 rows:
+    // 18 -> 27 us).
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const uint64_t resident = (uint64_t)sms * 4;
-    p.rows = (uint64_t)n * 16 >= 2 * resident ? 16 : ((uint64_t)n * 32 >= 2 * resident ? 8 : 4);
+    const uint64_t few16 = (L->kind == HV_LAYER_LINES ? 2 : 4) * resident, few8 = (L->kind == HV_LAYER_POINTS ? 4 : 2) * resident;
+    p.rows = (uint64_t)n * 16 >= few16 ? 16 : ((uint64_t)n * 32 >= few8 ? 8 : 4);
     p.strips = kTile / p.rows;
     // batches too small for the GPU even in 4-row strips also split each
     // strip into 2 or 4 column parts (a CTA per 128 or 64 columns)
