@@ -17,13 +17,13 @@
 // instructions per tile where the 8 x 4 block traversal took 5.7 M: 4,000
 // tiles 23.5 -> 11.8 ms; 341 tiles of 100,000 points at zoom 0-4, 1 px, MASK
 // 414 -> 73 us; one tile of 10M points 35 -> 29 us.  Segments: 4,000 tiles of 50M
-// segments at 1 px 19.7 -> 5.9 ms; the outlines of 1,000 tiles of 2M polygons
+// segments at 1 px 19.7 -> 5.6 ms; the outlines of 1,000 tiles of 2M polygons
 // 12 -> 8.5 ms (dense low-zoom tiles: 390 leaves of short edges per strip, 22
 // pieces and 71 (piece, row) pairs each).
 //
 // The fill draws polygon by polygon: one pass over a polygon's edges gives every
 // crossing of the strip's rows, and a parity scan per row the filled samples.
-// 1,000 tiles of 2M polygons: the fill launch 3.5 -> 1.3 ms, both 12.4 -> 10.5
+// 1,000 tiles of 2M polygons: the fill launch 3.5 -> 1.3 ms, both 12.4 -> 10.0
 // ms; 33 tiles with anti-aliased pattern fill 525 -> 360 us.
 //
 // Included by hv_render.cu (one translation unit with the cull).
@@ -43,8 +43,44 @@ struct SweepSmem : Front {
     int32_t reach[64];
     uint32_t stk_node[kWarps][kMaxLevels + 1];
     uint32_t stk_mask[kWarps][kMaxLevels + 1];
+    // per warp, what the (piece, row) or (edge, row) pairs of 32 objects share
+    float4 pair_obj[kWarps][kKind == HV_LAYER_POINTS ? 1 : (kKind == kPolyFill ? 32 : 64)];
+    int pair_row[kWarps][kKind == HV_LAYER_POINTS ? 1 : 32];
     int next_entry;
 };
+
+// Pairs (object, row) of a warp, numbered through over the objects that have
+// rows: `start` is the lane's first pair.  The objects lie in shared memory in order,
+// those without rows left out, so that a pair's object is the number of starts up to it: in
+// each round of 32 pairs one OR over the lanes marks the starts in it and the
+// bits up to the lane's own are counted.  (A binary search over the starts with
+// shuffles, and the object's fields by shuffles as well, took 15 shuffles a round
+// and held the fields in registers, spilling 96 bytes in the outline launch
+// against 52: 4,000 tiles of 50M segments 5.84 ms against 5.57, 1,000 tiles of
+// 2M polygons 10.38 ms against 9.96.)
+struct PairRounds {
+    int start, before;
+    bool some;
+    __device__ PairRounds(int start_, int count) : start(start_), before(0), some(count > 0) {}
+    // the object of pair base + lane, base = 0, 32, ..
+    __device__ __forceinline__ int object(int base, int lane) {
+        const int at = start - base;
+        const uint32_t marks = __reduce_or_sync(kFull, some && (uint32_t)at < 32u ? 1u << at : 0u);
+        const int k = before + __popc(marks & ((2u << lane) - 1u)) - 1;
+        before += __popc(marks);
+        return k;
+    }
+};
+
+// Inclusive prefix sum over the lanes.
+__device__ __forceinline__ int lane_sums(int v, int lane) {
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int u = __shfl_up_sync(kFull, v, d);
+        if (lane >= d) v += u;
+    }
+    return v;
+}
 
 // The CTA's samples: (i, j) lies at (xc + (i - hw) h, yc + (j - hh) h), h = 2^s.
 // Objects are taken relative to (xc, yc), the strip's middle, so that every
@@ -437,11 +473,10 @@ __device__ __forceinline__ void draw_row(uint32_t* bits, const Lattice& g, const
 
 // A segment leaf: 32 pieces, each with a run of open rows that it reaches.
 // The (piece, row) pairs are numbered through by a prefix sum over the lanes
-// and the lanes take them in turn (each finds its piece by a binary search
-// over the sums), so a leaf costs ceil(pairs / 32) rounds whatever the pieces'
-// heights.
-__device__ __forceinline__ void draw_segments(const Params& p, const Src& src, uint32_t* bits, const Lattice& g,
-                                              uint32_t leaf, uint32_t rows, int lane) {
+// and the lanes take them in turn, so a leaf costs ceil(pairs / 32) rounds
+// whatever the pieces' heights.
+__device__ __forceinline__ void draw_segments(const Params& p, const Src& src, uint32_t* bits, float4* pair_obj,
+                                              int* pair_row, const Lattice& g, uint32_t leaf, uint32_t rows, int lane) {
     const uint64_t i = (uint64_t)leaf * 32 + lane;
     int4 o = make_int4(0, 0, 0, 0), pb = make_int4(kEmptyLo, kEmptyLo, kEmptyHi, kEmptyHi);
     const int4* rec = (const int4*)src.obj + 2 * i;
@@ -454,33 +489,30 @@ __device__ __forceinline__ void draw_segments(const Params& p, const Src& src, u
     const int clo = max(g.hw - ((g.R - x0) >> g.s), 0), chi = min(((x1 + g.R) >> g.s) + g.hw, 2 * g.hw - 1);
     uint32_t mine = 0u;
     if (i < src.n && r0 <= r1 && clo <= chi) mine = rows & (~0u << r0) & (~0u >> (31 - r1));
+    const uint32_t some = __ballot_sync(kFull, mine != 0u);
+    if (some == 0u) return;
     // from the first to the last open row
     const int first = __ffs(mine) - 1, count = mine ? 32 - __clz(mine) - first : 0;
-    int sum = count;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int v = __shfl_up_sync(kFull, sum, d);
-        if (lane >= d) sum += v;
+    const int sum = lane_sums(count, lane), total = __shfl_sync(kFull, sum, 31), start = sum - count;
+    if (count) {
+        const PieceRow q = piece_row(g, o, x0, y0, x1, y1, clo, chi);
+        const int k = __popc(some & ((1u << lane) - 1u));
+        pair_obj[2 * k] = make_float4(q.mx, q.my, q.c0, q.E);
+        pair_obj[2 * k + 1] = make_float4(q.ta, q.tb, __uint_as_float(q.at), __uint_as_float(q.span));
+        pair_row[k] = (first - start) * 32 + lane;   // a pair's row less its number, and the piece
     }
-    const int total = __shfl_sync(kFull, sum, 31);
-    if (total == 0) return;
-    const PieceRow own = piece_row(g, o, x0, y0, x1, y1, clo, chi);
-    const int start = sum - count;   // the lane's first pair
+    __syncwarp();
+    PairRounds rounds(start, count);
     for (int base = 0; base < total; base += 32) {
-        const int j = base + lane;
-        // the last piece that starts at or before pair j (pieces without rows
-        // start where the next one does)
-        int k = 0;
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1)
-            if (__shfl_sync(kFull, start, k + d) <= j) k += d;
-        const int r = __shfl_sync(kFull, first, k) + j - __shfl_sync(kFull, start, k);
-        PieceRow q;
-        q.mx = __shfl_sync(kFull, own.mx, k), q.my = __shfl_sync(kFull, own.my, k);
-        q.c0 = __shfl_sync(kFull, own.c0, k), q.E = __shfl_sync(kFull, own.E, k);
-        q.ta = __shfl_sync(kFull, own.ta, k), q.tb = __shfl_sync(kFull, own.tb, k);
-        q.at = __shfl_sync(kFull, own.at, k), q.span = __shfl_sync(kFull, own.span, k);
-        if (j < total) draw_row(bits, g, q, (const int4*)src.obj + 2 * ((uint64_t)leaf * 32 + k), r);
+        const int k = rounds.object(base, lane), j = base + lane;
+        if (j < total) {
+            const float4 u = pair_obj[2 * k], v = pair_obj[2 * k + 1];
+            const int at = pair_row[k];
+            PieceRow q;
+            q.mx = u.x, q.my = u.y, q.c0 = u.z, q.E = u.w;
+            q.ta = v.x, q.tb = v.y, q.at = __float_as_uint(v.z), q.span = __float_as_uint(v.w);
+            draw_row(bits, g, q, (const int4*)src.obj + 2 * ((uint64_t)leaf * 32 + (at & 31)), (at >> 5) + j);
+        }
         __syncwarp();
     }
 }
@@ -515,8 +547,8 @@ __device__ __forceinline__ int crossing_end(const Lattice& g, int32_t lx, int32_
 // for the whole row.  Edges are taken 32 at a time, their (edge, row) pairs
 // shared over the lanes as for segments; then a lane per row turns the bits
 // into filled samples and clears them.
-__device__ __forceinline__ void fill_polygon(const Params& p, uint32_t* bits, uint32_t* cross, const Lattice& g,
-                                             uint64_t e0, uint64_t e1, int clo, int chi, uint32_t rows, int lane) {
+__device__ __forceinline__ void fill_polygon(const Params& p, uint32_t* bits, uint32_t* cross, int4* pair_obj,
+                                             int* pair_row, const Lattice& g, uint64_t e0, uint64_t e1, int clo, int chi, uint32_t rows, int lane) {
     const int rf = __ffs(rows) - 1, rl = 31 - __clz(rows);
     for (uint64_t base = e0; base < e1; base += 32) {
         int4 e = make_int4(0, 0, 0, 0);   // a level edge straddles no row
@@ -526,27 +558,26 @@ __device__ __forceinline__ void fill_polygon(const Params& p, uint32_t* bits, ui
         // rows with ly <= y < hy
         const int r0 = max(g.hh - ((-ly) >> g.s), rf), r1 = min(g.hh - ((-hy) >> g.s) - 1, rl);
         const int count = max(r1 - r0 + 1, 0);
-        int sum = count;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int v = __shfl_up_sync(kFull, sum, d);
-            if (lane >= d) sum += v;
+        const uint32_t some = __ballot_sync(kFull, count > 0);
+        if (some == 0u) continue;
+        const int sum = lane_sums(count, lane), total = __shfl_sync(kFull, sum, 31), start = sum - count;
+        if (count) {
+            const int k = __popc(some & ((1u << lane) - 1u));
+            pair_obj[k] = make_int4(lx, ly, ex, ey);
+            pair_row[k] = r0 - start;
         }
-        const int total = __shfl_sync(kFull, sum, 31), start = sum - count;
+        __syncwarp();
+        PairRounds rounds(start, count);
         for (int first = 0; first < total; first += 32) {
-            const int j = first + lane;
-            int k = 0;
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1)
-                if (__shfl_sync(kFull, start, k + d) <= j) k += d;
-            const int r = __shfl_sync(kFull, r0, k) + j - __shfl_sync(kFull, start, k);
-            const int32_t klx = __shfl_sync(kFull, lx, k), kly = __shfl_sync(kFull, ly, k);
-            const int32_t kex = __shfl_sync(kFull, ex, k), key = __shfl_sync(kFull, ey, k);
+            const int k = rounds.object(first, lane), j = first + lane;
             if (j < total) {
-                const int t = crossing_end(g, klx, kly, kex, key, (r - g.hh) * (1 << g.s), clo, chi + 1);
+                const int4 o = pair_obj[k];
+                const int r = pair_row[k] + j;
+                const int t = crossing_end(g, o.x, o.y, o.z, o.w, (r - g.hh) * (1 << g.s), clo, chi + 1);
                 if (t > clo) atomicXor(cross + r * kBitStride + (t >> 5), 1u << (t & 31));
             }
         }
+        __syncwarp();
     }
     __syncwarp();
     if (lane >= rf && lane <= rl) {
@@ -574,7 +605,7 @@ __device__ __forceinline__ void fill_polygon(const Params& p, uint32_t* bits, ui
 
 // A leaf of the polygon-box tree: the polygons whose box holds an open sample.
 __device__ __forceinline__ void fill_polygons(const Params& p, const Src& src, uint32_t* bits, uint32_t* cross,
-                                              const int32_t* reach, const Lattice& g, uint32_t leaf, uint32_t rows,
+                                              int4* pair_obj, int* pair_row, const int32_t* reach, const Lattice& g, uint32_t leaf, uint32_t rows,
                                               int lane) {
     const uint64_t i = (uint64_t)leaf * 32 + lane;
     int4 b = make_int4(kEmptyLo, kEmptyLo, kEmptyHi, kEmptyHi);
@@ -603,7 +634,7 @@ __device__ __forceinline__ void fill_polygons(const Params& p, const Src& src, u
             continue;
         }
         const int clo = max(g.hw - ((-kx0) >> g.s), 0), chi = min((kx1 >> g.s) + g.hw, 2 * g.hw - 1);
-        fill_polygon(p, bits, cross, g, e0, e1, clo, chi, open, lane);
+        fill_polygon(p, bits, cross, pair_obj, pair_row, g, e0, e1, clo, chi, open, lane);
     }
 }
 
@@ -643,9 +674,9 @@ __device__ __forceinline__ void sweep_entry(const Params& p, SweepSmem<kKind>& s
             log_read(p, kKind == kPolyFill ? kLogPolyLeaf : kLogLeaf, node, lane);
             t0 = tick<kProf>();
             if constexpr (kKind == kPolyFill)
-                fill_polygons(p, src, sm.bits, sm.cross[warp], sm.reach, g, node, rows, lane);
+                fill_polygons(p, src, sm.bits, sm.cross[warp], (int4*)sm.pair_obj[warp], sm.pair_row[warp], sm.reach, g, node, rows, lane);
             else
-                draw_segments(p, src, sm.bits, g, node, rows, lane);
+                draw_segments(p, src, sm.bits, sm.pair_obj[warp], sm.pair_row[warp], g, node, rows, lane);
         } else if (lvl == 0) {
             log_read(p, kLogLeaf, node, lane);
             t0 = tick<kProf>();
