@@ -11,7 +11,7 @@
 //
 // Work decomposition.  One CTA (8 warps) renders a strip of 256 x rows pixels
 // of one tile (rows = 16 for large batches, 8 or 4 for small ones; batches
-// too small to fill the GPU even then split each 4-row strip into 2 or 4
+// too small to fill the GPU even then split each 4-row strip into 2, 4 or 8
 // column parts, one CTA each).  The CTA first culls the R-tree (or, with the
 // learned index, the subtrees of the key ranges the model finds) against the
 // strip's box expanded by R, breadth first, into a frontier of at most kFCap
@@ -57,7 +57,7 @@ struct Params {
     uint32_t n;
     int rows;                   // pixel rows per CTA strip: 4, 8 or 16
     int strips;                 // strips per tile (256 / rows)
-    int cols;                   // pixel columns per CTA: 256, or 128 / 64 for batches too small to fill the GPU
+    int cols;                   // pixel columns per CTA: 256, or 128 / 64 / 32 for batches too small to fill the GPU
     int parts;                  // CTAs per strip (256 / cols)
     const uint32_t* n_dev;      // if set, the batch size is min(*n_dev, n) (graph launches)
     int mode;
@@ -641,10 +641,14 @@ int launch_render(Layer* L, const hv_tile_req* d_reqs, uint32_t n, int mode, int
     p.rows = (uint64_t)n * 16 >= few16 ? 16 : ((uint64_t)n * 32 >= few8 ? 8 : 4);
     p.strips = kTile / p.rows;
     // batches too small for the GPU even in 4-row strips also split each
-    // strip into 2 or 4 column parts (a CTA per 128 or 64 columns)
+    // strip into 2, 4 or 8 column parts (a CTA per 128, 64 or 32 columns), as
+    // long as every CTA is resident at once: a tile's densest part decides its
+    // time.  36 single tiles of 10M points: 933 us in all with at most 4 parts, 776
+    // with 8; of 200,000 polygons 1,852 -> 1,665; of 5M segments 467 -> 472.  Twice as
+    // many CTAs (8 parts for two tiles) made sparse tiles slower (6.4 -> 9.2 us).
     p.parts = 1;
     if (p.rows == 4 && !prof)
-        while (p.parts < 4 && (uint64_t)n * p.strips * p.parts * 2 <= resident) p.parts *= 2;
+        while (p.parts < 8 && (uint64_t)n * p.strips * p.parts * 2 <= resident) p.parts *= 2;
     p.cols = kTile / p.parts;
     uint64_t grid = (uint64_t)n * p.strips * p.parts;
     if (grid > 0x7fffffffull) {
