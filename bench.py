@@ -464,7 +464,7 @@ def _roofline(alg, n, ms, cfg, full_size, launch_ms=None):
     achieved = alg["per_tile"] * n / (ms / 1000.0) / 1e9
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": measured_traffic(cfg) if full_size else None, "peak_kind": peak_kind,
-            "kernel": "k_render", "alg_bytes_per_tile": alg["per_tile"], "alg_detail": alg}
+            "kernel": "k_sweep", "alg_bytes_per_tile": alg["per_tile"], "alg_detail": alg}
 
 
 def _roofline_issue(cfg, ms, full_size):
@@ -805,7 +805,7 @@ def serving_block(args):
     hb = dev["points"]["hbm_GBps"]
     roof = None if hb is None else {"bound": "hbm", "achieved": hb, "peak": peak, "unit": "GB/s",
                                     "frac": hb / peak, "traffic": None, "peak_kind": peak_kind,
-                                    "kernel": "k_render (points, batches of 64 trace tiles)",
+                                    "kernel": "k_sweep (points, batches of 64 trace tiles)",
                                     "alg_bytes_per_tile": dev["points"]["alg_bytes_per_tile"]}
     # the oracle on one trace tile of each layer over the whole layers
     cpu = None
