@@ -813,18 +813,20 @@ __device__ __forceinline__ uint32_t pixel_count(uint32_t top, uint32_t bottom, i
     return (uint32_t)(__popc((top >> (2 * q)) & 3u) + __popc((bottom >> (2 * q)) & 3u));
 }
 
-// CTAs per SM.  Points: six, 11.5 ms for 4,000 tiles of 100M points against 11.9
+// CTAs per SM.  Points: six, 11.0 ms for 4,000 tiles of 100M points against 11.4
 // with five and 12.6 with four (40 registers with a small spill; the dependent
-// steps of a row leave issue slots that more warps fill).  Segments: four, 24
-// tiles of 5M segments 68 us, 1,000 polygon tiles 12.0 ms, against 72 us and
-// 12.4 ms with five (4,000 line tiles 5.9 against 5.7 ms).
-template <int kKind>
+// steps of a row leave issue slots that more warps fill); in column parts, where
+// a grid is resident at four per SM, five: one tile 17.2 against 18.0 us.
+// Segments, outlines and fill: four; with five for segments and outlines 1,000
+// polygon tiles 10.3 against 9.7 ms, 33 styled ones 361 against 341 us, 4,000
+// line tiles 5.55 ms with either.
+template <int kKind, bool kSplit>
 struct SweepTraits {
-    static constexpr int kPerSM = kKind == HV_LAYER_POINTS ? 6 : 4;
+    static constexpr int kPerSM = kKind == HV_LAYER_POINTS ? (kSplit ? 5 : 6) : 4;
 };
 
 template <int kKind, bool kProf, bool kSplit>
-__global__ void __launch_bounds__(kThreads, SweepTraits<kKind>::kPerSM) k_sweep(const Params p) {
+__global__ void __launch_bounds__(kThreads, SweepTraits<kKind, kSplit>::kPerSM) k_sweep(const Params p) {
     __shared__ SweepSmem<kKind> sm;
     const int tid = threadIdx.x;
     const long long t_start = tick<kProf>();
