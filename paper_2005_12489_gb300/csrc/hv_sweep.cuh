@@ -442,8 +442,11 @@ __device__ __noinline__ void draw_row_slow(uint32_t* bits, const Lattice& g, con
 // Set the samples of row r within R of the segment.  Where both discs meet the
 // row well inside (half-chords w with w^2 >= 8 R E), a distance error of E
 // moves an end by E R / w, and by at most an eighth more for the curvature:
-// a column nearer to the end than 1.25 E R / w takes the exact test, every
-// other column is decided by its side of the end.
+// a column nearer to the end than e = 1.25 E R / w takes the exact test, every
+// other column is decided by its side of the end.  One column at most is that
+// near only while e < 1/2, that is w^2 > 6.25 (R E)^2, which the first condition
+// implies for R up to about 200 spacings (every radius in pixels); rows of larger
+// ground radii where e may reach 1/2 go to draw_row_slow, which tests them all.
 __device__ __forceinline__ void draw_row(uint32_t* bits, const Lattice& g, const PieceRow& q, const int4* seg, int r) {
     const int col = (int)(q.at & 0xffffu) - 1024, row = (int)(q.at >> 16) - 1024;
     const float rho = (float)g.R * __int_as_float((127 - g.s) << 23);
@@ -452,7 +455,7 @@ __device__ __forceinline__ void draw_row(uint32_t* bits, const Lattice& g, const
     const float tl = fminf(fmaxf((ym - rm) * inv, q.ta), q.tb), tr = fminf(fmaxf((ym + rm) * inv, q.ta), q.tb);
     const float dl = fmaf(-tl, q.my, ym), dr = fmaf(-tr, q.my, ym);
     const float al = fmaf(-dl, dl, r2), ar = fmaf(-dr, dr, r2);
-    if (!(fminf(al, ar) >= 8.f * rE) || q.E >= rho) {
+    if (!(fminf(al, ar) >= rE * fmaxf(8.f, 6.5f * rE)) || q.E >= rho) {
         // beyond R + E of the row both half-chords are imaginary
         if (!(fmaxf(al, ar) < -8.f * rE - 2.f * q.E * q.E)) draw_row_slow(bits, g, q, seg, r);
         return;

@@ -1,0 +1,120 @@
+"""Segment rows of the strip sweep at every ratio of radius to sample spacing
+(ground radii at street zooms reach 2^26 spacings): the kernel's own piece_row
+and draw_row, compiled for the host, against the 128-bit predicate on every
+column in reach, for pieces whose capsule passes within a few units, or a few
+spacings, of a sample of the strip, at every slope, with contacts at the
+segment's inside and at its ends."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import sweep_host
+
+ENTRIES = r"""
+static bool inside(int4 o, int64_t x, int64_t y, int64_t R) {   // the definition, in 128 bits
+    typedef __int128 W;
+    const W dx = (int64_t)o.z - o.x, dy = (int64_t)o.w - o.y, wx = x - o.x, wy = y - o.y, R2 = (W)R * R;
+    const W t = wx * dx + wy * dy, L = dx * dx + dy * dy;
+    if (t <= 0) return wx * wx + wy * wy <= R2;
+    if (t >= L) return (W)(x - o.z) * (x - o.z) + (W)(y - o.w) * (y - o.w) <= R2;
+    const W c = wx * dy - wy * dx;                               // |c| < 2^64, L < 2^63, R2 < 2^59
+    const unsigned __int128 a = (unsigned __int128)(c < 0 ? -c : c);
+    return a < ((unsigned __int128)1 << 64) && a * a <= (unsigned __int128)R2 * (unsigned __int128)L;
+}
+static int64_t fdiv(int64_t a, int64_t b) { return a / b - (a % b != 0 && (a < 0) != (b < 0)); }
+// the box of piece k of m, as the index build forms it
+static int4 piece_box(int4 s, int64_t k, int64_t m) {
+    const int64_t dx = (int64_t)s.z - s.x, dy = (int64_t)s.w - s.y;
+    const int64_t xa = s.x + fdiv(dx * k, m), xb = s.x + fdiv(dx * (k + 1), m);
+    const int64_t ya = s.y + fdiv(dy * k, m), yb = s.y + fdiv(dy * (k + 1), m);
+    return make_int4((int)max(min(xa, xb), (int64_t)min(s.x, s.z)), (int)max(min(ya, yb), (int64_t)min(s.y, s.w)),
+                     (int)min(max(xa, xb) + 1, (int64_t)max(s.x, s.z)), (int)min(max(ya, yb) + 1, (int64_t)max(s.y, s.w)));
+}
+struct Result { int64_t wrong, columns, covered, rows; };
+// the rows of one piece, at most `most` of them
+static void compare(const Lattice& g, int4 o, int4 pb, int most, std::mt19937_64& rng, Result* res) {
+    const int32_t x0 = rel32(pb.x, g.xc), y0 = rel32(pb.y, g.yc), x1 = rel32(pb.z, g.xc), y1 = rel32(pb.w, g.yc);
+    const int r0 = max(g.hh - ((g.R - y0) >> g.s), 0), r1 = min(((y1 + g.R) >> g.s) + g.hh, 2 * g.hh - 1);
+    const int clo = max(g.hw - ((g.R - x0) >> g.s), 0), chi = min(((x1 + g.R) >> g.s) + g.hw, 2 * g.hw - 1);
+    if (r0 > r1 || clo > chi) return;
+    const PieceRow q = piece_row(g, o, x0, y0, x1, y1, clo, chi);
+    for (int n = 0; n < most && n <= r1 - r0; n++) {
+        const int r = r1 - r0 < most ? r0 + n : r0 + (int)(rng() % (uint64_t)(r1 - r0 + 1));
+        uint32_t bits[kSampleRows * kBitStride] = {};
+        draw_row(bits, g, q, &o, r);
+        for (int c = 0; c < 2 * g.hw; c++) {
+            const bool got = (bits[r * kBitStride + (c >> 5)] >> (c & 31)) & 1u;
+            const bool want = c >= clo && c <= chi &&
+                              inside(o, (int64_t)g.xc + (int64_t)(c - g.hw) * (1 << g.s), (int64_t)g.yc + (int64_t)(r - g.hh) * (1 << g.s), g.R);
+            res->wrong += got != want;
+            res->covered += want;
+        }
+        res->columns += 2 * g.hw;
+        res->rows++;
+    }
+}
+static Lattice lattice(int s, int hw, int hh, int32_t xc, int32_t yc, int32_t R) {
+    Lattice g;
+    g.s = s, g.hw = hw, g.hh = hh, g.xc = xc, g.yc = yc, g.R = R, g.R2 = (int64_t)R * R;
+    g.rs = max(32 - __clz(R) - 6, 0), g.narrow = R <= kNarrow;
+    return g;
+}
+// radii of 2^lo .. 2^hi sample spacings
+extern "C" void fuzz_rows(uint64_t seed, int64_t n, double lo, double hi, Result* res) {
+    std::mt19937_64 rng(seed);
+    auto u = [&](double a, double b) { return a + (b - a) * ((double)(rng() >> 11) * 0x1p-53); };
+    auto pick = [&](int64_t a, int64_t b) { return a + (int64_t)(rng() % (uint64_t)(b - a + 1)); };
+    const double kPi = 3.14159265358979323846;
+    for (int64_t i = 0; i < n;) {
+        const int s = (int)pick(3, 21);
+        const double h = std::ldexp(1.0, s), Rd = std::exp2(u(lo, hi)) * h;
+        if (Rd > 536870912.0) continue;
+        const int32_t R = (int32_t)Rd;
+        const int hw = 16 << pick(0, 4), hh = 2 << pick(0, 3);
+        const int64_t zone = ((1ll << 30) >> s) - hw;
+        if (zone < 0) continue;
+        const Lattice g = lattice(s, hw, hh, (int32_t)(pick(-zone, zone) * (1 << s) + (1 << s >> 1)),
+                                  (int32_t)(pick(-zone, zone) * (1 << s) + (1 << s >> 1)), R);
+        const double px = g.xc + (double)pick(-hw, hw - 1) * h, py = g.yc + (double)pick(-hh, hh - 1) * h;
+        const int slope = (int)pick(0, 5);
+        double th = slope == 0 ? 0.0 : slope == 1 ? kPi / 2 : u(0, 2 * kPi);
+        if (slope == 2) th = std::pow(10.0, u(-7, -0.5)) * (rng() & 1 ? 1 : -1);
+        if (slope == 3) th = kPi / 2 + std::pow(10.0, u(-7, -0.5)) * (rng() & 1 ? 1 : -1);
+        const double d = R + (rng() & 1 ? (double)pick(-3, 3) : u(-2, 2) * h);
+        const double size = rng() & 1 ? h * std::exp2(u(-3, 12)) : std::exp2(u(s, 30));
+        const double side = rng() & 1 ? 1 : -1, along = rng() % 4 ? u(0, 1) : (double)(rng() & 1);
+        const double turn = along == 0.0 || along == 1.0 ? u(-kPi / 2, kPi / 2) : 0.0;   // end caps: any direction outwards
+        const double nx = -std::sin(th + turn) * side, ny = std::cos(th + turn) * side;
+        const double ax = px + nx * d - std::cos(th) * size * along, ay = py + ny * d - std::sin(th) * size * along;
+        const double bx = ax + std::cos(th) * size, by = ay + std::sin(th) * size;
+        const double e = 1073741823.0;
+        if (std::fabs(ax) > e || std::fabs(ay) > e || std::fabs(bx) > e || std::fabs(by) > e) {
+            if (rng() % 8) continue;   // mostly drawn again; some cut off at the grid
+        }
+        const int4 o = make_int4((int)std::lround(max(min(ax, e), -e)), (int)std::lround(max(min(ay, e), -e)),
+                                 (int)std::lround(max(min(bx, e), -e)), (int)std::lround(max(min(by, e), -e)));
+        const int64_t m = rng() & 1 ? 1 : pick(1, 64);
+        compare(g, o, piece_box(o, pick(0, m - 1), m), 4, rng, res);
+        i++;
+    }
+}
+"""
+
+
+class Result(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_int64) for n in ("wrong", "columns", "covered", "rows")]
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    return sweep_host.library(tmp_path_factory.mktemp("sweep"), ENTRIES)
+
+
+@pytest.mark.parametrize("lo, hi", [(-4, 7), (7, 10), (10, 14), (14, 18), (18, 22), (22, 26)])
+def test_rows_equal_the_predicate(lib, lo, hi):
+    res = Result()
+    lib.fuzz_rows(ctypes.c_uint64(1000 + lo), ctypes.c_int64(60_000), ctypes.c_double(lo), ctypes.c_double(hi),
+                  ctypes.byref(res))
+    assert res.rows > 50_000 and 0.05 < res.covered / res.columns < 0.95
+    assert res.wrong == 0, (res.wrong, res.columns)
