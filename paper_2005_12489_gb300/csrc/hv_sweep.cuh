@@ -192,12 +192,14 @@ __device__ __forceinline__ void splat(uint32_t* bits, const Lattice& g, int32_t 
 
 // The half-widths of reach by row distance, for the tests that only need an
 // upper bound: reach[k] >= floor(sqrt(R^2 - f^2)) for every f with f >> rs = k,
-// where rs makes R >> rs at most 63.  (Single precision, rounded up; a
-// table read in place of a root per row.)
+// where rs makes R >> rs at most 63.  (Single precision, rounded up, the
+// factors formed as integers: a radius above 2^24 need not be a float, and
+// its rounding could cancel all of R - f.  A table read in place of a root per
+// row.)
 __device__ __forceinline__ void fill_reach(int32_t* reach, const Lattice& g, int tid) {
     if (tid <= (g.R >> g.rs)) {
-        const float fR = (float)g.R, f = (float)(tid << g.rs);
-        reach[tid] = min((int32_t)(sqrt_approx(fmaxf((fR - f) * (fR + f), 0.f)) * (1.f + 0x1p-19f)) + 1, g.R);
+        const int32_t f = tid << g.rs;
+        reach[tid] = min((int32_t)(sqrt_approx((float)(g.R - f) * (float)(g.R + f)) * (1.f + 0x1p-19f)) + 1, g.R);
     }
 }
 

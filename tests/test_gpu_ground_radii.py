@@ -95,3 +95,14 @@ def test_grazing_segments(ctx, z, radius):
             # a third vertex farther from the tile than the segment
             far = np.clip(np.round(seg.mean(0) * 1.5), -HALF, HALF - 1)
             check(ctx, "polygons", np.concatenate([seg, far[None]]), (z, t, t, 1), radius)
+
+
+@pytest.mark.parametrize("kind", ["points", "lines", "polygons"])
+@pytest.mark.parametrize("radius, f", [((1 << 24) + 1, 1 << 24), ((1 << 25) + 1, 1 << 25), ((1 << 28) + 15, 1 << 28)])
+@pytest.mark.parametrize("offset", [4, 8])
+def test_row_that_is_only_just_within_reach(ctx, kind, radius, f, offset):
+    """An object left of the tile, f above its first super-sample or pixel row:
+    the radius is no float, and the row is reached by the last few units of it."""
+    y = offset - f
+    xy = [(-3000, y), (-2000, y)] + ([(-2500, y - 100_000)] if kind == "polygons" else [])
+    check(ctx, kind, xy, (19, 262144, 262144, 1), radius)

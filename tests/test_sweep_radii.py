@@ -5,8 +5,9 @@ column in reach, for pieces whose capsule passes within a few units, or a few
 spacings, of a sample of the strip, at every slope, with contacts at the
 segment's inside and at its ends."""
 import ctypes
+import math
+import random
 
-import numpy as np
 import pytest
 
 import sweep_host
@@ -102,6 +103,15 @@ extern "C" void fuzz_rows(uint64_t seed, int64_t n, double lo, double hi, Result
 """
 
 
+ENTRIES += r"""
+extern "C" int reach_table(int32_t R, int32_t* reach) {
+    const Lattice g = lattice(3, 256, 16, 0, 0, R);
+    for (int tid = 0; tid < 256; tid++) fill_reach(reach, g, tid);
+    return g.rs;
+}
+"""
+
+
 class Result(ctypes.Structure):
     _fields_ = [(n, ctypes.c_int64) for n in ("wrong", "columns", "covered", "rows")]
 
@@ -118,3 +128,19 @@ def test_rows_equal_the_predicate(lib, lo, hi):
                   ctypes.byref(res))
     assert res.rows > 50_000 and 0.05 < res.covered / res.columns < 0.95
     assert res.wrong == 0, (res.wrong, res.columns)
+
+
+def test_reach_table_is_an_upper_bound(lib):
+    """reach[k] bounds the half-width of every row distance f with f >> rs = k
+    (the largest is f = k << rs), at radii that are no float (above 2^24) as well."""
+    rng = random.Random(5)
+    radii = [0, 1, 2, 63, 64, 65, 46340, 46341] + [(1 << b) + d for b in range(6, 29) for d in (-1, 0, 1, 15)]
+    radii += [(1 << 29) - 1, 1 << 29] + [int(2 ** rng.uniform(0, 29)) for _ in range(2000)]
+    radii += [rng.randrange(1 << 24, 1 << 29) for _ in range(4000)]
+    radii += [(rng.randrange(33, 64) << (24 - 5 + b)) + rng.randrange(1, 40) for b in range(5) for _ in range(400)]
+    table = (ctypes.c_int32 * 64)()
+    for R in (r for r in radii if 0 <= r <= 1 << 29):
+        rs = lib.reach_table(R, table)
+        for k in range((R >> rs) + 1):
+            f = k << rs
+            assert math.isqrt(R * R - f * f) <= table[k] <= R, (R, k, table[k])
