@@ -326,6 +326,8 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return r;
 }
 
+__device__ __forceinline__ uint32_t magnitude(int32_t v) { return v < 0 ? 0u - (uint32_t)v : (uint32_t)v; }
+
 // The line's offset and the nearer end's position along it (from either end
 // the offset is the same; the far end lies |d| beyond the near one).  Inside
 // the reach every coordinate is at most M = the visible box's size + R / h + 3;
@@ -352,7 +354,8 @@ __device__ __forceinline__ PieceRow piece_row(const Lattice& g, int4 o, int32_t 
     const float M = fmaxf((float)max(ex1 - ex0, 0) + rho + 3.f, Y);
     q.E = 0x1p-17f * M;
     if (o.w < o.y || (o.w == o.y && o.z < o.x)) o = make_int4(o.z, o.w, o.x, o.y);
-    // relative to the middle, wrapping: a value that wraps is still beyond 2^29
+    // relative to the middle, wrapping: a value that wraps is still beyond 2^29,
+    // by its magnitude as an unsigned number (a difference of 2^31 has none as an int)
     const uint32_t ox = (uint32_t)g.xc + (uint32_t)(mc << g.s), oy = (uint32_t)g.yc + (uint32_t)(mr << g.s);
     const int32_t ax = (int32_t)((uint32_t)o.x - ox), ay = (int32_t)((uint32_t)o.y - oy);
     const int32_t bx = (int32_t)((uint32_t)o.z - ox), by = (int32_t)((uint32_t)o.w - oy);
@@ -362,7 +365,7 @@ __device__ __forceinline__ PieceRow piece_row(const Lattice& g, int4 o, int32_t 
     const float inv = L2 > 0.f ? rsqrt_approx(L2) : 0.f, D = L2 * inv;
     q.mx = L2 > 0.f ? fx * inv : 1.f;
     q.my = fy * inv;
-    const uint32_t fa = (uint32_t)max(abs(ax), abs(ay)), fb = (uint32_t)max(abs(bx), abs(by));
+    const uint32_t fa = max(magnitude(ax), magnitude(ay)), fb = max(magnitude(bx), magnitude(by));
     bool from_a = fa <= fb;
     float near_t;
     const uint32_t fn = min(fa, fb);

@@ -110,6 +110,40 @@ extern "C" int reach_table(int32_t R, int32_t* reach) {
     return g.rs;
 }
 """
+ENTRIES += r"""
+static int4 turned(int4 o, int how) {   // mirrored, transposed, ends exchanged
+    if (how & 1) o = make_int4(o.y, o.x, o.w, o.z);
+    if (how & 2) o = make_int4(o.z, o.w, o.x, o.y);
+    return o;
+}
+// strips along the grid's borders at zooms 0 to 2 and segments from there to the
+// opposite border, cut into many pieces: coordinate differences of up to 2^31 + half a spacing
+extern "C" void border_rows(uint64_t seed, int64_t n, Result* res) {
+    std::mt19937_64 rng(seed);
+    auto pick = [&](int64_t a, int64_t b) { return a + (int64_t)(rng() % (uint64_t)(b - a + 1)); };
+    const int64_t lo = -(1ll << 30), hi = (1ll << 30) - 1;
+    for (int64_t i = 0; i < n; i++) {
+        const int z = (int)pick(0, 2), centres = (int)(rng() & 1), L = 23 - z, s = centres ? L : L - 1;
+        const int rows = 4 << pick(0, 2), cols = rows == 4 ? 32 << pick(0, 3) : 256;
+        const int64_t half = 1ll << s >> 1, ps = 1ll << L;
+        const int64_t col0 = rng() & 1 ? 0 : pick(0, 256 / cols - 1) * cols, strip = rng() & 1 ? 0 : pick(0, 256 / rows - 1);
+        const int32_t R = (int32_t)(pick(1, rng() & 1 ? 3 : 64) << (19 - z));
+        Lattice g = lattice(s, centres ? cols / 2 : cols, centres ? rows / 2 : rows,
+                                  (int32_t)(lo + (col0 + cols / 2) * ps + half), (int32_t)(lo + (strip * rows + rows / 2) * ps + half), R);
+        const int64_t far_end = pick(0, 3) ? (1ll << 30) - half + pick(-2, 1) : hi - pick(0, 1 << 23);
+        const int64_t x = max(lo, min(hi, lo + pick(0, 40) * half + pick(-2, 2)));
+        const int64_t slant = pick(0, 2) == 0 ? pick(0, 1 << 24) : 0;
+        const int how = (int)pick(0, 3);
+        int4 o = turned(make_int4((int)x, (int)(lo + (rng() & 1 ? 0 : pick(0, 1 << 22))), (int)min(hi, x + slant), (int)min(hi, far_end)), how);
+        if (rng() & 1) {   // the right and bottom borders
+            g.xc = -g.xc + (1 << s), g.yc = -g.yc + (1 << s);
+            o = make_int4((int)min(hi, -(int64_t)o.x), (int)min(hi, -(int64_t)o.y), (int)min(hi, -(int64_t)o.z), (int)min(hi, -(int64_t)o.w));
+        }
+        const int64_t m = 1 << pick(0, 12), k = rng() & 1 ? pick(0, min(m - 1, (int64_t)8)) : pick(0, m - 1);
+        compare(g, o, piece_box(o, how & 2 ? m - 1 - k : k, m), 6, rng, res);
+    }
+}
+"""
 
 
 class Result(ctypes.Structure):
@@ -127,6 +161,13 @@ def test_rows_equal_the_predicate(lib, lo, hi):
     lib.fuzz_rows(ctypes.c_uint64(1000 + lo), ctypes.c_int64(60_000), ctypes.c_double(lo), ctypes.c_double(hi),
                   ctypes.byref(res))
     assert res.rows > 50_000 and 0.05 < res.covered / res.columns < 0.95
+    assert res.wrong == 0, (res.wrong, res.columns)
+
+
+def test_rows_at_the_grid_border(lib):
+    res = Result()
+    lib.border_rows(ctypes.c_uint64(3), ctypes.c_int64(40_000), ctypes.byref(res))
+    assert res.rows > 20_000 and res.covered > 0
     assert res.wrong == 0, (res.wrong, res.columns)
 
 
