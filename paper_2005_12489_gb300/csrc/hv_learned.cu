@@ -305,28 +305,36 @@ __device__ __forceinline__ void prediction_error(const LModel& m, uint64_t i, ui
 
 // Per-piece error bounds (and summed errors) over every stored key, of the
 // lines alone and, with kMlp, of lines and network, in one pass with the steps
-// that the lookups take.  One warp per piece: the piece's parameters and
-// the network are read once (the weights as floats in shared memory) and its
-// maximum and sum are formed in registers; only keys equal to the next
-// piece's first key belong elsewhere and go there by themselves.  (Without
+// that the lookups take.  A group of `lanes` neighbouring lanes (a power of two)
+// takes one of the `parts` parts of a piece: a whole warp the piece, at the default
+// length of 512 keys; longer pieces fall into parts of kEpsKeys keys (10 M keys in
+// 10 pieces, one training step included: 40 ms with a warp per piece, now 0.5 ms), and
+// pieces shorter than a warp share one (pieces of 1 key: 17.4 -> 2.9 ms).  The
+// piece's parameters and the network are read once (the weights as floats in
+// shared memory) and its maximum and sum are formed in registers; only keys equal to
+// the next piece's first key belong elsewhere and go there by themselves.  (Without
 // kMlp there is nothing to choose between pieces and sum_l is one number.)
+constexpr uint32_t kEpsKeys = 512;
+
 template <bool kMlp>
-__global__ void __launch_bounds__(256) k_eps(LModel m, uint32_t* eps_l, uint32_t* eps_m, unsigned long long* sum_l,
-                                             unsigned long long* sum_m) {
+__global__ void __launch_bounds__(256) k_eps(LModel m, uint32_t lanes, uint32_t parts, uint32_t* eps_l, uint32_t* eps_m,
+                                             unsigned long long* sum_l, unsigned long long* sum_m) {
     __shared__ float sw[kLearnNW];
     if (kMlp) {
         for (int i = threadIdx.x; i < kLearnNW; i += blockDim.x) sw[i] = __bfloat162float(m.w[i]);
         __syncthreads();
     }
-    const uint64_t j0 = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (j0 >= m.n_seg) return;
-    const uint64_t i0 = j0 * m.P, i1 = i0 + m.P < m.n ? i0 + m.P : m.n;
+    const uint64_t group = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) / lanes;
+    const uint32_t sub = threadIdx.x & (lanes - 1);
+    // (groups beyond the last piece take no keys, but part in the warp's shuffles)
+    const uint64_t j0 = min(group / parts, (uint64_t)m.n_seg - 1), part = group % parts;
+    const uint64_t i0 = j0 * m.P + part * kEpsKeys;
+    const uint64_t end = group / parts < m.n_seg ? min(j0 * m.P + min((part + 1) * kEpsKeys, (uint64_t)m.P), m.n) : 0;
     const uint64_t next = j0 + 1 < m.n_seg ? m.kb[j0 + 1] : ~0ull;
     uint32_t el = 0, em = 0;
     unsigned long long sl = 0, sm = 0;
     const NetF32 net{sw};
-    for (uint64_t i = i0 + lane; i < i1; i += 32) {
+    for (uint64_t i = i0 + sub; i < end; i += lanes) {
         const uint64_t k = __ldg(m.keys + i);
         const bool own = k < next;
         const uint32_t j = own ? (uint32_t)j0 : learn_piece(m, k);
@@ -354,20 +362,22 @@ __global__ void __launch_bounds__(256) k_eps(LModel m, uint32_t* eps_l, uint32_t
             }
         }
     }
-    el = __reduce_max_sync(kFull, el);
-    if (kMlp) em = __reduce_max_sync(kFull, em);
-    for (int o = 16; o > 0; o >>= 1) {
-        sl += __shfl_xor_sync(kFull, sl, o);
-        if (kMlp) sm += __shfl_xor_sync(kFull, sm, o);
+    // without kMlp the sum is the warp's
+    for (uint32_t o = 16; o > 0; o >>= 1) {
+        const uint32_t ul = __shfl_xor_sync(kFull, el, o), um = kMlp ? __shfl_xor_sync(kFull, em, o) : 0u;
+        const unsigned long long vl = __shfl_xor_sync(kFull, sl, o), vm = kMlp ? __shfl_xor_sync(kFull, sm, o) : 0ull;
+        if (o < lanes) el = max(el, ul), em = max(em, um), sm += vm;
+        if (o < lanes || !kMlp) sl += vl;
     }
-    if (lane == 0) {
+    if (sub == 0 && i0 < end) {
         atomicMax(eps_l + j0, el);
-        atomicAdd(sum_l + (kMlp ? j0 : 0), sl);
         if (kMlp) {
+            atomicAdd(sum_l + j0, sl);
             atomicMax(eps_m + j0, em);
             atomicAdd(sum_m + j0, sm);
         }
     }
+    if (!kMlp && (threadIdx.x & 31) == 0) atomicAdd(sum_l, sl);
 }
 
 // Keep the MLP term for a piece only where it narrows the piece's bound.
@@ -542,7 +552,9 @@ static int build_one(Ctx* c, Learned* L, const uint64_t* keys, uint64_t n, const
               A.get((void**)&emb, (uint64_t)n_seg * 16) == HV_OK && A.get((void**)&gemb, (uint64_t)n_seg * 16) == HV_OK &&
               A.get((void**)&wb, nw * 2) == HV_OK && A.get((void**)&embb, (uint64_t)n_seg * 8) == HV_OK;
     uint32_t pieces_mlp = 0;
-    const uint32_t piece_blocks = blocks_for((uint64_t)n_seg * 32, 256);
+    uint32_t lanes = 1;
+    while (lanes < 32 && lanes < P) lanes *= 2;
+    const uint32_t parts = (P + kEpsKeys - 1) / kEpsKeys, eps_blocks = blocks_for((uint64_t)n_seg * parts * lanes, 256);
     if (ok && steps > 0 && H > 0) {
         cudaMemset(gw, 0, nw * 4);
         cudaMemset(mo, 0, nw * 4);
@@ -570,7 +582,7 @@ static int build_one(Ctx* c, Learned* L, const uint64_t* keys, uint64_t n, const
         // (the embeddings' gradient array, no longer needed, holds the summed errors)
         unsigned long long *sum_l = (unsigned long long*)gemb, *sum_m = sum_l + n_seg;
         HV_CUDA(cudaMemset(gemb, 0, (uint64_t)n_seg * 16));
-        k_eps<true><<<piece_blocks, 256>>>(mm, eps_l, eps, sum_l, sum_m);
+        k_eps<true><<<eps_blocks, 256>>>(mm, lanes, parts, eps_l, eps, sum_l, sum_m);
         HV_TRY(bounds(eps_l, sum_l, &eps_lin, &mean_lin, &sum_lin));
         HV_TRY(bounds(eps, sum_m, &eps_mlp, &mean_mlp, &sum_mlp));
         // ... then each piece keeps the model with the narrower bound, and that
@@ -586,7 +598,7 @@ static int build_one(Ctx* c, Learned* L, const uint64_t* keys, uint64_t n, const
         if (pieces_mlp) m = mm;
     } else {
         // (one sum over all pieces: nothing to choose between)
-        k_eps<false><<<piece_blocks, 256>>>(m, eps_l, nullptr, scratch + 3, nullptr);
+        k_eps<false><<<eps_blocks, 256>>>(m, lanes, parts, eps_l, nullptr, scratch + 3, nullptr);
         HV_TRY(bounds(eps_l, nullptr, &eps_lin, &mean_lin, &sum_lin));
     }
     cudaEventRecord(t1);
