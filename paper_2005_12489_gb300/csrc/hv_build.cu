@@ -72,8 +72,8 @@ __device__ __forceinline__ int4 warp_union(int4 b) {
                      __reduce_max_sync(kFull, b.z), __reduce_max_sync(kFull, b.w));
 }
 
-// The points of sorted keys and (if asked for) the boxes of their leaves: one
-// warp per leaf, so that the points are not read again for their boxes.
+// The points of sorted keys and the boxes of their leaves: one warp per leaf, so
+// that the points are not read again for their boxes.
 __global__ void k_key_points(const uint64_t* keys, uint64_t n, int2* obj, int4* box) {
     const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     if ((i & ~31ull) >= n) return;
@@ -83,7 +83,6 @@ __global__ void k_key_points(const uint64_t* keys, uint64_t n, int2* obj, int4* 
         obj[i] = o;
         b = PointObj::box(o);
     }
-    if (box == nullptr) return;
     b = warp_union(b);
     if ((i & 31) == 0) box[i >> 5] = b;
 }
@@ -183,46 +182,48 @@ int sort_objects(Ctx* c, typename O::T** obj, uint64_t n, uint64_t** keys_out, u
     return HV_OK;
 }
 
-// Sort points by Hilbert key.  A point's key determines the point (the curve
+// Boxes of the levels of a tree over n objects, two levels at a time.
+uint64_t level_box_bytes(uint64_t n) {
+    const uint64_t n_leaf = (n + 31) / 32;
+    return (n_leaf + (n_leaf + 31) / 32 + 1) * 16;
+}
+
+// The sorted Hilbert keys of points.  A point's key determines the point (the curve
 // visits every grid position once), so the keys alone are sorted, without a
 // permutation and a gather through it, and the points are read off the sorted
-// keys afterwards (k_key_points): *obj is left as room for them.  The sort's
-// second buffer is the points' own array, as wide as the keys; one
-// allocation of n keys is all that grows with n but the sort's counters.
-// If the sort fails the points are gone: *obj is released and set to NULL.
-int sort_points(Ctx* c, int2** obj, uint64_t n, uint64_t** keys_out) {
-    uint64_t* keys;
-    HV_TRY(dev_alloc(c, (void**)&keys, n * 8));
-    Tmp tmp(c);
-    cub::DoubleBuffer<uint64_t> buf(keys, (uint64_t*)*obj);
+// keys afterwards (k_key_points).  The points are only read, so that a layer whose
+// sort fails still has them (the points' array as the sort's second buffer saved 0.4
+// of the 12 ms that 100M points take to load, index and view).  *room: one scratch
+// allocation of `tmp` for the second buffer and the sort's counters, free for the
+// levels' boxes when the keys are sorted.
+int sort_points(Ctx* c, const int2* obj, uint64_t n, uint64_t* keys, Tmp& tmp, void** room) {
+    cub::DoubleBuffer<uint64_t> buf(keys, keys);
     size_t temp_bytes = 0;
-    void* temp = nullptr;
     cudaError_t e = cub::DeviceRadixSort::SortKeys(nullptr, temp_bytes, buf, (uint32_t)n, 0, 62);
-    int rc = HV_ECUDA;
-    if (e == cudaSuccess)
-        rc = tmp.get(&temp, temp_bytes);
-    else
-        set_error("radix sort failed: %s", cudaGetErrorString(e));
-    if (rc != HV_OK) { dev_free(c, keys, n * 8); return rc; }
-    k_point_keys<<<grid_for((n + 1) / 2, 256), 256>>>(*obj, n, keys);
-    e = cub::DeviceRadixSort::SortKeys(temp, temp_bytes, buf, (uint32_t)n, 0, 62);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) {
+        const uint64_t second = (std::max(n * 8, level_box_bytes(n)) + 255) & ~255ull;
+        HV_TRY(tmp.get(room, second + temp_bytes));
+        buf = cub::DoubleBuffer<uint64_t>(keys, (uint64_t*)*room);
+        k_point_keys<<<grid_for((n + 1) / 2, 256), 256>>>(obj, n, keys);
+        e = cub::DeviceRadixSort::SortKeys((uint8_t*)*room + second, temp_bytes, buf, (uint32_t)n, 0, 62);
+        // (an odd number of passes ends in the second buffer)
+        if (e == cudaSuccess && buf.Current() != keys)
+            e = cudaMemcpyAsync(keys, buf.Current(), n * 8, cudaMemcpyDeviceToDevice, 0);
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    }
     if (e != cudaSuccess) {
         set_error("radix sort failed: %s", cudaGetErrorString(e));
-        dev_free(c, keys, n * 8);
-        dev_free(c, *obj, n * 8);
-        *obj = nullptr;
         return HV_ECUDA;
     }
-    *keys_out = buf.Current();
-    *obj = (int2*)buf.Alternate();
     return HV_OK;
 }
 
 // Build the inner levels over sorted objects.  point_keys: the sorted keys of a
-// point layer whose points are still to be read off them.
+// point layer whose points are still to be read off them, with room for the
+// levels' boxes (level_box_bytes).
 template <class O>
-int build_levels(Ctx* c, typename O::T* obj, uint64_t n, Tree* t, const uint64_t* point_keys = nullptr) {
+int build_levels(Ctx* c, typename O::T* obj, uint64_t n, Tree* t, const uint64_t* point_keys = nullptr,
+                 void* room = nullptr) {
     *t = Tree();
     t->view.n_obj = n;
     if (n == 0) return HV_OK;
@@ -239,9 +240,8 @@ int build_levels(Ctx* c, typename O::T* obj, uint64_t n, Tree* t, const uint64_t
         total += counts[top];
         below = counts[top];
     } while (below > 1);
-    int4 *box_a, *box_b;
-    HV_TRY(tmp.get((void**)&box_a, n_leaf * 16));
-    HV_TRY(tmp.get((void**)&box_b, ((n_leaf + 31) / 32) * 16 + 16));
+    if (!room) HV_TRY(tmp.get(&room, level_box_bytes(n)));
+    int4 *box_a = (int4*)room, *box_b = box_a + n_leaf;
     HV_TRY(dev_alloc(c, (void**)&t->nodes, total * 512));
     t->nodes_bytes = total * 512;
     t->n_nodes = total;
@@ -460,14 +460,15 @@ void free_tree(Ctx* c, Tree* t) {
 int build_tree_points(Layer* L) {
     Ctx* c = L->ctx;
     const uint64_t n = L->n_obj;
-    if (n) {
-        if (!L->obj) { set_error("the layer lost its points in a failed index build"); return HV_ESTATE; }
-        HV_TRY(sort_points(c, (int2**)&L->obj, n, &L->keys));
-    }
-    const int rc = build_levels<PointObj>(c, (int2*)L->obj, n, &L->tree, L->keys);
+    if (n == 0) return build_levels<PointObj>(c, nullptr, 0, &L->tree);
+    Tmp tmp(c);
+    void* room = nullptr;
+    HV_TRY(dev_alloc(c, (void**)&L->keys, n * 8));
+    int rc = sort_points(c, (const int2*)L->obj, n, L->keys, tmp, &room);
+    // (up to here the points are in their input order, then in the keys': either way
+    // a failed build leaves them for another attempt)
+    if (rc == HV_OK) rc = build_levels<PointObj>(c, (int2*)L->obj, n, &L->tree, L->keys, room);
     if (rc != HV_OK) {
-        // the layer keeps its points (in their order), for another attempt
-        if (n) k_key_points<<<grid_for(n, 256), 256>>>(L->keys, n, (int2*)L->obj, nullptr);
         cudaDeviceSynchronize();
         free_tree(c, &L->tree);
         dev_free(c, L->keys, n * 8);
