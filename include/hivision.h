@@ -353,23 +353,22 @@ enum {
     HV_PHASE_TOTAL = 0,       /* warp-cycles of the launch (CTA lifetimes x warps) */
     HV_PHASE_PROLOGUE,        /* request decode, result init (fill: outline decode) */
     HV_PHASE_CULL,            /* tile cull of the strip: R-tree or learned lookup */
-    HV_PHASE_BIN,             /* binning the frontier by block column (0 for points) */
-    HV_PHASE_BLOCKS_CTA,      /* the pixel-block phase (points: the sweep of the
-                                 frontier), CTA time x warps */
+    HV_PHASE_BIN,             /* unused: 0 */
+    HV_PHASE_BLOCKS_CTA,      /* the sweep of the strip's frontier, CTA time x warps */
     HV_PHASE_BLOCKS_WARP,     /* ... of which warps were busy (rest: waiting) */
     HV_PHASE_LEAF,            /* ... of which in leaf visits (exact predicates) */
     HV_PHASE_DESCEND,         /* ... of which below the frontier: node tests and
                                  leaf visits (the rest of the busy time is the
-                                 blocks' scans of the frontier) */
+                                 tests of the frontier's entries) */
     HV_PHASE_ENCODE,          /* output encode */
     HV_PHASE_CTAS,            /* counts: CTAs, */
-    HV_PHASE_BLOCK_COUNT,     /*   8 x 4 pixel blocks, */
+    HV_PHASE_BLOCK_COUNT,     /*   8 x 4 pixel blocks of the strips swept, */
     HV_PHASE_LEAF_VISITS,     /*   leaf visits, */
     HV_PHASE_NODE_VISITS,     /*   inner-node visits in descents, */
-    HV_PHASE_FRONTIER_TESTS,  /*   frontier entries tested by blocks (points: once per strip), */
-    HV_PHASE_LEAF_EMPTY,      /*   leaf visits with no record in reach of an
-                                   undecided sample (0 for points), */
-    HV_PHASE_LEAF_DECIDED,    /*   leaf visits that decided a sample (0 for points) */
+    HV_PHASE_FRONTIER_TESTS,  /*   frontier entries tested (once per strip), */
+    HV_PHASE_LEAF_EMPTY,      /*   leaf visits that decided no sample, with no record
+                                   in reach of an undecided one, */
+    HV_PHASE_LEAF_DECIDED,    /*   leaf visits that decided a sample */
     HV_PHASE_COUNT = 16
 };
 

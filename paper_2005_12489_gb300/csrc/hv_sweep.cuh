@@ -153,17 +153,23 @@ __device__ __forceinline__ int32_t half_width(const Lattice& g, int32_t f, int32
 // Columns of sample row `row` (bits of its words): set [lo, hi], 0 <= lo <= hi.
 // Bits that are set already are left alone (a plain read first: most words
 // that meet dense data are full, and the reads of one word are a broadcast
-// where the atomics would queue).
-__device__ __forceinline__ void set_columns(uint32_t* row, int lo, int hi) {
+// where the atomics would queue).  True if a bit of them was not set: this and the
+// functions that draw objects report it to the phase profile, which counts the leaf
+// visits that decided a sample; elsewhere nothing reads it.
+__device__ __forceinline__ bool set_bits(uint32_t* word, uint32_t m) {
+    return (m & ~*(volatile uint32_t*)word) && (m & ~atomicOr(word, m));
+}
+__device__ __forceinline__ bool set_columns(uint32_t* row, int lo, int hi) {
     const int k0 = lo >> 5, k1 = hi >> 5;
     uint32_t m = ~0u << (lo & 31);
     const uint32_t last = ~0u >> (31 - (hi & 31));
+    bool fresh = false;
     for (int k = k0; k < k1; k++) {
-        if (m & ~*(volatile uint32_t*)(row + k)) atomicOr(row + k, m);
+        fresh |= set_bits(row + k, m);
         m = ~0u;
     }
     m &= last;
-    if (m & ~*(volatile uint32_t*)(row + k1)) atomicOr(row + k1, m);
+    return set_bits(row + k1, m) | fresh;
 }
 
 // Set the samples that lie within R of every point of the lane's box
@@ -173,12 +179,13 @@ __device__ __forceinline__ void set_columns(uint32_t* row, int lo, int hi) {
 // |y - y1|), and with w = floor(sqrt(R^2 - f^2)) the columns are [x1 - w, x0 + w].
 // Only the rows of `open` (a bit per sample row) are drawn.
 template <bool kNarrowR>
-__device__ __forceinline__ void splat(uint32_t* bits, const Lattice& g, int32_t x0, int32_t y0, int32_t x1,
+__device__ __forceinline__ bool splat(uint32_t* bits, const Lattice& g, int32_t x0, int32_t y0, int32_t x1,
                                       int32_t y1, uint32_t open) {
     const int r0 = max(g.hh - ((g.R - y1) >> g.s), 0);
     const int r1 = min(((y0 + g.R) >> g.s) + g.hh, 2 * g.hh - 1);
-    if (r0 > r1) return;
+    if (r0 > r1) return false;
     open &= (~0u << r0) & (~0u >> (31 - r1));
+    bool fresh = false;
     while (open) {
         const int r = __ffs(open) - 1;
         open &= open - 1;
@@ -186,8 +193,9 @@ __device__ __forceinline__ void splat(uint32_t* bits, const Lattice& g, int32_t 
         const int32_t f = max(abs(y - y0), abs(y - y1));
         const int32_t w = half_width<kNarrowR>(g, f, x0, x1);
         const int lo = max(g.hw - ((w - x1) >> g.s), 0), hi = min(((x0 + w) >> g.s) + g.hw, 2 * g.hw - 1);
-        if (lo <= hi) set_columns(bits + r * kBitStride, lo, hi);
+        if (lo <= hi) fresh |= set_columns(bits + r * kBitStride, lo, hi);
     }
+    return fresh;
 }
 
 // The half-widths of reach by row distance, for the tests that only need an
@@ -263,8 +271,9 @@ __device__ __forceinline__ uint32_t shl32(uint32_t v, int n) {
 // atomics on the same word where the boxes crowd), but every lane takes part
 // in every row.
 template <bool kNarrowR>
-__device__ __forceinline__ void splat_window(uint32_t* bits, const Lattice& g, int32_t x0, int32_t y0, int32_t x1,
+__device__ __forceinline__ bool splat_window(uint32_t* bits, const Lattice& g, int32_t x0, int32_t y0, int32_t x1,
                                              int32_t y1, int c0, bool active, uint32_t rows, int lane) {
+    bool fresh = false;
     const int32_t origin = (c0 - g.hw) * (1 << g.s);
     x0 -= origin;
     x1 -= origin;
@@ -289,9 +298,10 @@ __device__ __forceinline__ void splat_window(uint32_t* bits, const Lattice& g, i
         const int k = c0 >> 5, sh = c0 & 31, words = g.hw >> 4;
         uint32_t* row = bits + lane * kBitStride;
         const uint32_t a = acc << sh, b = sh ? acc >> (32 - sh) : 0u;
-        if (k >= 0 && k < words && (a & ~*(volatile uint32_t*)(row + k))) atomicOr(row + k, a);
-        if (k + 1 >= 0 && k + 1 < words && (b & ~*(volatile uint32_t*)(row + k + 1))) atomicOr(row + k + 1, b);
+        if (k >= 0 && k < words) fresh |= set_bits(row + k, a);
+        if (k + 1 >= 0 && k + 1 < words) fresh |= set_bits(row + k + 1, b);
     }
+    return fresh;
 }
 
 // A box of points is worth drawing when it is no wider than about R (the
@@ -394,12 +404,13 @@ __device__ __forceinline__ PieceRow piece_row(const Lattice& g, int4 o, int32_t 
 }
 
 // Exact test of one sample (column i of row r), unless it is set already.
-__device__ __forceinline__ void test_sample(uint32_t* bits, const Lattice& g, const int4* seg, int i, int r) {
+__device__ __forceinline__ bool test_sample(uint32_t* bits, const Lattice& g, const int4* seg, int i, int r) {
     uint32_t* word = bits + r * kBitStride + (i >> 5);
-    if ((*(volatile uint32_t*)word >> (i & 31)) & 1u) return;
+    if ((*(volatile uint32_t*)word >> (i & 31)) & 1u) return false;
     const int4 o = __ldg(seg);
-    if (segment_within(o.x, o.y, o.z, o.w, g.xc + (i - g.hw) * (1 << g.s), g.yc + (r - g.hh) * (1 << g.s), g.R2))
-        atomicOr(word, 1u << (i & 31));
+    if (!segment_within(o.x, o.y, o.z, o.w, g.xc + (i - g.hw) * (1 << g.s), g.yc + (r - g.hh) * (1 << g.s), g.R2))
+        return false;
+    return !((atomicOr(word, 1u << (i & 31)) >> (i & 31)) & 1u);
 }
 
 // The capsule of radius r around a segment meets a row in one interval.  Its
@@ -412,7 +423,9 @@ __device__ __forceinline__ void test_sample(uint32_t* bits, const Lattice& g, co
 // more than a rounding for one, and pieces without a finite E.  Columns inside
 // the interval of radius R - E are covered, columns outside that of R + E are
 // not, and those between take the exact test.
-__device__ __noinline__ void draw_row_slow(uint32_t* bits, const Lattice& g, const PieceRow q, const int4* seg, int r) {
+// (Without kProf the result is false.)
+template <bool kProf>
+__device__ __noinline__ bool draw_row_slow(uint32_t* bits, const Lattice& g, const PieceRow q, const int4* seg, int r) {
     const int col = (int)(q.at & 0xffffu) - 1024, row = (int)(q.at >> 16) - 1024;
     const int clo = (int)(q.span & 0xffffu) - col, chi = (int)(q.span >> 16) - col;
     const float rho = (float)g.R * __int_as_float((127 - g.s) << 23);
@@ -431,17 +444,19 @@ __device__ __noinline__ void draw_row_slow(uint32_t* bits, const Lattice& g, con
         hi[k] = min(__float2int_rd(fmaf(tr, q.mx, -xm) + sqrt_approx(fmaxf(ar, 0.f))), chi);
         met[k] = k ? rad > 0.f && fminf(al, ar) >= 0.f : fmaxf(al, ar) >= 0.f;
     }
-    if (!met[0] || lo[0] > hi[0]) return;
+    if (!met[0] || lo[0] > hi[0]) return false;
     lo[1] = max(lo[1], lo[0]);
     hi[1] = min(hi[1], hi[0]);
+    bool fresh = false;
     if (met[1] && lo[1] <= hi[1])
-        set_columns(bits + r * kBitStride, lo[1] + col, hi[1] + col);
+        fresh = set_columns(bits + r * kBitStride, lo[1] + col, hi[1] + col);
     else
         lo[1] = hi[0] + 1, hi[1] = hi[0];
     for (int c = lo[0]; c <= hi[0]; c++) {
         if (c == lo[1]) c = hi[1] + 1;
-        if (c <= hi[0]) test_sample(bits, g, seg, c + col, r);
+        if (c <= hi[0]) fresh |= test_sample(bits, g, seg, c + col, r);
     }
+    return kProf && fresh;
 }
 
 // Set the samples of row r within R of the segment.  Where both discs meet the
@@ -452,7 +467,8 @@ __device__ __noinline__ void draw_row_slow(uint32_t* bits, const Lattice& g, con
 // near only while e < 1/2, that is w^2 > 6.25 (R E)^2, which the first condition
 // implies for R up to about 200 spacings (every radius in pixels); rows of larger
 // ground radii where e may reach 1/2 go to draw_row_slow, which tests them all.
-__device__ __forceinline__ void draw_row(uint32_t* bits, const Lattice& g, const PieceRow& q, const int4* seg, int r) {
+template <bool kProf = false>
+__device__ __forceinline__ bool draw_row(uint32_t* bits, const Lattice& g, const PieceRow& q, const int4* seg, int r) {
     const int col = (int)(q.at & 0xffffu) - 1024, row = (int)(q.at >> 16) - 1024;
     const float rho = (float)g.R * __int_as_float((127 - g.s) << 23);
     const float ym = (float)(r - row) - q.c0 * q.mx, xm = q.c0 * q.my, inv = rcp_approx(q.my);
@@ -462,8 +478,7 @@ __device__ __forceinline__ void draw_row(uint32_t* bits, const Lattice& g, const
     const float al = fmaf(-dl, dl, r2), ar = fmaf(-dr, dr, r2);
     if (!(fminf(al, ar) >= rE * fmaxf(8.f, 6.5f * rE)) || q.E >= rho) {
         // beyond R + E of the row both half-chords are imaginary
-        if (!(fmaxf(al, ar) < -8.f * rE - 2.f * q.E * q.E)) draw_row_slow(bits, g, q, seg, r);
-        return;
+        return !(fmaxf(al, ar) < -8.f * rE - 2.f * q.E * q.E) && draw_row_slow<kProf>(bits, g, q, seg, r);
     }
     const float wl = sqrt_approx(al), wr = sqrt_approx(ar);
     const float xl = fmaf(tl, q.mx, -xm) - wl, xr = fmaf(tr, q.mx, -xm) + wr;
@@ -474,17 +489,28 @@ __device__ __forceinline__ void draw_row(uint32_t* bits, const Lattice& g, const
     const int clo = (int)(q.span & 0xffffu) - col, chi = (int)(q.span >> 16) - col;
     // a doubtful column is left out of the interval and tested
     const int lo = max(il + (vl || nl < xl ? 1 : 0), clo), hi = min(ir - (vr || nr > xr ? 1 : 0), chi);
-    if (lo <= hi) set_columns(bits + r * kBitStride, lo + col, hi + col);
-    if (vl && il >= clo && il <= chi) test_sample(bits, g, seg, il + col, r);
-    if (vr && ir >= clo && ir <= chi) test_sample(bits, g, seg, ir + col, r);
+    bool fresh = false;
+    if (lo <= hi) fresh = set_columns(bits + r * kBitStride, lo + col, hi + col);
+    if (vl && il >= clo && il <= chi) fresh |= test_sample(bits, g, seg, il + col, r);
+    if (vr && ir >= clo && ir <= chi) fresh |= test_sample(bits, g, seg, ir + col, r);
+    return fresh;
 }
+
+// What a leaf visit came to, per lane, for the phase profile.
+struct Visit {
+    bool reached = false;   // an object that an open sample is in reach of
+    bool decided = false;   // a sample decided
+};
 
 // A segment leaf: 32 pieces, each with a run of open rows that it reaches.
 // The (piece, row) pairs are numbered through by a prefix sum over the lanes
 // and the lanes take them in turn, so a leaf costs ceil(pairs / 32) rounds
 // whatever the pieces' heights.
-__device__ __forceinline__ void draw_segments(const Params& p, const Src& src, uint32_t* bits, float4* pair_obj,
-                                              int* pair_row, const Lattice& g, uint32_t leaf, uint32_t rows, int lane) {
+template <bool kProf>
+__device__ __forceinline__ Visit draw_segments(const Params& p, const Src& src, uint32_t* bits, float4* pair_obj,
+                                               int* pair_row, const int32_t* reach, const Lattice& g, uint32_t leaf,
+                                               uint32_t rows, int lane) {
+    Visit v;
     const uint64_t i = (uint64_t)leaf * 32 + lane;
     int4 o = make_int4(0, 0, 0, 0), pb = make_int4(kEmptyLo, kEmptyLo, kEmptyHi, kEmptyHi);
     const int4* rec = (const int4*)src.obj + 2 * i;
@@ -497,8 +523,9 @@ __device__ __forceinline__ void draw_segments(const Params& p, const Src& src, u
     const int clo = max(g.hw - ((g.R - x0) >> g.s), 0), chi = min(((x1 + g.R) >> g.s) + g.hw, 2 * g.hw - 1);
     uint32_t mine = 0u;
     if (i < src.n && r0 <= r1 && clo <= chi) mine = rows & (~0u << r0) & (~0u >> (31 - r1));
+    if (kProf) v.reached = mine != 0u && box_open(bits, reach, g, x0, y0, x1, y1, mine);
     const uint32_t some = __ballot_sync(kFull, mine != 0u);
-    if (some == 0u) return;
+    if (some == 0u) return v;
     // from the first to the last open row
     const int first = __ffs(mine) - 1, count = mine ? 32 - __clz(mine) - first : 0;
     const int sum = lane_sums(count, lane), total = __shfl_sync(kFull, sum, 31), start = sum - count;
@@ -514,15 +541,16 @@ __device__ __forceinline__ void draw_segments(const Params& p, const Src& src, u
     for (int base = 0; base < total; base += 32) {
         const int k = rounds.object(base, lane), j = base + lane;
         if (j < total) {
-            const float4 u = pair_obj[2 * k], v = pair_obj[2 * k + 1];
+            const float4 a = pair_obj[2 * k], b = pair_obj[2 * k + 1];
             const int at = pair_row[k];
             PieceRow q;
-            q.mx = u.x, q.my = u.y, q.c0 = u.z, q.E = u.w;
-            q.ta = v.x, q.tb = v.y, q.at = __float_as_uint(v.z), q.span = __float_as_uint(v.w);
-            draw_row(bits, g, q, (const int4*)src.obj + 2 * ((uint64_t)leaf * 32 + (at & 31)), (at >> 5) + j);
+            q.mx = a.x, q.my = a.y, q.c0 = a.z, q.E = a.w;
+            q.ta = b.x, q.tb = b.y, q.at = __float_as_uint(b.z), q.span = __float_as_uint(b.w);
+            v.decided |= draw_row<kProf>(bits, g, q, (const int4*)src.obj + 2 * ((uint64_t)leaf * 32 + (at & 31)), (at >> 5) + j);
         }
         __syncwarp();
     }
+    return v;
 }
 
 // ---- polygon fill ---------------------------------------------------------------
@@ -555,7 +583,7 @@ __device__ __forceinline__ int crossing_end(const Lattice& g, int32_t lx, int32_
 // for the whole row.  Edges are taken 32 at a time, their (edge, row) pairs
 // shared over the lanes as for segments; then a lane per row turns the bits
 // into filled samples and clears them.
-__device__ __forceinline__ void fill_polygon(const Params& p, uint32_t* bits, uint32_t* cross, int4* pair_obj,
+__device__ __forceinline__ bool fill_polygon(const Params& p, uint32_t* bits, uint32_t* cross, int4* pair_obj,
                                              int* pair_row, const Lattice& g, uint64_t e0, uint64_t e1, int clo, int chi, uint32_t rows, int lane) {
     const int rf = __ffs(rows) - 1, rl = 31 - __clz(rows);
     for (uint64_t base = e0; base < e1; base += 32) {
@@ -588,6 +616,7 @@ __device__ __forceinline__ void fill_polygon(const Params& p, uint32_t* bits, ui
         __syncwarp();
     }
     __syncwarp();
+    bool fresh = false;
     if (lane >= rf && lane <= rl) {
         uint32_t carry = 0u;
         uint32_t* c = cross + lane * kBitStride;
@@ -605,16 +634,18 @@ __device__ __forceinline__ void fill_polygon(const Params& p, uint32_t* bits, ui
             carry ^= 0u - (s & 1u);
             if (d) c[k] = 0u;
             if (k == k0) f &= ~0u << (clo & 31);
-            if (k < g.hw >> 4 && (f & ~*(volatile uint32_t*)(row + k))) atomicOr(row + k, f);
+            if (k < g.hw >> 4) fresh |= set_bits(row + k, f);
         }
     }
     __syncwarp();
+    return fresh;
 }
 
 // A leaf of the polygon-box tree: the polygons whose box holds an open sample.
-__device__ __forceinline__ void fill_polygons(const Params& p, const Src& src, uint32_t* bits, uint32_t* cross,
-                                              int4* pair_obj, int* pair_row, const int32_t* reach, const Lattice& g, uint32_t leaf, uint32_t rows,
-                                              int lane) {
+__device__ __forceinline__ Visit fill_polygons(const Params& p, const Src& src, uint32_t* bits, uint32_t* cross,
+                                               int4* pair_obj, int* pair_row, const int32_t* reach, const Lattice& g,
+                                               uint32_t leaf, uint32_t rows, int lane) {
+    Visit v;
     const uint64_t i = (uint64_t)leaf * 32 + lane;
     int4 b = make_int4(kEmptyLo, kEmptyLo, kEmptyHi, kEmptyHi);
     uint32_t id = 0;
@@ -624,6 +655,7 @@ __device__ __forceinline__ void fill_polygons(const Params& p, const Src& src, u
     }
     const int32_t x0 = rel32(b.x, g.xc), y0 = rel32(b.y, g.yc), x1 = rel32(b.z, g.xc), y1 = rel32(b.w, g.yc);
     uint32_t m = __ballot_sync(kFull, b.x <= b.z && i < src.n && box_open(bits, reach, g, x0, y0, x1, y1, rows));
+    v.reached = m != 0u;
     while (m) {
         const int k = __ffs(m) - 1;
         m &= m - 1;
@@ -642,8 +674,9 @@ __device__ __forceinline__ void fill_polygons(const Params& p, const Src& src, u
             continue;
         }
         const int clo = max(g.hw - ((-kx0) >> g.s), 0), chi = min((kx1 >> g.s) + g.hw, 2 * g.hw - 1);
-        fill_polygon(p, bits, cross, pair_obj, pair_row, g, e0, e1, clo, chi, open, lane);
+        v.decided |= fill_polygon(p, bits, cross, pair_obj, pair_row, g, e0, e1, clo, chi, open, lane);
     }
+    return v;
 }
 
 // ---- traversal ----------------------------------------------------------------
@@ -678,13 +711,14 @@ __device__ __forceinline__ void sweep_entry(const Params& p, SweepSmem<kKind>& s
     while (true) {
         int32_t x0 = 0, y0 = 0, x1 = 0, y1 = 0;
         bool draw = false;
+        Visit visit;
         if (lvl == 0 && kKind != HV_LAYER_POINTS) {
             log_read(p, kKind == kPolyFill ? kLogPolyLeaf : kLogLeaf, node, lane);
             t0 = tick<kProf>();
             if constexpr (kKind == kPolyFill)
-                fill_polygons(p, src, sm.bits, sm.cross[warp], (int4*)sm.pair_obj[warp], sm.pair_row[warp], sm.reach, g, node, rows, lane);
+                visit = fill_polygons(p, src, sm.bits, sm.cross[warp], (int4*)sm.pair_obj[warp], sm.pair_row[warp], sm.reach, g, node, rows, lane);
             else
-                draw_segments(p, src, sm.bits, sm.pair_obj[warp], sm.pair_row[warp], g, node, rows, lane);
+                visit = draw_segments<kProf>(p, src, sm.bits, sm.pair_obj[warp], sm.pair_row[warp], sm.reach, g, node, rows, lane);
         } else if (lvl == 0) {
             log_read(p, kLogLeaf, node, lane);
             t0 = tick<kProf>();
@@ -694,6 +728,7 @@ __device__ __forceinline__ void sweep_entry(const Params& p, SweepSmem<kKind>& s
             if (draw) o = __ldg((const int2*)src.obj + i);
             x0 = x1 = rel32(o.x, g.xc);
             y0 = y1 = rel32(o.y, g.yc);
+            if (kProf) visit.reached = draw && box_open(sm.bits, sm.reach, g, x0, y0, x1, y1, rows);
         } else {
             const int32_t* base = src.lvl[lvl] + (uint64_t)node * 128;
             if (p.log != nullptr)
@@ -708,15 +743,20 @@ __device__ __forceinline__ void sweep_entry(const Params& p, SweepSmem<kKind>& s
             draw = draw && small_box(g, x0, y0, x1, y1);
             const int c0 = g.hw - ((g.R - bx0) >> g.s);
             if (((bx1 + g.R) >> g.s) + g.hw - c0 < 32 && __popc(rows) <= reach_rows) {
-                if (__any_sync(kFull, draw)) splat_window<kNarrowR>(sm.bits, g, x0, y0, x1, y1, c0, draw, rows, lane);
+                if (__any_sync(kFull, draw))
+                    visit.decided = splat_window<kNarrowR>(sm.bits, g, x0, y0, x1, y1, c0, draw, rows, lane);
             } else if (draw) {
-                splat<kNarrowR>(sm.bits, g, x0, y0, x1, y1, rows);
+                visit.decided = splat<kNarrowR>(sm.bits, g, x0, y0, x1, y1, rows);
             }
         }
         __syncwarp();
         if (lvl == 0) {
             prof_since<kProf>(sm, kPLeaf, t0, lane);
             prof_add<kProf>(sm, kPLeafVisits, 1, lane);
+            if constexpr (kProf) {
+                const bool decided = __any_sync(kFull, visit.decided), reached = __any_sync(kFull, visit.reached);
+                prof_add<kProf>(sm, decided ? kPLeafDecided : kPLeafEmpty, decided || !reached, lane);
+            }
             if (level == 0) return;
             lvl = 1;
         } else {
