@@ -144,6 +144,28 @@ extern "C" void border_rows(uint64_t seed, int64_t n, Result* res) {
     }
 }
 """
+ENTRIES += r"""
+// grid-wide segments in wide pieces (or whole) over strips that their boxes cover: exact tests taken
+extern "C" int64_t wide_pieces(uint64_t seed, int64_t n, int32_t R, Result* res) {
+    std::mt19937_64 rng(seed);
+    auto pick = [&](int64_t a, int64_t b) { return a + (int64_t)(rng() % (uint64_t)(b - a + 1)); };
+    const int64_t reads = g_reads, e = (1ll << 30) - 1;
+    for (int64_t i = 0; i < n; i++) {
+        const int s = (int)pick(6, 18), hw = 256, hh = 2 << pick(0, 3);
+        const int64_t zone = ((1ll << 30) >> s) - hw;
+        const Lattice g = lattice(s, hw, hh, (int32_t)(pick(-zone, zone) * (1 << s) + (1 << s >> 1)),
+                                  (int32_t)(pick(-zone, zone) * (1 << s) + (1 << s >> 1)), R < 0 ? -R << s >> 3 : R);
+        // through a point within a piece's extent of the strip
+        const int64_t m = pick(1, 4), near = 1ll << pick(s, 29);
+        const int64_t px = max(-e, min(e, g.xc + pick(-near, near))), py = max(-e, min(e, g.yc + pick(-near, near)));
+        const int4 o = make_int4((int)pick(-e, e), (int)pick(-e, e), 0, 0);
+        const int64_t bx = 2 * px - o.x, by = 2 * py - o.y;
+        if (bx < -e || bx > e || by < -e || by > e) continue;
+        compare(g, make_int4(o.x, o.y, (int)bx, (int)by), piece_box(make_int4(o.x, o.y, (int)bx, (int)by), pick(0, m - 1), m), 4, rng, res);
+    }
+    return g_reads - reads;
+}
+"""
 
 
 class Result(ctypes.Structure):
@@ -162,6 +184,27 @@ def test_rows_equal_the_predicate(lib, lo, hi):
                   ctypes.byref(res))
     assert res.rows > 50_000 and 0.05 < res.covered / res.columns < 0.95
     assert res.wrong == 0, (res.wrong, res.columns)
+
+
+@pytest.mark.parametrize("lo, hi", [(-24, -10), (-10, -4)])
+def test_rows_at_radii_of_a_few_units(lib, lo, hi):
+    res = Result()
+    lib.fuzz_rows(ctypes.c_uint64(7 - lo), ctypes.c_int64(60_000), ctypes.c_double(lo), ctypes.c_double(hi),
+                  ctypes.byref(res))
+    assert res.rows > 20_000 and res.covered > 0
+    assert res.wrong == 0, (res.wrong, res.columns)
+
+
+@pytest.mark.parametrize("R", [0, 1, 999, -1, -8, -64])     # units; below zero: eighths of a spacing
+def test_wide_pieces_take_few_exact_tests(lib, R):
+    """A piece's box may cover the strip while its line passes far away or crosses
+    a few columns of a row: an exact test for a column of every other row at most
+    on average, where testing the box's columns would take up to 512 a row."""
+    res = Result()
+    lib.wide_pieces.restype = ctypes.c_int64
+    tests = lib.wide_pieces(ctypes.c_uint64(9), ctypes.c_int64(40_000), ctypes.c_int32(R), ctypes.byref(res))
+    assert res.rows > 10_000 and res.wrong == 0, (res.rows, res.wrong)
+    assert tests < res.rows / 2, (tests, res.rows)
 
 
 def test_rows_at_the_grid_border(lib):
