@@ -98,6 +98,7 @@ struct Lattice {
 };
 
 constexpr int32_t kNarrow = 46340;   // floor(sqrt(2^31))
+constexpr int kTableReach = 16;      // spacings
 constexpr int32_t kRelMax = (1 << 30) + (1 << 22);
 
 __device__ __forceinline__ int32_t rel32(int32_t v, int32_t c) { return max(min(v - c, kRelMax), -kRelMax); }
@@ -211,6 +212,20 @@ __device__ __forceinline__ void fill_reach(int32_t* reach, const Lattice& g, int
     }
 }
 
+// An upper bound of the half-width at row distance f <= R.  The table's is off by up
+// to about R f / 64 w: with R of many spacings that is columns, in which samples
+// outside every object's reach stay open and keep boxes from being pruned.  There
+// (kFine) a root is taken, good to 2^-19.  300 tiles of 200,000 crowded points at
+// 64 px 9.56 -> 0.35 ms, of 50,000 polygons' outlines 28.1 -> 1.87 ms; as a branch taken
+// for each row instead of an instantiation 4,000 tiles of 100M points at 2 px lose 7%.
+// From kTableReach = 16 spacings on: the table is off by a quarter of a column there (8
+// and 32 measured alike).
+template <bool kFine>
+__device__ __forceinline__ int32_t reach_width(const int32_t* reach, const Lattice& g, int32_t f) {
+    if (!kFine) return reach[f >> g.rs];
+    return min((int32_t)(sqrt_approx((float)(g.R - f) * (float)(g.R + f)) * (1.f + 0x1p-19f)) + 1, g.R);
+}
+
 // Is a sample of columns lo..hi of the row open?
 __device__ __forceinline__ bool columns_open(const uint32_t* row, int lo, int hi) {
     const int k1 = hi >> 5;
@@ -231,17 +246,19 @@ __device__ __forceinline__ bool row_open(const uint32_t* row, const Lattice& g, 
 // Sample rows (one lane each) with an open sample that an object inside the
 // box could cover: within R of the box (rounded up).  Zero: nothing below the
 // box matters.
+template <bool kFine>
 __device__ __forceinline__ uint32_t open_rows(const uint32_t* bits, const int32_t* reach, const Lattice& g, int32_t x0,
                                               int32_t y0, int32_t x1, int32_t y1, int lane) {
     const int32_t y = (lane - g.hh) << g.s;
     const int32_t f = max(max(y0 - y, y - y1), 0);
-    const bool open = lane < 2 * g.hh && f <= g.R && row_open(bits + lane * kBitStride, g, x0, x1, reach[f >> g.rs]);
+    const bool open = lane < 2 * g.hh && f <= g.R && row_open(bits + lane * kBitStride, g, x0, x1, reach_width<kFine>(reach, g, f));
     return __ballot_sync(kFull, open);
 }
 
 // open_rows for the lane's own box: is any sample in reach open (in one of
 // the given rows)?  One pass for the 32 children of a node; those that pass
 // take open_rows again when their turn comes, after their siblings.
+template <bool kFine>
 __device__ __forceinline__ bool box_open(const uint32_t* bits, const int32_t* reach, const Lattice& g, int32_t x0,
                                          int32_t y0, int32_t x1, int32_t y1, uint32_t rows) {
     const int r0 = max(g.hh - ((g.R - y0) >> g.s), 0), r1 = min(((y1 + g.R) >> g.s) + g.hh, 2 * g.hh - 1);
@@ -251,7 +268,7 @@ __device__ __forceinline__ bool box_open(const uint32_t* bits, const int32_t* re
         const int r = __ffs(rows) - 1;
         rows &= rows - 1;
         const int32_t y = (r - g.hh) << g.s;
-        if (row_open(bits + r * kBitStride, g, x0, x1, reach[max(max(y0 - y, y - y1), 0) >> g.rs])) return true;
+        if (row_open(bits + r * kBitStride, g, x0, x1, reach_width<kFine>(reach, g, max(max(y0 - y, y - y1), 0)))) return true;
     }
     return false;
 }
@@ -539,7 +556,7 @@ __device__ __forceinline__ Visit draw_segments(const Params& p, const Src& src, 
     const int clo = max(g.hw - ((g.R - x0) >> g.s), 0), chi = min(((x1 + g.R) >> g.s) + g.hw, 2 * g.hw - 1);
     uint32_t mine = 0u;
     if (i < src.n && r0 <= r1 && clo <= chi) mine = rows & (~0u << r0) & (~0u >> (31 - r1));
-    if (kProf) v.reached = mine != 0u && box_open(bits, reach, g, x0, y0, x1, y1, mine);
+    if (kProf) v.reached = mine != 0u && box_open<true>(bits, reach, g, x0, y0, x1, y1, mine);
     const uint32_t some = __ballot_sync(kFull, mine != 0u);
     if (some == 0u) return v;
     // from the first to the last open row
@@ -670,13 +687,13 @@ __device__ __forceinline__ Visit fill_polygons(const Params& p, const Src& src, 
         id = __ldg(src.ids + i);
     }
     const int32_t x0 = rel32(b.x, g.xc), y0 = rel32(b.y, g.yc), x1 = rel32(b.z, g.xc), y1 = rel32(b.w, g.yc);
-    uint32_t m = __ballot_sync(kFull, b.x <= b.z && i < src.n && box_open(bits, reach, g, x0, y0, x1, y1, rows));
+    uint32_t m = __ballot_sync(kFull, b.x <= b.z && i < src.n && box_open<false>(bits, reach, g, x0, y0, x1, y1, rows));
     v.reached = m != 0u;
     while (m) {
         const int k = __ffs(m) - 1;
         m &= m - 1;
         const int32_t kx0 = __shfl_sync(kFull, x0, k), kx1 = __shfl_sync(kFull, x1, k);
-        const uint32_t open = open_rows(bits, reach, g, kx0, __shfl_sync(kFull, y0, k), kx1, __shfl_sync(kFull, y1, k), lane);
+        const uint32_t open = open_rows<false>(bits, reach, g, kx0, __shfl_sync(kFull, y0, k), kx1, __shfl_sync(kFull, y1, k), lane);
         if (open == 0) continue;
         const uint32_t pid = __shfl_sync(kFull, id, k);
         log_read(p, kLogPoly, pid, lane);
@@ -707,7 +724,7 @@ __device__ __forceinline__ Visit fill_polygons(const Params& p, const Src& src, 
 // and below it only the rows with such a sample matter.  (One drawing site and
 // one reach test for leaves and nodes keep the loop small for the instruction
 // cache.)
-template <int kKind, bool kNarrowR, bool kProf>
+template <int kKind, bool kNarrowR, bool kFine, bool kProf>
 __device__ __forceinline__ void sweep_entry(const Params& p, SweepSmem<kKind>& sm, const Src& src, const Lattice& g,
                                              int level, uint32_t id, uint32_t rows, int32_t bx0, int32_t bx1,
                                              int lane, int warp) {
@@ -744,7 +761,7 @@ __device__ __forceinline__ void sweep_entry(const Params& p, SweepSmem<kKind>& s
             if (draw) o = __ldg((const int2*)src.obj + i);
             x0 = x1 = rel32(o.x, g.xc);
             y0 = y1 = rel32(o.y, g.yc);
-            if (kProf) visit.reached = draw && box_open(sm.bits, sm.reach, g, x0, y0, x1, y1, rows);
+            if (kProf) visit.reached = draw && box_open<kFine>(sm.bits, sm.reach, g, x0, y0, x1, y1, rows);
         } else {
             const int32_t* base = src.lvl[lvl] + (uint64_t)node * 128;
             if (p.log != nullptr)
@@ -777,7 +794,7 @@ __device__ __forceinline__ void sweep_entry(const Params& p, SweepSmem<kKind>& s
             lvl = 1;
         } else {
             prof_add<kProf>(sm, kPNodeVisits, 1, lane);
-            const uint32_t m = __ballot_sync(kFull, valid && box_open(sm.bits, sm.reach, g, x0, y0, x1, y1, rows));
+            const uint32_t m = __ballot_sync(kFull, valid && box_open<kFine>(sm.bits, sm.reach, g, x0, y0, x1, y1, rows));
             if (lvl == 1) {
                 mask1 = m;
                 node1 = node;
@@ -819,7 +836,7 @@ __device__ __forceinline__ void sweep_entry(const Params& p, SweepSmem<kKind>& s
                 bx1 = rel32(__ldg(nb + 64), g.xc), by1 = rel32(__ldg(nb + 96), g.yc);
                 node = up * 32u + (uint32_t)c;
             }
-            rows = open_rows(sm.bits, sm.reach, g, bx0, by0, bx1, by1, lane);
+            rows = open_rows<kFine>(sm.bits, sm.reach, g, bx0, by0, bx1, by1, lane);
             if (rows == 0) continue;
             if (node >= src.lvl_n[lvl - 1]) {
                 if (lane == 0) check_failed(p, 3, ((uint64_t)(lvl - 1) << 40) | node);
@@ -833,7 +850,7 @@ __device__ __forceinline__ void sweep_entry(const Params& p, SweepSmem<kKind>& s
 
 // Every frontier entry of the strip, taken by the warps in turn, and the side
 // tree (objects longer than the learned index's halo) as one more entry.
-template <int kKind, bool kNarrowR, bool kProf>
+template <int kKind, bool kNarrowR, bool kFine, bool kProf>
 __device__ void sweep_pass(const Params& p, SweepSmem<kKind>& sm, const Src& src, const Src& side, const TreeArg& st,
                            bool side_hit, const Lattice& g, int tid) {
     const int lane = tid & 31, warp = tid >> 5;
@@ -862,10 +879,10 @@ __device__ void sweep_pass(const Params& p, SweepSmem<kKind>& sm, const Src& src
         const bool from_side = e >= f_count;
         const int4 b = from_side ? st.root_box : sm.fbox[fb][e];
         const int32_t x0 = rel32(b.x, g.xc), x1 = rel32(b.z, g.xc);
-        const uint32_t rows = open_rows(bits, sm.reach, g, x0, rel32(b.y, g.yc), x1, rel32(b.w, g.yc), lane);
+        const uint32_t rows = open_rows<kFine>(bits, sm.reach, g, x0, rel32(b.y, g.yc), x1, rel32(b.w, g.yc), lane);
         if (rows == 0) continue;
         const long long t0 = tick<kProf>();
-        sweep_entry<kKind, kNarrowR, kProf>(p, sm, from_side ? side : src, g, from_side ? st.top : f_level,
+        sweep_entry<kKind, kNarrowR, kFine, kProf>(p, sm, from_side ? side : src, g, from_side ? st.top : f_level,
                                             from_side ? 0u : sm.fid[fb][e], rows, x0, x1, lane, warp);
         prof_since<kProf>(sm, kPDescend, t0, lane);
     }
@@ -980,10 +997,12 @@ __global__ void __launch_bounds__(kThreads, SweepTraits<kKind, kSplit>::kPerSM) 
                 side.ids = p.mside_ids;
             }
             // (segments draw the same way at every radius)
-            if (kKind != HV_LAYER_POINTS || g.narrow)
-                sweep_pass<kKind, true, kProf>(p, sm, src, side, stree, side_hit, g, tid);
+            if (kKind != kPolyFill && (g.R >> g.s) > kTableReach)
+                sweep_pass<kKind, false, true, kProf>(p, sm, src, side, stree, side_hit, g, tid);
+            else if (kKind != HV_LAYER_POINTS || g.narrow)
+                sweep_pass<kKind, true, false, kProf>(p, sm, src, side, stree, side_hit, g, tid);
             else
-                sweep_pass<kKind, false, kProf>(p, sm, src, side, stree, side_hit, g, tid);
+                sweep_pass<kKind, false, false, kProf>(p, sm, src, side, stree, side_hit, g, tid);
             __syncthreads();
             if (tid == 0) prof_since<kProf>(sm, kPBlocksCta, t_pass, 0);
         }

@@ -24,9 +24,9 @@ def ctx():
     hv.hv_destroy(c)
 
 
-def profile(L, mode=hv.HV_MODE_COVERAGE):
+def profile(L, mode=hv.HV_MODE_COVERAGE, req=REQ):
     hv.hv_layer_build_index(L)
-    d = torch.from_numpy(hv.make_requests(REQ).view(np.uint8).copy()).cuda()
+    d = torch.from_numpy(hv.make_requests(req).view(np.uint8).copy()).cuda()
     out = torch.zeros((1, hv.hv_tile_bytes(mode)), dtype=torch.uint8, device="cuda")
     ph = torch.zeros(2 * hv.HV_PHASE_COUNT, dtype=torch.int64, device="cuda")
     hv.hv_render_tiles_phases(L, d, 1, mode, hv.HV_INDEX_RTREE, None, out, out.numel(), ph)
@@ -66,3 +66,22 @@ def test_polygons(ctx):
     (fill, outline), tile = profile(hv.hv_layer_load_polygons(ctx, xy, ro, po))
     assert fill[2] == strips_with(tile & 8) and fill[0] == fill[1] + fill[2]
     assert outline[2] == strips_with(tile & 7) and outline[0] >= outline[1] + outline[2]
+
+
+@pytest.mark.parametrize("lines", [False, True])
+def test_wide_reach_around_a_crowd(ctx, lines):
+    """20,000 records within a tenth of a sample spacing and a radius of 64 px: the
+    samples beside the disc are in no record's reach, so that a strip that the disc's
+    border crosses visits a few of the 625 leaves (all of them, when reach was
+    bounded to a column or two only)."""
+    rng = np.random.default_rng(4)
+    a = rng.integers(-600, 600, (20_000, 2)) + (8192, 8192)      # on a super-sample of tile (8, 128, 128)
+    a += 64 * ps(8)
+    req = np.array([[8, 128, 128, 1024]], dtype=np.uint32)
+    if lines:
+        xy = np.stack([a, a + rng.integers(-50, 50, a.shape)], 1).reshape(-1, 2).astype(np.int32)
+        L = hv.hv_layer_load_linestrings(ctx, xy, np.arange(0, len(xy) + 1, 2, dtype=np.uint64))
+    else:
+        L = hv.hv_layer_load_points(ctx, a.astype(np.int32))
+    (got, _), tile = profile(L, req=req)
+    assert 16 <= strips_with(tile) <= 40 and got[0] < 64 * 100, got

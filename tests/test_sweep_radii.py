@@ -109,6 +109,7 @@ extern "C" int reach_table(int32_t R, int32_t* reach) {
     for (int tid = 0; tid < 256; tid++) fill_reach(reach, g, tid);
     return g.rs;
 }
+extern "C" int32_t reach_by_root(int32_t R, int32_t f) { return reach_width<true>(nullptr, lattice(3, 256, 16, 0, 0, R), f); }
 """
 ENTRIES += r"""
 static int4 turned(int4 o, int how) {   // mirrored, transposed, ends exchanged
@@ -228,3 +229,13 @@ def test_reach_table_is_an_upper_bound(lib):
         for k in range((R >> rs) + 1):
             f = k << rs
             assert math.isqrt(R * R - f * f) <= table[k] <= R, (R, k, table[k])
+
+
+def test_reach_by_root_is_a_close_upper_bound(lib):
+    rng = random.Random(6)
+    lib.reach_by_root.restype = ctypes.c_int32
+    for i in range(100_000):
+        R = rng.randrange(1, 1 << 29) >> rng.randrange(0, 22) if i > 100 else (1 << 29) - i
+        f = rng.choice([0, R, max(R - rng.randrange(0, 50), 0), rng.randrange(0, R + 1)])
+        w = math.isqrt(R * R - f * f)
+        assert w <= lib.reach_by_root(R, f) <= min(R, w + 2 + (w >> 18)), (R, f)
