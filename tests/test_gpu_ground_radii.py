@@ -106,3 +106,40 @@ def test_row_that_is_only_just_within_reach(ctx, kind, radius, f, offset):
     y = offset - f
     xy = [(-3000, y), (-2000, y)] + ([(-2500, y - 100_000)] if kind == "polygons" else [])
     check(ctx, kind, xy, (19, 262144, 262144, 1), radius)
+
+
+@pytest.mark.parametrize("kind", ["points", "lines", "polygons"])
+def test_radius_beyond_the_tile(ctx, kind):
+    """Every sample of the tiles lies within the radius of any record: all are
+    covered, and a layer of many records takes about the time of one record (drawing
+    each of its boxes took a dozen times as long)."""
+    rng = np.random.default_rng(8)
+    z, radius = 10, 1 << 28
+    d = torch.from_numpy(hv.make_requests(np.repeat(np.array([[z, 512, 511, 1]]), 60, 0)).view(np.uint8).copy()).cuda()
+    out = torch.zeros((60, 65536), dtype=torch.uint8, device="cuda")
+    ms = []
+    for n in (1, 50_000):
+        xy = rng.integers(-2 ** 22, 2 ** 22, (3 * n, 2)).astype(np.int32)
+        if kind == "points":
+            L = hv.hv_layer_load_points(ctx, xy)
+        elif kind == "lines":
+            L = hv.hv_layer_load_linestrings(ctx, xy, np.arange(0, 3 * n + 1, 3, dtype=np.uint64))
+        else:
+            xy = np.repeat(xy[::3], 3, 0) + np.tile([[0, 0], [900, 0], [0, 900]], (n, 1)).astype(np.int32)
+            L = hv.hv_layer_load_polygons(ctx, xy, np.arange(0, 3 * n + 1, 3, dtype=np.uint64), np.arange(n + 1, dtype=np.uint64))
+        hv.hv_layer_build_index(L)
+        best = 1e9
+        for _ in range(20):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            out.zero_()
+            a.record()
+            hv.hv_render_buffer(L, d, 60, hv.HV_MODE_COVERAGE, hv.HV_INDEX_RTREE, radius, None, out, out.numel(),
+                                torch.cuda.current_stream())
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+            assert bool(((out & 7) == 4).all())
+        ms.append(best)
+        assert hv.hv_layer_take_status(L) == 0
+        hv.hv_layer_free(L)
+    assert ms[1] < 4 * ms[0], ms

@@ -109,6 +109,10 @@ extern "C" int reach_table(int32_t R, int32_t* reach) {
     for (int tid = 0; tid < 256; tid++) fill_reach(reach, g, tid);
     return g.rs;
 }
+extern "C" int covers(int s, int hw, int hh, int32_t xc, int32_t yc, int32_t R, int32_t x0, int32_t y0, int32_t x1, int32_t y1) {
+    const Lattice g = lattice(s, hw, hh, xc, yc, R);
+    return covers_strip(g, rel32(x0, xc), rel32(y0, yc), rel32(x1, xc), rel32(y1, yc));
+}
 extern "C" int32_t reach_by_root(int32_t R, int32_t f) { return reach_width<true>(nullptr, lattice(3, 256, 16, 0, 0, R), f); }
 """
 ENTRIES += r"""
@@ -239,3 +243,28 @@ def test_reach_by_root_is_a_close_upper_bound(lib):
         f = rng.choice([0, R, max(R - rng.randrange(0, 50), 0), rng.randrange(0, R + 1)])
         w = math.isqrt(R * R - f * f)
         assert w <= lib.reach_by_root(R, f) <= min(R, w + 2 + (w >> 18)), (R, f)
+
+
+def test_box_that_covers_a_strip(lib):
+    """covers_strip against the distances of the strip's corner samples to the box's
+    corners: never true for a box that does not cover, and true unless it only just does."""
+    rng = random.Random(7)
+    seen = [0, 0]
+    for _ in range(50_000):
+        s, hw, hh = rng.randrange(3, 23), 16 << rng.randrange(5), 2 << rng.randrange(4)
+        h = 1 << s
+        if hw * h > 1 << 30:
+            continue
+        zone = ((1 << 30) - hw * h) // h
+        xc, yc = (rng.randrange(-zone, zone + 1) * h + h // 2 for _ in range(2))
+        R = min(1 << 29, int(hw * h * rng.choice([1, 1.001, 1.01, 1.5, 4])) + rng.randrange(-2, 3))
+        near = rng.choice([4, h, R // 8 + 1, 1 << 30])
+        x0, y0 = (max(-2 ** 30, min(2 ** 30 - 1, c + rng.randrange(-near, near))) for c in (xc, yc))
+        x1, y1 = (min(2 ** 30 - 1, v + rng.randrange(0, rng.choice([2, h, R // 8 + 1]))) for v in (x0, y0))
+        far = max((x - a) ** 2 + (y - b) ** 2 for x in (x0, x1) for y in (y0, y1)
+                  for a in (xc - hw * h, xc + (hw - 1) * h) for b in (yc - hh * h, yc + (hh - 1) * h))
+        got = bool(lib.covers(s, hw, hh, xc, yc, R, x0, y0, x1, y1))
+        assert not got or far <= R * R
+        assert got or far + 3 * h * R + (R * R >> 17) > R * R      # (a column and row more than the strip has, and rounding)
+        seen[got] += 1
+    assert min(seen) > 5000, seen
