@@ -461,6 +461,18 @@ __device__ __noinline__ bool draw_row_slow(uint32_t* bits, const Lattice& g, con
     const float rho = (float)g.R * __int_as_float((127 - g.s) << 23);
     const float inv = rcp_approx(q.my);
     bool fresh = false;
+    if (q.my == 0.f) {
+        // a level segment (or a point): the row's distance is a whole number, which decides
+        // the row at once (tested, a long one that grazes the row leaves 512 columns to
+        // one lane: 60 us in a tile that took 46 without)
+        const int4 o = __ldg(seg);
+        const int32_t f = abs(rel32(o.y, g.yc) - (r - g.hh) * (1 << g.s));
+        if (f > g.R) return false;
+        const int32_t w = (int32_t)isqrt_wide((uint64_t)(g.R2 - (int64_t)f * f));
+        const int c0 = max(g.hw - ((w - rel32(min(o.x, o.z), g.xc)) >> g.s), clo + col);
+        const int c1 = min(((rel32(max(o.x, o.z), g.xc) + w) >> g.s) + g.hw, chi + col);
+        return c0 <= c1 && set_columns(bits + r * kBitStride, c0, c1) && kProf;
+    }
     if (q.E < 0.f) {
         // (beyond 4 M = 2^19 |E| there are no samples; 0 / 0 leaves a side open, and
         // the quotients are good to 2^-21 of themselves)

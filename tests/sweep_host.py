@@ -33,8 +33,8 @@ struct float4 { float x, y, z, w; };
 inline int2 make_int2(int x, int y) { return {x, y}; }
 inline int4 make_int4(int x, int y, int z, int w) { return {x, y, z, w}; }
 inline float4 make_float4(float x, float y, float z, float w) { return {x, y, z, w}; }
-static int64_t g_reads = 0;   // of __ldg: one per exact test of a sample
-template <class T> T __ldg(const T* p) { g_reads++; return *p; }
+static int64_t g_tests = 0;   // exact tests of samples, and sides taken
+template <class T> T __ldg(const T* p) { return *p; }
 inline float __int_as_float(int v) { float f; memcpy(&f, &v, 4); return f; }
 inline float __uint_as_float(uint32_t v) { float f; memcpy(&f, &v, 4); return f; }
 inline uint32_t __float_as_uint(float v) { uint32_t u; memcpy(&u, &v, 4); return u; }
@@ -77,7 +77,7 @@ def source():
     sweep = re.sub(r'asm\("shl\.b32[^;]*;[^;]*;', "r = (uint32_t)n > 31u ? 0u : v << n;", sweep)
     sweep = re.sub(r'asm\("(sqrt|rsqrt|rcp)\.[^;]*;[^;]*;', r"r = host_\1(x);", sweep)
     assert "asm(" not in sweep
-    return SHIM + dev + sweep
+    return SHIM + re.sub(r"((?:bool segment_within|int side_of_nearest)\([^)]*\) \{)", r"\1 g_tests++;", dev + sweep)
 
 
 def library(tmp_path, entries):

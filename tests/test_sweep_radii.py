@@ -154,7 +154,7 @@ ENTRIES += r"""
 extern "C" int64_t wide_pieces(uint64_t seed, int64_t n, int32_t R, Result* res) {
     std::mt19937_64 rng(seed);
     auto pick = [&](int64_t a, int64_t b) { return a + (int64_t)(rng() % (uint64_t)(b - a + 1)); };
-    const int64_t reads = g_reads, e = (1ll << 30) - 1;
+    const int64_t before = g_tests, e = (1ll << 30) - 1;
     for (int64_t i = 0; i < n; i++) {
         const int s = (int)pick(6, 18), hw = 256, hh = 2 << pick(0, 3);
         const int64_t zone = ((1ll << 30) >> s) - hw;
@@ -168,7 +168,30 @@ extern "C" int64_t wide_pieces(uint64_t seed, int64_t n, int32_t R, Result* res)
         if (bx < -e || bx > e || by < -e || by > e) continue;
         compare(g, make_int4(o.x, o.y, (int)bx, (int)by), piece_box(make_int4(o.x, o.y, (int)bx, (int)by), pick(0, m - 1), m), 4, rng, res);
     }
-    return g_reads - reads;
+    return g_tests - before;
+}
+"""
+ENTRIES += r"""
+// level segments (edges of large squares) whose border lies within a unit or so of a sample row: the most tests of one row
+extern "C" int64_t grazing_level(uint64_t seed, int64_t n, Result* res) {
+    std::mt19937_64 rng(seed);
+    auto pick = [&](int64_t a, int64_t b) { return a + (int64_t)(rng() % (uint64_t)(b - a + 1)); };
+    int64_t most = 0;
+    for (int64_t i = 0; i < n; i++) {
+        const int s = (int)pick(6, 14), hw = 256, hh = 2 << pick(0, 3);
+        const int64_t zone = (1ll << 24) >> s, h = 1ll << s;
+        const Lattice g = lattice(s, hw, hh, (int32_t)(pick(-zone, zone) * h + h / 2), (int32_t)(pick(-zone, zone) * h + h / 2),
+                                  (int32_t)max(h * pick(1, 64) / 16, (int64_t)1));
+        const int64_t y = g.yc + pick(-hh, hh - 1) * h + (rng() & 1 ? 1 : -1) * (g.R + pick(-2, 1));
+        const int64_t x = g.xc + pick(-300, 300) * h, d = pick(h, 1 << 24), a = pick(0, d);
+        const int4 o = make_int4((int)(x - a), (int)y, (int)(x - a + d), (int)y);
+        for (int k = 0; k < 3; k++) {
+            const int64_t before = g_tests, rows = res->rows;
+            compare(g, o, piece_box(o, 0, 1), 1, rng, res);
+            if (res->rows > rows) most = max(most, g_tests - before);
+        }
+    }
+    return most;
 }
 """
 
@@ -210,6 +233,17 @@ def test_wide_pieces_take_few_exact_tests(lib, R):
     tests = lib.wide_pieces(ctypes.c_uint64(9), ctypes.c_int64(40_000), ctypes.c_int32(R), ctypes.byref(res))
     assert res.rows > 10_000 and res.wrong == 0, (res.rows, res.wrong)
     assert tests < res.rows / 2, (tests, res.rows)
+
+
+def test_grazing_level_segments_take_no_run_of_tests(lib):
+    """A level segment just above or below a row left up to 512 columns doubtful; its
+    distance from the row is a whole number, so that the row is decided at once (rows
+    that do not graze: one test at most at either end)."""
+    res = Result()
+    lib.grazing_level.restype = ctypes.c_int64
+    most = lib.grazing_level(ctypes.c_uint64(2), ctypes.c_int64(100_000), ctypes.byref(res))
+    assert res.rows > 30_000 and res.covered > 0 and res.wrong == 0
+    assert most <= 2, most
 
 
 def test_rows_at_the_grid_border(lib):
