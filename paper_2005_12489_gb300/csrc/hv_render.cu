@@ -57,11 +57,9 @@ struct Params {
     uint32_t n;
     int rows;                   // pixel rows per CTA strip: 4, 8 or 16
     int strips;                 // strips per tile (256 / rows)
-    int cols;                   // pixel columns per CTA: 256, or 128 / 64 / 32 for batches too small to fill the GPU
-    int parts;                  // CTAs per strip (256 / cols)
+    int parts;                  // CTAs per strip: 1, or 2 / 4 / 8 (128 / 64 / 32 columns each) for batches too small to fill the GPU
     const uint32_t* n_dev;      // if set, the batch size is min(*n_dev, n) (graph launches)
     int mode;
-    int kind;
     uchar4 line;
     uchar4 fill;
     uint8_t* out;
@@ -277,9 +275,8 @@ __device__ void cull(const Params& p, const TreeArg& t, bool fill, Front& sm, in
 }
 
 // Learned cull (replaces the breadth-first R-tree cull): cover the strip's
-// box, widened by the halo of object extents, with at most 256 aligned
-// Hilbert cells (one per thread; a cell's keys are a contiguous run of the
-// sorted order), find each cell's position range through the learned model,
+// box, widened by the halo of object extents, with at most kCullCells aligned
+// Hilbert cells (a cell's keys are a contiguous run of the sorted order), find each cell's position range through the learned model,
 // and turn the ranges into R-tree subtrees at the finest level whose entries
 // fit the frontier.  Every object whose centre lies in the box is under one of
 // the entries; the sweep then proceeds exactly as after the R-tree cull.
@@ -578,7 +575,6 @@ int launch_render(Layer* L, const hv_tile_req* d_reqs, uint32_t n, int mode, int
     p.n = n;
     p.n_dev = n_dev;
     p.mode = mode;
-    p.kind = L->kind;
     if (style) {
         p.line = make_uchar4(style->line_rgba[0], style->line_rgba[1], style->line_rgba[2], 0);
         p.fill = make_uchar4(style->fill_rgba[0], style->fill_rgba[1], style->fill_rgba[2], 0);
@@ -649,7 +645,6 @@ int launch_render(Layer* L, const hv_tile_req* d_reqs, uint32_t n, int mode, int
     p.parts = 1;
     if (p.rows == 4 && !prof)
         while (p.parts < 8 && (uint64_t)n * p.strips * p.parts * 2 <= resident) p.parts *= 2;
-    p.cols = kTile / p.parts;
     uint64_t grid = (uint64_t)n * p.strips * p.parts;
     if (grid > 0x7fffffffull) {
         set_error("too many tiles in one call");

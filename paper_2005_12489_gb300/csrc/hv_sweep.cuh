@@ -12,14 +12,16 @@
 // 8 x 4 pixel block that it reaches, and only while a sample that it can reach
 // is still open; inner nodes and frontier entries are pruned by the same test.
 //
-// Bound: instruction issue (72% of the slots busy; DRAM a few percent).  Drawn
-// by strips, 600 tiles of 100M clustered points at 2 px take 2.4 M warp
-// instructions per tile where the 8 x 4 block traversal took 5.7 M: 4,000
-// tiles 23.5 -> 11.8 ms; 341 tiles of 100,000 points at zoom 0-4, 1 px, MASK
-// 414 -> 72 us; 36 single tiles of 10M points 1,340 -> 776 us in all.  Segments: 4,000 tiles of 50M
-// segments at 1 px 19.7 -> 5.6 ms; the outlines of 1,000 tiles of 2M polygons
-// 12 -> 8.5 ms (dense low-zoom tiles: 390 leaves of short edges per strip, 22
-// pieces and 71 (piece, row) pairs each).
+// Bound: instruction issue for points and outlines (71% and 68% of the slots busy);
+// segments and fill (53%, 50%), with few leaves per strip, wait at barriers and for
+// their reads.  DRAM 5 to 11% of the measured copy rate.  Drawn by strips, 600
+// tiles of 100M clustered points at 2 px take 2.4 M warp instructions per tile
+// where the 8 x 4 block traversal took 5.7 M: 4,000 tiles 23.5 -> 11 ms; 341 tiles of
+// 100,000 points at zoom 0-4, 1 px, MASK 414 -> 72 us; 36 single tiles of 10M
+// points 1,340 -> 776 us in all.  Segments: 4,000 tiles of 50M segments at 1 px
+// 19.7 -> 5.5 ms; the outlines of 1,000 tiles of 2M polygons 12 -> 8.5 ms (dense
+// low-zoom tiles: 390 leaves of short edges per strip, 22 pieces and 71 (piece, row)
+// pairs each).
 //
 // The fill draws polygon by polygon: one pass over a polygon's edges gives every
 // crossing of the strip's rows, and a parity scan per row the filled samples.
@@ -218,8 +220,8 @@ __device__ __forceinline__ void fill_reach(int32_t* reach, const Lattice& g, int
 // (kFine) a root is taken, good to 2^-19.  300 tiles of 200,000 crowded points at
 // 64 px 9.56 -> 0.35 ms, of 50,000 polygons' outlines 28.1 -> 1.87 ms; as a branch taken
 // for each row instead of an instantiation 4,000 tiles of 100M points at 2 px lose 7%.
-// From kTableReach = 16 spacings on: the table is off by a quarter of a column there (8
-// and 32 measured alike).
+// From kTableReach = 16 spacings on, where the table is off by a quarter of a column (616
+// calls with radii of 12 to 64 px: 221 ms in all, 272 from 32 spacings on, 456 from 64).
 template <bool kFine>
 __device__ __forceinline__ int32_t reach_width(const int32_t* reach, const Lattice& g, int32_t f) {
     if (!kFine) return reach[f >> g.rs];
@@ -612,9 +614,9 @@ __device__ __forceinline__ Visit draw_segments(const Params& p, const Src& src, 
 // End of the columns that an edge crosses strictly to the right in the row at
 // height y (Algorithm 2's ray test): column c is crossed when (c - hw) h ey < N
 // with N = ex (y - ly) + lx ey, so the columns are those before ceil(N / (h ey))
-// + hw, cut off to lo..hi.  The quotient is estimated in single precision, once
-// more from the exact remainder (an edge far longer than the strip leaves the
-// first estimate columns off), and settled by the exact remainder's sign.
+// + hw, cut off to lo..hi.  The quotient is estimated in single precision (cut off to
+// the strip, a hundredth of a column or less away, then truncated towards zero), raised
+// by the exact remainder's quotient, and settled by the sign of what remains.
 // |N| <= 2^62: it is ey times the crossing's coordinate.
 __device__ __forceinline__ int crossing_end(const Lattice& g, int32_t lx, int32_t ly, int32_t ex, int32_t ey, int32_t y,
                                             int lo, int hi) {
