@@ -150,7 +150,7 @@ def measured_peak_hbm():
 
 
 KERNEL_SOURCES = ("hv_render.cu", "hv_sweep.cuh", "hv_device.cuh", "hv_learned.cuh", "hv_internal.h")
-PROFILES = {2: "k_render_points_gmm100M.md", 3: "k_render_lines_walk50M.md", 4: "k_render_polygons_star2M.md"}
+PROFILES = {2: "k_sweep_points_gmm100M.md", 3: "k_sweep_lines_walk50M.md", 4: "k_sweep_polygons_star2M.md"}
 
 
 def _code_only(text):
@@ -436,9 +436,9 @@ def phase_profile(hv, torch, layer, d_req, n, mode, index, style, d_out, kind):
         tot = max(c[0], 1.0)
         busy, leaf, desc = c[5], c[6], c[7]
         parts[name] = {
-            "share": {"prologue": c[1] / tot, "cull": c[2] / tot, "bin": c[3] / tot,
-                      "frontier_scan": (busy - desc) / tot, "node_tests": (desc - leaf) / tot,
-                      "leaf_visits": leaf / tot, "blocks_waiting": (c[4] - busy) / tot, "encode": c[8] / tot},
+            "share": {"prologue": c[1] / tot, "cull": c[2] / tot,
+                      "frontier_tests": (busy - desc) / tot, "node_tests": (desc - leaf) / tot,
+                      "leaf_visits": leaf / tot, "warps_waiting": (c[4] - busy) / tot, "encode": c[8] / tot},
             "per_tile": {"blocks": c[10] / n, "leaf_visits": c[11] / n, "node_visits": c[12] / n,
                          "frontier_tests": c[13] / n, "leaf_visits_empty": c[14] / n,
                          "leaf_visits_deciding": c[15] / n},
@@ -476,7 +476,8 @@ def _roofline_issue(cfg, ms, full_size):
     return {"bound": "alu", "achieved": achieved_i, "peak": ipk, "unit": "G warp-instructions/s",
             "frac": achieved_i / ipk, "instructions_per_launch": n_inst,
             "peak_basis": "SMs x 4 schedulers x 1 warp instruction/cycle x max SM clock",
-            "note": "the integer pipe bounds this kernel; instruction count from the committed ncu summary"}
+            "note": "instruction issue, not memory, bounds this kernel; instruction count from the committed ncu "
+                    "summary"}
 
 
 def measure_batch(args, cfg, steps, warmup, dist=None, headline=False, r16_sweep=None):
@@ -660,6 +661,39 @@ def measure_batch(args, cfg, steps, warmup, dist=None, headline=False, r16_sweep
     return out
 
 
+def _pick(d, *keys):
+    """The given keys of a dict (None stays None)."""
+    return None if d is None else {k: d[k] for k in keys if k in d}
+
+
+def result_line(line):
+    """The result line: the contract's keys and a few figures per block, a few
+    kilobytes in all, so that whoever keeps only the end of the output still has it
+    whole.  (Everything measured goes to stderr.)"""
+    nested = {"learned", "latency", "phases", "r16_sweep", "host_resident", "step_ms", "configs", "roofline", "cpu_baseline",
+              "cpu_rtree_mt"}
+    out = {k: v for k, v in line.items() if k not in nested}
+    short = ("bound", "achieved", "peak", "unit", "frac", "traffic", "peak_kind", "kernel", "alg_bytes_per_tile")
+    out["roofline"] = _pick(line.get("roofline"), *short)
+    for k in ("cpu_baseline", "cpu_rtree_mt"):
+        out[k] = _pick(line.get(k), "value", "unit", "cores", "kind", "sample")
+    out["learned"] = _pick(line.get("learned"), "value", "ms_per_step", "unit", "learned_over_rtree")
+    out["latency"] = {k: _pick(v, "p50_ms", "p99_ms", "mean_ms") for k, v in (line.get("latency") or {}).items()}
+    out["host_resident"] = _pick(line.get("host_resident"), "value", "unit", "ms_per_step")
+    out["configs"] = {}
+    for k, b in (line.get("configs") or {}).items():
+        c = _pick(b, "metric", "value", "unit", "ms_per_step", "steps", "gpu_launches", "wall_s")
+        c["e2e"] = _pick(b.get("e2e"), "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")
+        c["roofline"] = _pick(b.get("roofline"), "bound", "achieved", "unit", "frac", "traffic")
+        c["cpu_baseline"] = _pick(b.get("cpu_baseline"), "value", "unit", "kind")
+        if "learned" in b:
+            c["learned"] = _pick(b["learned"], "value", "learned_over_rtree")
+        if "per_rate" in b:
+            c["per_rate"] = [_pick(r, "rate", "index", "tiles_per_s", "p50_ms", "p99_ms") for r in b["per_rate"]]
+        out["configs"][k] = c
+    return out
+
+
 def run_gb300(args):
     import torch
 
@@ -688,7 +722,8 @@ def run_gb300(args):
         blocks["5"]["wall_s"] = time.time() - t0
         line["configs"] = blocks
     if rank == 0 and line is not None:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(line if args.profile_steps else result_line(line)), flush=True)
     if dist is not None:
         dist.barrier()
         dist.destroy_process_group()
